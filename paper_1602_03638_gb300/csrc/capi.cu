@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <array>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -207,23 +208,24 @@ bool same_scheme(const RkScheme& x, const RkScheme& y) {
   return true;
 }
 
-// exp(-2 pi i t / N) in FP64 with exact quadrant/octant symmetry.
-void twiddle(long t, long N, double* re, double* im) {
+// exp(-2 pi i t / N) in R (double, long double) with exact quadrant/octant symmetry.
+template <typename R>
+void twiddle(long t, long N, R* re, R* im) {
   t %= N;
   const long q = (4 * t) / N;
   const long r = 4 * t - q * N;  // angle = q pi/2 + (pi/2) r/N, 0 <= r < N
-  const double pi = 3.14159265358979323846;
-  double c, s;
+  const R pi = (R)3.14159265358979323846264338327950288L;
+  R c, s;
   if (2 * r <= N) {
-    const double phi = pi * (double)r / (2.0 * (double)N);
+    const R phi = pi * (R)r / (R)(2 * N);
     c = std::cos(phi);
     s = std::sin(phi);
   } else {
-    const double phi = pi * (double)(N - r) / (2.0 * (double)N);
+    const R phi = pi * (R)(N - r) / (R)(2 * N);
     c = std::sin(phi);
     s = std::cos(phi);
   }
-  double C, S;
+  R C, S;
   switch (q & 3) {
     case 0: C = c; S = s; break;
     case 1: C = -s; S = c; break;
@@ -232,6 +234,15 @@ void twiddle(long t, long N, double* re, double* im) {
   }
   *re = C;
   *im = -S;
+}
+
+// v (|v| <= 1) in units of 2^-62 as out[0] 2^32 + out[1] with |out[1]| < 2^31 (fixed_point.cuh)
+void fixed_factor(long double v, int* out) {
+  long long w = std::llroundl(std::ldexp(v, 62));
+  if ((int)(unsigned)w == INT_MIN) ++w;
+  const long long lo = (int)(unsigned)w;
+  out[0] = (int)((w - lo) >> 32);
+  out[1] = (int)lo;
 }
 
 }  // namespace
@@ -561,14 +572,24 @@ int dns_create3(int Nx, int Ny, int Nz, double nu, double dt, int dtype, dns_han
   if (rc == DNS_OK) rc = dev_alloc(h, &h->tw, (size_t)TW * cb, "twiddles");
   if (rc == DNS_OK) rc = dev_alloc(h, (void**)&h->diag, (DIAG_BLOCKS * 4 + 8) * sizeof(double), "diagnostics");
   if (rc == DNS_OK) {
-    std::vector<double> t64(2 * TW);
-    for (int t = 0; t < TW; ++t) twiddle(t, TW, &t64[2 * t], &t64[2 * t + 1]);
     if (dtype == DNS_F32) {
       std::vector<float> t32(2 * TW);
-      for (int i = 0; i < 2 * TW; ++i) t32[i] = (float)t64[i];
+      for (int t = 0; t < TW; ++t) {
+        double re, im;
+        twiddle(t, TW, &re, &im);
+        t32[2 * t] = (float)re;
+        t32[2 * t + 1] = (float)im;
+      }
       ce = cudaMemcpy(h->tw, t32.data(), t32.size() * sizeof(float), cudaMemcpyHostToDevice);
-    } else {
-      ce = cudaMemcpy(h->tw, t64.data(), t64.size() * sizeof(double), cudaMemcpyHostToDevice);
+    } else {  // the FP64 form's line transforms run on fixed point
+      std::vector<int> tfx(4 * TW);
+      for (int t = 0; t < TW; ++t) {
+        long double re, im;
+        twiddle(t, TW, &re, &im);
+        fixed_factor(re, &tfx[4 * t]);
+        fixed_factor(im, &tfx[4 * t + 2]);
+      }
+      ce = cudaMemcpy(h->tw, tfx.data(), tfx.size() * sizeof(int), cudaMemcpyHostToDevice);
     }
     if (ce == cudaSuccess) ce = cudaMemset(h->U, 0, 3 * h->fs * cb);
     if (ce != cudaSuccess) rc = cuda_fail(ce, "dns_create initialisation");

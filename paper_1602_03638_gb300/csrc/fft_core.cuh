@@ -36,6 +36,11 @@ __device__ __forceinline__ cx<T> cmul(cx<T> a, cx<T> b) {
 }
 template <typename T>
 __device__ __forceinline__ cx<T> conjg(cx<T> a) { return mk(a.x, -a.y); }
+// the sign bit of a double flipped by the integer unit: an FP64 negation is an addition on the FP64 pipe
+__device__ __forceinline__ double neg64(double a) {
+  return __hiloint2double(__double2hiint(a) ^ (int)0x80000000, __double2loint(a));
+}
+__device__ __forceinline__ cx<double> conjg(cx<double> a) { return mk(a.x, neg64(a.y)); }
 template <typename T>
 __device__ __forceinline__ cx<T> scal(cx<T> a, T s) { return mk(a.x * s, a.y * s); }
 // a * (-i)
@@ -44,6 +49,7 @@ __device__ __forceinline__ cx<T> mul_mi(cx<T> a) { return mk(a.y, -a.x); }
 // a * (+i)
 template <typename T>
 __device__ __forceinline__ cx<T> mul_pi(cx<T> a) { return mk(-a.y, a.x); }
+__device__ __forceinline__ cx<double> mul_pi(cx<double> a) { return mk(neg64(a.y), a.x); }
 
 // Read-only cached load of one complex value (twiddle tables).
 __device__ __forceinline__ cx<float> ldro(const cx<float>* p) {
@@ -228,6 +234,13 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int padp(int p) { return p + (p >> 4); }
 __host__ __device__ constexpr int padded_len(int L) { return L + L / 16 + 1; }
+// The padding by type: FP64 lines (16-byte values, eight of them to all the banks) are padded every 8,
+// so that the radix-8 Stockham stores of a quarter-warp (rows 9 j) hit distinct banks; padded every 16
+// they met two by two.
+template <typename T>
+__host__ __device__ constexpr int padt(int p) { return sizeof(T) == 8 ? p + (p >> 3) : padp(p); }
+template <typename T>
+__host__ __device__ constexpr int padt_len(int L) { return sizeof(T) == 8 ? padt<T>(L - 1) + 1 : padded_len(L); }
 
 constexpr int ilog2c(int x) {
   int r = 0;
@@ -323,20 +336,20 @@ struct IsPow2 {
 
 // Access policies for the warp FFT. at(p) gives the address of position p;
 // for power-of-two plans every pass touches positions base + d with
-// padp(base + d) = padp(base) + padp(d), so off(d) is a compile-time offset.
+// padt(base + d) = padt(base) + padt(d), so off(d) is a compile-time offset.
 template <typename T, int ES>
 struct SLine {  // a line in shared memory at padded positions, element stride ES
   cx<T>* s;
-  __device__ __forceinline__ cx<T>* at(int p) const { return s + padp(p) * ES; }
-  static constexpr int off(int d) { return padp(d) * ES; }
+  __device__ __forceinline__ cx<T>* at(int p) const { return s + padt<T>(p) * ES; }
+  static constexpr int off(int d) { return padt<T>(d) * ES; }
   __device__ __forceinline__ cx<T> load(const cx<T>* q) const { return *q; }
   __device__ __forceinline__ void store(cx<T>* q, int, cx<T> v) const { *q = v; }
 };
 template <typename T, int ES>
 struct SLineConj {  // shared-memory line read conjugated (inverse DFT of staged data)
   cx<T>* s;
-  __device__ __forceinline__ cx<T>* at(int p) const { return s + padp(p) * ES; }
-  static constexpr int off(int d) { return padp(d) * ES; }
+  __device__ __forceinline__ cx<T>* at(int p) const { return s + padt<T>(p) * ES; }
+  static constexpr int off(int d) { return padt<T>(d) * ES; }
   __device__ __forceinline__ cx<T> load(const cx<T>* q) const { return conjg(*q); }
 };
 template <typename T>
@@ -401,16 +414,10 @@ __device__ __forceinline__ void warp_fft_pass(const Src& src, const Work& work, 
         }
       }
       if constexpr (NS > 1) {
-        if constexpr (sizeof(T) == 4) {
-          cx<T> w[R];
-          twiddle_powers<R>(ldro(tw + (j % NS) * TWC), w);
+        cx<T> w[R];
+        twiddle_powers<R>(ldro(tw + (j % NS) * TWC), w);
 #pragma unroll
-          for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
-        } else {  // FP64 multiplies are scarcer than loads: read every power
-          const int kc = (j % NS) * TWC;
-#pragma unroll
-          for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], ldro(tw + r * kc));
-        }
+        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
       }
       dft<R>(v[b]);
     }
@@ -489,16 +496,10 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b][r] = ln[padp(j + r * NB) * LD];
       if constexpr (NS > 1) {
-        if constexpr (sizeof(T) == 4) {
-          cx<T> w[R];
-          twiddle_powers<R>(ldro(tw + (j % NS) * TWC), w);
+        cx<T> w[R];
+        twiddle_powers<R>(ldro(tw + (j % NS) * TWC), w);
 #pragma unroll
-          for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
-        } else {
-          const int kc = (j % NS) * TWC;
-#pragma unroll
-          for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], ldro(tw + r * kc));
-        }
+        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], w[r]);
       }
       dft<R>(v[b]);
     }
@@ -523,120 +524,6 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
 template <typename T, int L, int TWN, int G, int LD, int V = 0>
 __device__ __forceinline__ void warp_fft_lines(cx<T>* s0, const cx<T>* __restrict__ tw, int lane) {
   warp_fft_lines_pass<T, L, TWN, G, LD, 0, V>(s0, tw, lane);
-}
-
-// ---------------------------------------------------------------------------
-// Register-resident warp FFT ("canonical" layout): lane l holds positions
-// l + 32 m, m < L/32, in v[m]. Every pass reads its butterfly inputs from the
-// lane's own registers (positions j + r L/R with j = l + 32 b); the Stockham
-// outputs go through the shared-memory line `ln` (padded positions, element
-// stride es) and are read back canonically; the last pass's outputs are
-// already canonical and stay in registers. Needs L/R >= 32 in every pass.
-// ---------------------------------------------------------------------------
-template <int L>
-struct CanonPlan {
-  static constexpr int npass = (L == 128) ? 4 : WarpPlan<L>::npass;
-  static constexpr int radix(int p) { return (L == 128) ? (p < 3 ? 4 : 2) : WarpPlan<L>::radix(p); }
-  static constexpr int ns(int p) {
-    int r = 1;
-    for (int q = 0; q < p; ++q) r *= radix(q);
-    return r;
-  }
-  static constexpr bool valid() {
-    if (L % 32) return false;
-    for (int p = 0; p < npass; ++p)
-      if ((L / radix(p)) % 32) return false;
-    return true;
-  }
-};
-
-// Per-lane twiddle bases of the canonical FFT, loaded once per kernel: for
-// every pass P >= 1 and butterfly slot b, w1 = exp(-2 pi i ((l + 32 b) mod NS) / (NS R)).
-template <typename T, int L, int TWN>
-struct CanonTw {
-  using PL = CanonPlan<L>;
-  static constexpr int off(int P) {
-    int o = 0;
-    for (int q = 1; q < P; ++q) o += (L / PL::radix(q)) / 32;
-    return o;
-  }
-  static constexpr int count() { return off(PL::npass) > 0 ? off(PL::npass) : 1; }
-  cx<T> w[count()];
-  __device__ __forceinline__ void load(const cx<T>* __restrict__ tw, int lane) {
-    load_pass<1>(tw, lane);
-  }
-  template <int P>
-  __device__ __forceinline__ void load_pass(const cx<T>* __restrict__ tw, int lane) {
-    if constexpr (P < PL::npass) {
-      constexpr int R = PL::radix(P), NS = PL::ns(P), BPL = (L / R) / 32, TWC = TWN / (NS * R);
-#pragma unroll
-      for (int b = 0; b < BPL; ++b) w[off(P) + b] = ldro(tw + ((lane + 32 * b) % NS) * TWC);
-      load_pass<P + 1>(tw, lane);
-    }
-  }
-};
-
-template <typename T, int L, int TWN, int ES, int P>
-__device__ __forceinline__ void warp_fft_canon_pass(cx<T> (&v)[L / 32], cx<T>* ln, const CanonTw<T, L, TWN>& ctw,
-                                                    const cx<T>* __restrict__ tw, int lane) {
-  using PL = CanonPlan<L>;
-  constexpr int R = PL::radix(P);
-  constexpr int NS = PL::ns(P);
-  constexpr int NB = L / R;
-  constexpr int BPL = NB / 32;
-  constexpr bool LAST = (P + 1 == PL::npass);
-  constexpr int TWC = TWN / (NS * R);
-  static_assert(NB % 32 == 0, "canonical warp FFT needs L/R >= 32");
-  static_assert(IsPow2<L>::value, "canonical warp FFT needs a power-of-two length");
-  cx<T> u[BPL][R];
-#pragma unroll
-  for (int b = 0; b < BPL; ++b) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) u[b][r] = v[b + r * BPL];
-    if constexpr (NS > 1) {
-      if constexpr (sizeof(T) == 4) {
-        cx<T> w[R];
-        twiddle_powers<R>(ctw.w[CanonTw<T, L, TWN>::off(P) + b], w);
-#pragma unroll
-        for (int r = 1; r < R; ++r) u[b][r] = cmul(u[b][r], w[r]);
-      } else {
-        const int kc = ((lane + 32 * b) % NS) * TWC;
-#pragma unroll
-        for (int r = 1; r < R; ++r) u[b][r] = cmul(u[b][r], ldro(tw + r * kc));
-      }
-    }
-    dft<R>(u[b]);
-  }
-  if constexpr (LAST) {
-    // outputs j + r NS with NS = NB: canonical index b + r BPL
-#pragma unroll
-    for (int b = 0; b < BPL; ++b)
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[b + r * BPL] = u[b][r];
-  } else {
-#pragma unroll
-    for (int b = 0; b < BPL; ++b) {
-      const int j = lane + 32 * b;
-      cx<T>* q = ln + padp((j / NS) * NS * R + (j % NS)) * ES;
-#pragma unroll
-      for (int r = 0; r < R; ++r) q[padp(r * NS) * ES] = u[b][r];
-    }
-    __syncwarp();
-    const cx<T>* rb = ln + padp(lane) * ES;
-#pragma unroll
-    for (int m = 0; m < L / 32; ++m) v[m] = rb[34 * m * ES];
-    __syncwarp();
-    warp_fft_canon_pass<T, L, TWN, ES, P + 1>(v, ln, ctw, tw, lane);
-  }
-}
-
-// Forward DFT of the canonical register array v (length L) by one warp, using
-// the shared-memory line ln (L padded positions, element stride ES) for the
-// exchanges. The caller must have finished reading ln (and __syncwarp'ed).
-template <typename T, int L, int TWN, int ES>
-__device__ __forceinline__ void warp_fft_canon(cx<T> (&v)[L / 32], cx<T>* ln, const CanonTw<T, L, TWN>& ctw,
-                                               const cx<T>* __restrict__ tw, int lane) {
-  warp_fft_canon_pass<T, L, TWN, ES, 0>(v, ln, ctw, tw, lane);
 }
 
 }  // namespace dns

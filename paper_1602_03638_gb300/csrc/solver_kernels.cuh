@@ -23,12 +23,15 @@
 
 #include "dns_internal.h"
 #include "fft_core.cuh"
+#include "fixed_point.cuh"
 
 namespace dns {
 
 constexpr int XP_THREADS = 192;  // 6 warps: one per line of a row (u, omega)
 constexpr int YP_THREADS = 256;
-constexpr int ZP_THREADS = 256;
+// z-pass: 12 warps for the 24 + 12 lines of an FP64 tile of 4 columns
+template <typename T>
+constexpr int ZP_THREADS = sizeof(T) == 8 ? 384 : 256;
 constexpr int DG_THREADS = 256;
 
 constexpr int pow2_part(int n) {
@@ -56,25 +59,26 @@ struct Geometry {
   // omega transforms over rows 3-8).
   // Where 6 padded lines and the 9 rows fit in 64 KB (XWIDE), omega keeps
   // its own 3 padded lines instead (faster at N = 512 FP32).
-  static constexpr int XLS = padded_len(N);
+  static constexpr int XLS = padt_len<T>(N);
   static constexpr bool XWIDE = (size_t)((6 * XLS + 1) / 2 * 2 + 9 * N) * CB <= 64 * 1024;
   static constexpr int XST = ((XWIDE ? 6 : 3) * XLS + 1) / 2 * 2;  // 16-byte aligned start of the state rows
-  static constexpr bool XPRE = (size_t)(XST + 9 * N) * CB <= 100 * 1024;
+  static constexpr bool XPRE = CB == 8 && (size_t)(XST + 9 * N) * CB <= 100 * 1024;
   static constexpr size_t XSMEM = (size_t)6 * XLS * CB;
   static constexpr size_t XSMEM_ST = XPRE ? (size_t)(XST + 9 * N) * CB : XSMEM;  // XM_STAGE, XM_RHS
   // z-pass: ZTX adjacent x at fixed y, 6 fields of M values each, <= 112 KB
   // (two blocks per SM); rows narrower than one 32-byte sector may use up to 200 KB.
-  static constexpr size_t zbytes(int t) { return (size_t)padded_len(M) * odd_ld(6 * t) * CB; }
+  static constexpr size_t zbytes(int t) { return (size_t)padt_len<T>(M) * odd_ld(6 * t) * CB; }
+  static constexpr size_t ZBLOCK = (CB == 16 ? 113 : 112) * 1024;  // half an SM's shared memory
   static constexpr int ztx() {
     int t = cmin(16, pow2_part(N));
-    while (t > 1 && zbytes(t) > 112 * 1024 && !(t * CB <= 32 && zbytes(t) <= 200 * 1024)) t /= 2;
+    while (t > 1 && zbytes(t) > ZBLOCK && !(t * CB <= 32 && zbytes(t) <= 200 * 1024)) t /= 2;
     return t;
   }
   static constexpr int ZTX = ztx();
   // Minimum resident blocks per SM for the register cap: lines longer than 4 KB
   // hold 32+ registers of data per lane in the warp FFT, so allow more registers.
   static constexpr int LINE_BYTES = N * CB;
-  static constexpr int XMIN = LINE_BYTES > 4096 ? 2 : 4;
+  static constexpr int XMIN = CB == 16 ? (N <= 256 ? 4 : (N <= 512 ? 3 : 2)) : (LINE_BYTES > 4096 ? 2 : 4);
   static constexpr int ZMIN = (M * CB > 4096) ? 1 : 2;
   static constexpr int ZLD = odd_ld(6 * ZTX);
   static constexpr size_t ZSMEM = zbytes(ZTX);
@@ -93,8 +97,8 @@ struct YCfg {
   static constexpr int TX = TXO > 0 ? TXO : cmin(((INV || CB == 16) && NY <= 512 ? 128 : 64) / CB, pow2_part(N));
   static constexpr int THREADS = cmin(32 * TX, 256);
   static constexpr int LD = odd_ld(TX);
-  static constexpr size_t SMEM = (size_t)padded_len(NY) * LD * CB;
-  static constexpr int MINB = (CB == 8 && NY <= 512) ? (INV ? 3 : 4) : 2;
+  static constexpr size_t SMEM = (size_t)padt_len<T>(NY) * LD * CB;
+  static constexpr int MINB = CB == 16 ? (NY <= 256 ? 3 : 2) : (NY <= 512 ? (INV ? 3 : 4) : 2);
 };
 
 __device__ __forceinline__ int kfreq(int i, int N) { return i < N / 2 ? i : i - N; }
@@ -128,12 +132,14 @@ enum ZMode { ZM_CROSS = 0, ZM_STORE = 1, ZM_LOAD = 2, ZM_MAXABS = 3 };
 // Writes conj(u/N^3) and conj(i k x u / N^3) of one mode into the 6 line
 // buffers (stride LS) at padded position pos (conjugated because the following
 // x transform is an inverse one).
-template <typename T>
+template <bool SCALE, typename T>
 __device__ __forceinline__ void put_curl_lines(cx<T>* s, int pos, int LS, cx<T> u0, cx<T> u1, cx<T> u2, T kx, T ky,
                                                T kz, T sc) {
-  u0 = scal(u0, sc);
-  u1 = scal(u1, sc);
-  u2 = scal(u2, sc);
+  if constexpr (SCALE) {
+    u0 = scal(u0, sc);
+    u1 = scal(u1, sc);
+    u2 = scal(u2, sc);
+  }
   // omega_hat = i k x u_hat
   const cx<T> w0 = mul_pi(mk(ky * u2.x - kz * u1.x, ky * u2.y - kz * u1.y));
   const cx<T> w1 = mul_pi(mk(kz * u0.x - kx * u2.x, kz * u0.y - kx * u2.y));
@@ -145,6 +151,17 @@ __device__ __forceinline__ void put_curl_lines(cx<T>* s, int pos, int LS, cx<T> 
   p[3 * LS] = conjg(w0);
   p[4 * LS] = conjg(w1);
   p[5 * LS] = conjg(w2);
+}
+
+// 1 / x for a positive normal x
+__device__ __forceinline__ float recip(float x) { return 1.f / x; }
+// in FP64 by Newton's iteration r <- r + r (1 - x r) from the hardware's approximation: four
+// operations of the FP64 pipe, last-bit accuracy (the division takes ten)
+__device__ __forceinline__ double recip(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
 }
 
 // Global store of one complex value of the RK state.
@@ -213,6 +230,9 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
   const int kz = row / NY, ky = row % NY;
   const size_t rb = (size_t)row * N;
   const T sc = (T)(1.0 / ((double)N * (double)NY * (double)NZ));
+  // the FP64 form's inverse transforms take a power of two in the conversion of their results
+  constexpr int E2 = sizeof(T) == 8 && IsPow2<N>::value && IsPow2<NY>::value && IsPow2<NZ>::value
+                         ? -(ilog2c(N) + ilog2c(NY) + ilog2c(NZ)) : 0;
   // wavenumbers of the row and of column j: integer index times 2 pi / L (1 on the 2 pi box)
   const T ksx = par<T>(a.ks[0], a.f_ks[0]);
   const T kzv = (T)kz * par<T>(a.ks[2], a.f_ks[2]), kyv = (T)kfreq(ky, NY) * par<T>(a.ks[1], a.f_ks[1]);
@@ -241,7 +261,7 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
       if (row_kept) {
         for (int e = threadIdx.x; e < 3 * N; e += NT) {
           const int f = e / N, j = e % N;
-          cp_async<sizeof(cx<T>)>(s + f * LS + padp(j), W + f * FS + rb + j);
+          cp_async<sizeof(cx<T>)>(s + f * LS + padt<T>(j), W + f * FS + rb + j);
         }
       }
       cp_async_commit();
@@ -263,13 +283,13 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
       __syncthreads();
       if (row_kept && warp < 3) {
         const SLine<T, 1> line{s + warp * LS};
-        warp_fft<T, N, TW, V>(line, line, line, tw, lane);
+        line_fft<T, N, TW, V>(line, line, line, tw, lane);
       }
       cp_async_wait<0>();
     } else {
       if (row_kept && warp < 3) {
         const SLine<T, 1> line{s + warp * LS};
-        warp_fft<T, N, TW, V>(GLoad<T, false>{W + warp * FS + rb}, line, line, tw, lane);
+        line_fft<T, N, TW, V>(GLoad<T, false>{W + warp * FS + rb}, line, line, tw, lane);
       }
     }
     __syncthreads();
@@ -284,8 +304,18 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
       for (int j = threadIdx.x; j < N; j += NT) {
         const int kxi = kfreq(j, N);
         const T kx = SCALED ? (T)kxi * ksx : (T)kxi;
-        const int pj = padp(j);
-        cx<T> n0 = mk((T)0, (T)0), n1 = n0, n2 = n0;
+        const int pj = padt<T>(j);
+        const cx<T> zero = mk((T)0, (T)0);
+        if (xbox && !kept(kxi, a.kmax3)) {  // the state stays zero there and is not written
+#pragma unroll
+          for (int f = 0; f < 3; ++f) {
+            s[f * LS + pj] = zero;
+            if constexpr (G::XPRE && !G::XWIDE) st[f * N + j] = zero;
+            else s[(3 + f) * LS + pj] = zero;
+          }
+          continue;
+        }
+        cx<T> n0 = zero, n1 = n0, n2 = n0;
         if (row_kept && kept(kxi, a.kmax3)) {
           n0 = s[0 * LS + pj];
           n1 = s[1 * LS + pj];
@@ -298,13 +328,11 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
           }
         }
         const T k2 = kx * kx + kyv * kyv + kzv * kzv;
-        const T ik2 = k2 > (T)0 ? (T)1 / k2 : (T)0;
+        const T ik2 = k2 > (T)0 ? recip(k2) : (T)0;
         // P = (k . N_hat) / |k|^2   (Eq. mod_pressure without the factor i)
         const cx<T> p = mk((kx * n0.x + kyv * n1.x + kzv * n2.x) * ik2, (kx * n0.y + kyv * n1.y + kzv * n2.y) * ik2);
         const size_t gi = rb + j;
-        const bool xin = !xbox || kept(kxi, a.kmax3);
-        const cx<T> zero = mk((T)0, (T)0);
-        const cx<T> u0 = xin ? ld_s(0, j) : zero, u1 = xin ? ld_s(1, j) : zero, u2 = xin ? ld_s(2, j) : zero;
+        const cx<T> u0 = ld_s(0, j), u1 = ld_s(1, j), u2 = ld_s(2, j);
         const T nk2 = nu * k2;
         // dU = N_hat - k P - nu |k|^2 u_hat   (Eq. NSfinal)
         const cx<T> d0 = mk(n0.x - kx * p.x - nk2 * u0.x, n0.y - kx * p.y - nk2 * u0.y);
@@ -317,9 +345,7 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
           out[2 * FS + gi] = d2;
         } else {
           cx<T> v0 = zero, v1 = zero, v2 = zero;
-          if (!xin) {
-            // outside the box: the state stays zero there and is not written
-          } else if constexpr (lsrk) {  // 2N stage: dU <- A_s dU + dt RHS, u <- u + B_s dU
+          if constexpr (lsrk) {  // 2N stage: dU <- A_s dU + dt RHS, u <- u + B_s dU
             const T cC = par<T>(a.cC, a.f_cC);
             cx<T> e0 = scal(d0, cC), e1 = scal(d1, cC), e2 = scal(d2, cC);
             if (stage > 0) {
@@ -385,7 +411,7 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
             st[1 * N + j] = conjg(mul_pi(mk(kzv * s0.x - kx * s2.x, kzv * s0.y - kx * s2.y)));
             st[2 * N + j] = conjg(mul_pi(mk(kx * s1.x - kyv * s0.x, kx * s1.y - kyv * s0.y)));
           } else {
-            put_curl_lines<T>(s, pj, LS, v0, v1, v2, kx, kyv, kzv, sc);
+            put_curl_lines<E2 == 0>(s, pj, LS, v0, v1, v2, kx, kyv, kzv, sc);
           }
         }
       }
@@ -399,21 +425,21 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
       if constexpr (G::XPRE && !G::XWIDE) {
         if (warp < 3) {
           const SLine<T, 1> line{s + warp * LS};
-          warp_fft<T, N, TW, V>(line, line, GStore<T, true>{W + warp * FS + rb}, tw, lane);
+          line_fft<T, N, TW, V, E2>(line, line, GStore<T, true>{W + warp * FS + rb}, tw, lane);
         } else {  // omega: from its unpadded row, through a padded work line over rows 3-8
           const int c = warp - 3;
           const SLine<T, 1> work{st + 3 * N + c * LS};
-          warp_fft<T, N, TW, V>(SRow<T>{st + c * N}, work, GStore<T, true>{W + warp * FS + rb}, tw, lane);
+          line_fft<T, N, TW, V, E2>(SRow<T>{st + c * N}, work, GStore<T, true>{W + warp * FS + rb}, tw, lane);
         }
       } else {
         const SLine<T, 1> line{s + warp * LS};
-        warp_fft<T, N, TW, V>(line, line, GStore<T, true>{W + warp * FS + rb}, tw, lane);
+        line_fft<T, N, TW, V, E2>(line, line, GStore<T, true>{W + warp * FS + rb}, tw, lane);
       }
     }
   } else if constexpr (MODE == XM_FWD_STORE) {
     if (warp < 3) {
       const SLine<T, 1> line{s + warp * LS};
-      warp_fft<T, N, TW, V>(GLoad<T, false>{U + warp * FS + rb}, line,
+      line_fft<T, N, TW, V>(GLoad<T, false>{U + warp * FS + rb}, line,
                         GStoreNyquistFree<T>{U + warp * FS + rb, N, ky == NY / 2}, tw, lane);
     }
   } else {
@@ -423,27 +449,27 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
     const bool xbox = MODE == XM_INV_CURL && box_vanish(a);  // columns |kx| >= N/3 hold zeros
     for (int j = threadIdx.x; j < N; j += NT) {
       const size_t gi = rb + j;
-      const int pj = padp(j);
+      const int pj = padt<T>(j);
       const bool xin = !xbox || kept(kfreq(j, N), a.kmax3);
       const cx<T> zero = mk((T)0, (T)0);
       const cx<T> u0 = xin ? U[gi] : zero, u1 = xin ? U[FS + gi] : zero, u2 = xin ? U[2 * FS + gi] : zero;
       const T kx = (T)kfreq(j, N) * ksx;
       if constexpr (MODE == XM_INV_CURL) {
-        put_curl_lines<T>(s, pj, LS, u0, u1, u2, kx, kyv, kzv, sc);
+        put_curl_lines<E2 == 0>(s, pj, LS, u0, u1, u2, kx, kyv, kzv, sc);
       } else if constexpr (MODE == XM_INV_PLAIN) {
-        s[0 * LS + pj] = conjg(scal(u0, sc));
-        s[1 * LS + pj] = conjg(scal(u1, sc));
-        s[2 * LS + pj] = conjg(scal(u2, sc));
+        s[0 * LS + pj] = conjg(E2 ? u0 : scal(u0, sc));
+        s[1 * LS + pj] = conjg(E2 ? u1 : scal(u1, sc));
+        s[2 * LS + pj] = conjg(E2 ? u2 : scal(u2, sc));
       } else {
         const cx<T> d = mul_pi(mk(kx * u0.x + kyv * u1.x + kzv * u2.x, kx * u0.y + kyv * u1.y + kzv * u2.y));
-        s[pj] = conjg(scal(d, sc));
+        s[pj] = conjg(E2 ? d : scal(d, sc));
       }
     }
     __syncthreads();
     cx<T>* dst = (MODE == XM_INV_DIV) ? reinterpret_cast<cx<T>*>(a.D) : W;
     if (warp < NF) {
       const SLine<T, 1> line{s + warp * LS};
-      warp_fft<T, N, TW, V>(line, line, GStore<T, true>{dst + warp * FS + rb}, tw, lane);
+      line_fft<T, N, TW, V, E2>(line, line, GStore<T, true>{dst + warp * FS + rb}, tw, lane);
     }
   }
 }
@@ -495,19 +521,19 @@ __device__ __noinline__ void ytile_fill_kept(cx<T>* s, const cx<T>* __restrict__
 #pragma unroll 8
     for (int e = threadIdx.x; e < TX * L; e += NT) {
       const int x = e % TX, y = ywalk_row<T, TX, L>(e / TX);
-      if (y < lo || y >= lo + gap) cp_async<sizeof(cx<T>)>(s + padp(y) * LD + x, base + (size_t)y * stride + x);
+      if (y < lo || y >= lo + gap) cp_async<sizeof(cx<T>)>(s + padt<T>(y) * LD + x, base + (size_t)y * stride + x);
     }
   } else {
 #pragma unroll 8
     for (int e = threadIdx.x; e < TX * (L - gap); e += NT) {
       const int x = e % TX, r = e / TX, y = r < lo ? r : r + gap;
-      cp_async<sizeof(cx<T>)>(s + padp(y) * LD + x, base + (size_t)y * stride + x);
+      cp_async<sizeof(cx<T>)>(s + padt<T>(y) * LD + x, base + (size_t)y * stride + x);
     }
   }
 #pragma unroll 4
   for (int e = threadIdx.x; e < TX * gap; e += NT) {
     const int x = e % TX, y = lo + e / TX;
-    s[padp(y) * LD + x] = mk((T)0, (T)0);
+    s[padt<T>(y) * LD + x] = mk((T)0, (T)0);
   }
 }
 
@@ -531,7 +557,7 @@ __device__ __forceinline__ void ypass_tile(cx<T>* __restrict__ base, const cx<T>
 #pragma unroll 8
     for (int e = threadIdx.x; e < TX * N; e += NT) {
       const int x = e % TX, y = ywalk_row<T, TX, N>(e / TX);
-      cp_async<sizeof(cx<T>)>(s + padp(y) * LD + x, base + (size_t)y * N + x);
+      cp_async<sizeof(cx<T>)>(s + padt<T>(y) * LD + x, base + (size_t)y * N + x);
     }
   }
   cp_async_commit();
@@ -540,15 +566,15 @@ __device__ __forceinline__ void ypass_tile(cx<T>* __restrict__ base, const cx<T>
 #pragma unroll 1
   for (int c = warp; c < TX; c += NT / 32) {  // warps loop over the columns
     const SLine<T, LD> line{s + c};
-    if constexpr (INV) warp_fft<T, N, N, V>(SLineConj<T, LD>{s + c}, line, line, tw, lane);
-    else warp_fft<T, N, N, V>(line, line, line, tw, lane);
+    if constexpr (INV) line_fft<T, N, N, V>(SLineConj<T, LD>{s + c}, line, line, tw, lane);
+    else line_fft<T, N, N, V>(line, line, line, tw, lane);
   }
   __syncthreads();
 #pragma unroll 8
   for (int e = threadIdx.x; e < TX * N; e += NT) {
     const int x = e % TX, y = ywalk_row<T, TX, N>(e / TX);
     if (PRUNE && !kept(kfreq(y, N), kmax3)) continue;
-    const cx<T> v = s[padp(y) * LD + x];
+    const cx<T> v = s[padt<T>(y) * LD + x];
     base[(size_t)y * N + x] = INV ? conjg(v) : v;
   }
 }
@@ -578,7 +604,7 @@ __global__ void __launch_bounds__(YCfg<T, N, INV, TXO, NY>::THREADS, (YCfg<T, N,
 #pragma unroll 8
     for (int e = threadIdx.x; e < TX * NY; e += NT) {
       const int x = e % TX, y = ywalk_row<T, TX, NY>(e / TX);
-      cp_async<sizeof(cx<T>)>(s + padp(y) * LD + x, base + (size_t)y * N + x);
+      cp_async<sizeof(cx<T>)>(s + padt<T>(y) * LD + x, base + (size_t)y * N + x);
     }
   }
   cp_async_commit();
@@ -587,15 +613,15 @@ __global__ void __launch_bounds__(YCfg<T, N, INV, TXO, NY>::THREADS, (YCfg<T, N,
 #pragma unroll 1
   for (int c = warp; c < TX; c += NT / 32) {
     const SLine<T, LD> line{s + c};
-    if constexpr (INV) warp_fft<T, NY, G::TW, V>(SLineConj<T, LD>{s + c}, line, line, tw, lane);
-    else warp_fft<T, NY, G::TW, V>(line, line, line, tw, lane);
+    if constexpr (INV) line_fft<T, NY, G::TW, V>(SLineConj<T, LD>{s + c}, line, line, tw, lane);
+    else line_fft<T, NY, G::TW, V>(line, line, line, tw, lane);
   }
   __syncthreads();
 #pragma unroll 8
   for (int e = threadIdx.x; e < TX * NY; e += NT) {
     const int x = e % TX, y = ywalk_row<T, TX, NY>(e / TX);
     if (PRUNE && !kept(kfreq(y, NY), kmax3)) continue;
-    const cx<T> v = s[padp(y) * LD + x];
+    const cx<T> v = s[padt<T>(y) * LD + x];
     base[(size_t)y * N + x] = INV ? conjg(v) : v;
   }
 }
@@ -613,6 +639,221 @@ __global__ void __launch_bounds__(YCfg<T, N, INV, TXO>::THREADS, (YCfg<T, N, INV
   cx<T>* base = reinterpret_cast<cx<T>*>(a.W) + (blockIdx.z % fields) * G::FS + (size_t)blockIdx.y * N * N +
                 blockIdx.x * Y::TX;
   ypass_tile<T, N, INV, PRUNE, TXO, Y::THREADS, V>(base, reinterpret_cast<const cx<T>*>(a.tw), a.kmax3, vanish);
+}
+
+// max of a z-pass block's values into *bits (non-negative doubles order like their bit patterns)
+template <int NT>
+__device__ __forceinline__ void zpass_block_max(double m, unsigned long long* bits) {
+  __shared__ double red[NT / 32];
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < NT / 32; ++w) m = fmax(m, red[w]);
+    atomicMax(bits, (unsigned long long)__double_as_longlong(m));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// z-pass of the FP64 form, on fixed point (fixed_point.cuh) from the tile's doubles to the
+// results. Every line has its own scale, except that the three components of u (of omega) of a
+// column share the largest of theirs, so that the products of one component can be added.
+//   c2r   z'/4 from the pair (X_k, X_{M-k}) (L1 of z' is at most four times that of X): physical
+//         values x = v 2^(K - 1083), |v| <= 2^62
+//   u x w products of the v / 2 cut at 2^-62: p = P 2^(Ku + Kw - 2102), |P| <= 2^61; then shifted by
+//         the L1 of the line of products, so that its DFT has 62 bits again
+//   r2c   V = X_k / 2 (quartered post-processing of the pair): X_k = V 2^(Ku + Kw + 1 - sh - 2102)
+// ---------------------------------------------------------------------------
+template <int N, int MODE, int TXO, int NY, int NZ, int V>
+__device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, const int by) {
+  using G = Geometry<double, N, NY, NZ>;
+  typedef cx<double> cd;
+  constexpr int M = G::M;
+  constexpr int TW = G::TW, TS = TW / NZ;
+  constexpr int TX = TXO > 0 ? TXO : G::ZTX;
+  constexpr int LD = odd_ld(6 * TX);
+  constexpr size_t FS = G::FS;
+  constexpr int NF = MODE == ZM_CROSS ? 6 : (MODE == ZM_MAXABS ? 1 : 3), NL = NF * TX;
+  constexpr int GL = cmin(FxLinesPerWarp<M, V>::value, TX);  // lines per warp
+  extern __shared__ unsigned char smraw[];
+  __shared__ int sK[NL];        // scale of a line
+  __shared__ unsigned sN[NL];   // its NaN word
+  __shared__ unsigned sQ[3 * TX];
+  cd* s = reinterpret_cast<cd*>(smraw);
+  fx* sf = reinterpret_cast<fx*>(smraw);
+  const cd* tw = reinterpret_cast<const cd*>(a.tw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int x0 = bx * TX, y = by;
+
+  int klim = M;  // planes kz >= klim hold zeros (a state that vanishes outside the 2/3 box): not read
+  if constexpr (MODE == ZM_LOAD) {
+    const cd* in = reinterpret_cast<const cd*>(a.in);
+    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<double>) {
+      const int n = e % M, x = (e / M) % TX, c = e / (M * TX);
+      cp_async<16>(s + padt<double>(n) * LD + c * TX + x, in + ((size_t)(c * N + x0 + x) * NY + y) * M + n);
+    }
+  } else {
+    const cd* src = reinterpret_cast<const cd*>(MODE == ZM_MAXABS ? a.D : a.W);
+    if constexpr (MODE == ZM_CROSS) {
+      if (rows_vanish(a)) klim = cmin(((NZ == N ? a.kmax3 : a.kmax3z) + 2) / 3, M);
+    }
+    for (int e = threadIdx.x; e < NL * M; e += ZP_THREADS<double>) {
+      const int x = e % TX, k = (e / TX) % M, f = e / (TX * M);
+      if (k < klim) cp_async<16>(s + padt<double>(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
+    }
+  }
+  if (MODE == ZM_CROSS && threadIdx.x < 3 * TX) sQ[threadIdx.x] = 0;
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+  // scales: SUB adjacent lanes walk a line
+  constexpr int SUB = M >= 64 ? 8 : (M >= 16 ? 4 : 2);
+  for (int l0 = warp * (32 / SUB); l0 < NL; l0 += (ZP_THREADS<double> / 32) * (32 / SUB)) {
+    const int l = l0 + lane / SUB, q = lane % SUB;
+    const cd* ln = s + (l < NL ? l : NL - 1);
+    unsigned m = 0;
+    for (int k = q; k < klim; k += SUB) m = max(m, fx_mag(ln[padt<double>(k) * LD]));
+#pragma unroll
+    for (int o = SUB / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int top = fx_top(m);
+    float t = 0.f;
+    for (int k = q; k < klim; k += SUB) {
+      const cd v = ln[padt<double>(k) * LD];
+      t += fx_rel(v.x, top) + fx_rel(v.y, top);
+    }
+    unsigned sh = fx_share(t);
+#pragma unroll
+    for (int o = SUB / 2; o > 0; o >>= 1) sh += __shfl_xor_sync(0xffffffffu, sh, o);
+    if (q == 0 && l < NL) {
+      const FxScale sc = fx_scale(m, sh);
+      sK[l] = sc.K;
+      sN[l] = sc.nan;
+    }
+  }
+  __syncthreads();
+  // the scale of the three components of u (g = 0) or omega (g = 1) of column x
+  auto scale3 = [&](int g, int x) {
+    const int* k = sK + 3 * g * TX + x;
+    return max(k[0], max(k[TX], k[2 * TX]));
+  };
+
+  if constexpr (MODE != ZM_LOAD) {
+    // c2r pre-processing (zpass_body), quartered
+    for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<double>) {
+      const int l = e % NL, k = e / NL;
+      const int K = MODE == ZM_CROSS ? scale3(l / (3 * TX), l % TX) : sK[l];
+      if (k == 0) {
+        const ll r0 = (fx_from(s[l].x, K) + 2) >> 2;  // Im X_0 ignored, X_M = 0
+        sf[l] = mk(r0, -r0);
+      } else {
+        const int pk = padt<double>(k) * LD + l, pm = padt<double>(M - k) * LD + l;
+        const fx xk = fx_from(s[pk], K);
+        const fx xm = M - k < klim ? fx_from(s[pm], K) : mk(0ll, 0ll);
+        int4 w = ldfx(tw + k * TS);
+        w.z = -w.z;
+        w.w = -w.w;
+        const fx A = fx_quarter(xk + conjg(xm)), P = mul_pi(fx_cmul<true>(xk - conjg(xm), w));
+        sf[pk] = conjg(A + P);
+        if (k != M - k) sf[pm] = A - P;
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int l = warp * GL; l < NL; l += (ZP_THREADS<double> / 32) * GL)
+      warp_fft_fx_lines<M, TW, GL, LD, 0, V, FX_IN>(s + l, tw, lane, nullptr);
+    __syncthreads();
+    // now conj(s) = x_{2n} + i x_{2n+1} (physical values, unnormalised c2r)
+  }
+
+  if constexpr (MODE == ZM_CROSS) {
+    auto half = [](fx v) { return mk(v.x >> 1, (-v.y) >> 1); };
+    auto mag = [](fx p) { return ((unsigned)abs((int)(p.x >> 32)) >> 9) + ((unsigned)abs((int)(p.y >> 32)) >> 9) + 2u; };
+    // a warp takes 32 / XW adjacent positions of XW columns: whole warps on one column where the line
+    // is long enough (no bank conflicts along a line)
+    constexpr int XW = M >= 32 ? 1 : TX, CH = 32 / XW, CHUNKS = (M + CH - 1) / CH;
+    static_assert(32 % XW == 0, "a lane keeps its column");
+    for (int it = warp; it < (TX / XW) * CHUNKS; it += ZP_THREADS<double> / 32) {
+      const int x = (it % (TX / XW)) * XW + lane % XW, n = (it / (TX / XW)) * CH + lane / XW;
+      unsigned q[3] = {0, 0, 0};
+      if (M % CH == 0 || n < M) {
+        fx* p = sf + padt<double>(n) * LD + x;
+        const fx u0 = half(p[0 * TX]), u1 = half(p[1 * TX]), u2 = half(p[2 * TX]);
+        const fx w0 = half(p[3 * TX]), w1 = half(p[4 * TX]), w2 = half(p[5 * TX]);
+        // u x omega on both packed points (real and imaginary parts)
+        const fx p0 = mk(fx_cross(u1.x, w2.x, u2.x, w1.x), fx_cross(u1.y, w2.y, u2.y, w1.y));
+        const fx p1 = mk(fx_cross(u2.x, w0.x, u0.x, w2.x), fx_cross(u2.y, w0.y, u0.y, w2.y));
+        const fx p2 = mk(fx_cross(u0.x, w1.x, u1.x, w0.x), fx_cross(u0.y, w1.y, u1.y, w0.y));
+        q[0] = mag(p0);
+        q[1] = mag(p1);
+        q[2] = mag(p2);
+        p[0 * TX] = p0;
+        p[1 * TX] = p1;
+        p[2 * TX] = p2;
+      }
+      // L1 of the three lines of products in units of 2^41
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if constexpr (XW == 1) {
+          q[c] = __reduce_add_sync(0xffffffffu, q[c]);
+        } else {
+#pragma unroll
+          for (int o = XW; o < 32; o *= 2) q[c] += __shfl_xor_sync(0xffffffffu, q[c], o);
+        }
+        if (lane < XW) atomicAdd(sQ + c * TX + x, q[c]);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 * TX) sQ[threadIdx.x] = (unsigned)(__clz(sQ[threadIdx.x]) - 11);
+    __syncthreads();
+  }
+
+  if constexpr (MODE == ZM_CROSS || MODE == ZM_LOAD) {
+#pragma unroll 1
+    for (int l = warp * GL; l < 3 * TX; l += (ZP_THREADS<double> / 32) * GL) {
+      if constexpr (MODE == ZM_CROSS)
+        warp_fft_fx_lines<M, TW, GL, LD, 0, V, FX_SHIFT>(s + l, tw, lane, reinterpret_cast<const int*>(sQ) + l);
+      else
+        warp_fft_fx_lines<M, TW, GL, LD, 0, V, FX_DOUBLE>(s + l, tw, lane, sK + l);
+    }
+    __syncthreads();
+    // r2c post-processing (zpass_body)
+    cd* dst = reinterpret_cast<cd*>(MODE == ZM_CROSS ? a.W : a.U);
+    int kc = M;
+    if (MODE == ZM_CROSS) kc = cmin(((NZ == N ? a.kmax3 : a.kmax3z) + 2) / 3, M);
+    for (int e = threadIdx.x; e < 3 * TX * kc; e += ZP_THREADS<double>) {
+      const int l = e % (3 * TX), k = e / (3 * TX), x = l % TX;
+      const fx zk = sf[padt<double>(k) * LD + l], zm = sf[padt<double>((M - k) % M) * LD + l];
+      const fx A = fx_quarter(zk + conjg(zm)), X = A + mul_mi(fx_cmul<true>(zk - conjg(zm), ldfx(tw + k * TS)));
+      int B;
+      unsigned nan;
+      if constexpr (MODE == ZM_CROSS) {
+        B = max(scale3(0, x) + scale3(1, x) - (int)sQ[l] - 1016, 64);
+        nan = 0;
+#pragma unroll
+        for (int f = 0; f < 6; ++f) nan |= sN[f * TX + x];
+        if (B > 2040) nan = 0x7ff80000u;
+      } else {
+        B = sK[l] + 1;
+        nan = sN[l];
+      }
+      dst[(l / TX) * FS + ((size_t)k * NY + y) * N + x0 + x] = fx_to(X, B, nan);
+    }
+  } else if constexpr (MODE == ZM_STORE) {
+    cd* out = reinterpret_cast<cd*>(a.out);
+    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<double>) {
+      const int n = e % M, x = (e / M) % TX, c = e / (M * TX), l = c * TX + x;
+      out[((size_t)(c * N + x0 + x) * NY + y) * M + n] =
+          fx_to(conjg(sf[padt<double>(n) * LD + l]), sK[l] + 2, sN[l]);
+    }
+  } else if constexpr (MODE == ZM_MAXABS) {
+    double m = 0.0;
+    for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<double>) {
+      const int l = e % TX;
+      const cd v = fx_to(sf[padt<double>(e / TX) * LD + l], sK[l] + 2, sN[l]);
+      m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+    }
+    zpass_block_max<ZP_THREADS<double>>(m, a.maxbits);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -644,7 +885,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     // physical lines (x0 + x, y, :) of the 3 components, packed in pairs
     // (the whole tile in flight at once by cp.async, no register staging)
     const cx<T>* in = reinterpret_cast<const cx<T>*>(a.in);
-    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS) {
+    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<T>) {
       const int n = e % M, x = (e / M) % TX, c = e / (M * TX);
       cp_async<sizeof(cx<T>)>(s + padp(n) * LD + c * TX + x, in + ((size_t)(c * N + x0 + x) * NY + y) * M + n);
     }
@@ -663,7 +904,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
       }
     }
     if (klim < M) {  // the walk of the full fill (compile-time divisors), planes past klim as zeros
-      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS) {
+      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS<T>) {
         const int x = e % TX, k = (e / TX) % M, f = e / (TX * M);
         if (k < klim)
           cp_async<sizeof(cx<T>)>(s + padp(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
@@ -671,7 +912,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
           s[padp(k) * LD + f * TX + x] = mk((T)0, (T)0);
       }
     } else {
-      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS) {
+      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS<T>) {
         const int x = e % TX, k = (e / TX) % M, f = e / (TX * M);
         cp_async<sizeof(cx<T>)>(s + padp(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
       }
@@ -682,7 +923,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     // c2r pre-processing: Z'_k = (X_k + conj X_{M-k}) + i e^{+2 pi i k/N} (X_k - conj X_{M-k}),
     // stored conjugated so that a forward DFT gives the inverse one.
     constexpr int NL = NF * TX;
-    for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS) {
+    for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<T>) {
       const int l = e % NL, k = e / NL;
       if (k == 0) {
         const T r0 = s[l].x;  // Im X_0 ignored, X_M = 0
@@ -704,13 +945,13 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     __syncthreads();
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;  // lines per warp
 #pragma unroll 1
-    for (int l = warp * GL; l < NL; l += (ZP_THREADS / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
+    for (int l = warp * GL; l < NL; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
     __syncthreads();
     // now conj(s) = x_{2n} + i x_{2n+1} (physical values, unnormalised c2r)
   }
 
   if constexpr (MODE == ZM_CROSS) {
-    for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS) {
+    for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<T>) {
       const int x = e % TX, n = e / TX;
       cx<T>* p = s + padp(n) * LD + x;
       const cx<T> u0 = conjg(p[0 * TX]), u1 = conjg(p[1 * TX]), u2 = conjg(p[2 * TX]);
@@ -726,7 +967,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
   if constexpr (MODE == ZM_CROSS || MODE == ZM_LOAD) {
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;
 #pragma unroll 1
-    for (int l = warp * GL; l < 3 * TX; l += (ZP_THREADS / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
+    for (int l = warp * GL; l < 3 * TX; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
     __syncthreads();
     // r2c post-processing: X_k = 1/2 [(Z_k + conj Z_{M-k}) - i e^{-2 pi i k/N} (Z_k - conj Z_{M-k})]
     cx<T>* dst = reinterpret_cast<cx<T>*>(MODE == ZM_CROSS ? a.W : a.U);
@@ -740,7 +981,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     auto post = [&](auto kcc) {
       constexpr int KC = decltype(kcc)::value;  // 0: kc known at run time only
       const int kk = KC > 0 ? KC : kc;
-      for (int e = threadIdx.x; e < 3 * TX * kk; e += ZP_THREADS) {
+      for (int e = threadIdx.x; e < 3 * TX * kk; e += ZP_THREADS<T>) {
         const int x = e % TX, k = (e / TX) % kk, c = e / (TX * kk);
         const int l = c * TX + x;
         const cx<T> zk = s[padp(k) * LD + l], zm = s[padp((M - k) % M) * LD + l];
@@ -758,227 +999,32 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
       post(std::integral_constant<int, 0>{});
   } else if constexpr (MODE == ZM_STORE) {
     cx<T>* out = reinterpret_cast<cx<T>*>(a.out);
-    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS) {
+    for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<T>) {
       const int n = e % M, x = (e / M) % TX, c = e / (M * TX);
       out[((size_t)(c * N + x0 + x) * NY + y) * M + n] = conjg(s[padp(n) * LD + c * TX + x]);
     }
   } else if constexpr (MODE == ZM_MAXABS) {
     double m = 0.0;
-    for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS) {
+    for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<T>) {
       const int x = e % TX, n = e / TX;
       const cx<T> v = s[padp(n) * LD + x];
       m = fmax(m, fmax(fabs((double)v.x), fabs((double)v.y)));
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ double red[ZP_THREADS / 32];
-    if (lane == 0) red[warp] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < ZP_THREADS / 32; ++w) m = fmax(m, red[w]);
-      // non-negative doubles order like their bit patterns
-      atomicMax(a.maxbits, (unsigned long long)__double_as_longlong(m));
-    }
+    zpass_block_max<ZP_THREADS<T>>(m, a.maxbits);
   }
 }
 
 template <typename T, int N, int MODE, int TXO = 0, int NY = N, int NZ = N, int V = 0>
-__global__ void __launch_bounds__(ZP_THREADS, (Geometry<T, N, NY, NZ>::ZMIN)) k_zpass(PassArgs a) {
-  zpass_body<T, N, MODE, TXO, NY, NZ, V>(a, blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(ZP_THREADS<T>, (Geometry<T, N, NY, NZ>::ZMIN)) k_zpass(PassArgs a) {
+  if constexpr (sizeof(T) == 8) zpass64_body<N, MODE, TXO, NY, NZ, V>(a, blockIdx.x, blockIdx.y);
+  else zpass_body<T, N, MODE, TXO, NY, NZ, V>(a, blockIdx.x, blockIdx.y);
 }
 
 // Batched form (ensembles): member blockIdx.z (TXO: a tuned tile width).
 template <typename T, int N, int MODE, int TXO = 0, int V = 0>
-__global__ void __launch_bounds__(ZP_THREADS, (Geometry<T, N>::ZMIN)) k_zpass_b(const __grid_constant__ BatchArgs B) {
-  zpass_body<T, N, MODE, TXO, N, N, V>(B.a[blockIdx.z], blockIdx.x, blockIdx.y);
-}
-
-// ---------------------------------------------------------------------------
-// z-pass of the right-hand side with register-resident columns (M = N/2 a
-// multiple of 32, M >= 128): a block owns ZTX adjacent x at fixed y and has one
-// warp per x. After a coalesced load of the 6 fields, each warp on its own
-// column: c2r of u (pre-processing fused into the first pass; physical values
-// parked in the column's own lines), c2r of omega one component at a time
-// with the cross product accumulated incrementally, r2c of each finished
-// component with the post-processing done through lane shuffles. Only the load
-// and the store need block barriers.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ cx<T> pmul(cx<T> a, cx<T> b) { return mk(a.x * b.x, a.y * b.y); }
-
-template <typename T, int N>
-struct ZCross {
-  static constexpr int M = N / 2;
-  static constexpr int V = M / 32;
-  static constexpr bool enabled = (M % 32 == 0) && (M >= 128) && CanonPlan<M>::valid();
-};
-
-// Twiddles the z-cross warps reuse for every line: the canonical-FFT bases
-// and exp(-2 pi i lane / N); exp(-2 pi i k / N) for k = lane + 32 m is then
-// tl * tw[32 m] (a broadcast load).
-template <typename T, int N>
-struct ZTw {
-  CanonTw<T, N / 2, N> fft;
-  cx<T> tl;
-  __device__ __forceinline__ void load(const cx<T>* __restrict__ tw, int lane) {
-    fft.load(tw, lane);
-    tl = ldro(tw + lane);
-  }
-  __device__ __forceinline__ cx<T> wk(const cx<T>* __restrict__ tw, int m) const {
-    if constexpr (sizeof(T) == 4) return m == 0 ? tl : cmul(tl, ldro(tw + 32 * m));
-    else return ldro(tw + (threadIdx.x & 31) + 32 * m);
-  }
-};
-
-// c2r of one column line (element k at ln[padp(k) * LD]) into canonical
-// physical pairs v[m] = x_{2n} + i x_{2n+1}, n = lane + 32 m. The pre-processing
-// Z'_k = (X_k + conj X_{M-k}) + i e^{+2 pi i k/N} (X_k - conj X_{M-k}) is fused
-// into the load (stored conjugated: a forward DFT then gives the inverse one).
-template <typename T, int N, int LD = Geometry<T, N>::ZLD>
-__device__ __forceinline__ void zc_c2r(cx<T> (&v)[N / 64], cx<T>* ln, const ZTw<T, N>& zt,
-                                       const cx<T>* __restrict__ tw, int lane) {
-  constexpr int M = N / 2, V = M / 32;
-  const cx<T>* pa = ln + padp(lane) * LD;            // X_k, k = lane + 32 m
-  const cx<T>* pb = ln + padp((32 - lane) & 31) * LD;  // X_{M-k} for lane > 0
-#pragma unroll
-  for (int m = 0; m < V; ++m) {
-    const cx<T> xk = pa[34 * m * LD];
-    cx<T> xm;
-    if (lane != 0) xm = pb[34 * (V - 1 - m) * LD];
-    else xm = (m == 0) ? mk((T)0, (T)0) : ln[34 * (V - m) * LD];
-    cx<T> z;
-    if (lane == 0 && m == 0) {
-      z = mk(xk.x, xk.x);  // Im X_0 ignored, X_M = 0
-    } else {
-      const cx<T> wk = zt.wk(tw, m);
-      const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
-      z = A + mul_pi(cmul(conjg(wk), B));
-    }
-    v[m] = conjg(z);
-  }
-  __syncwarp();
-  warp_fft_canon<T, M, N, LD>(v, ln, zt.fft, tw, lane);
-#pragma unroll
-  for (int m = 0; m < V; ++m) v[m] = conjg(v[m]);
-}
-
-// r2c of canonical physical pairs c, then X_k for k < kc written into line out:
-// X_k = 1/2 [(Z_k + conj Z_{M-k}) - i e^{-2 pi i k/N} (Z_k - conj Z_{M-k})],
-// the partner Z_{M-k} coming from lane 32 - lane (lane 0 holds both).
-template <typename T, int N, int LD = Geometry<T, N>::ZLD>
-__device__ __forceinline__ void zc_r2c(cx<T> (&c)[N / 64], cx<T>* scratch, cx<T>* out, int kc, const ZTw<T, N>& zt,
-                                       const cx<T>* __restrict__ tw, int lane) {
-  constexpr int M = N / 2, V = M / 32;
-  warp_fft_canon<T, M, N, LD>(c, scratch, zt.fft, tw, lane);
-  const int partner = (32 - lane) & 31;
-  cx<T>* po = out + padp(lane) * LD;
-#pragma unroll
-  for (int m = 0; m < V; ++m) {
-    cx<T> zo;
-    zo.x = __shfl_sync(0xffffffffu, c[V - 1 - m].x, partner);
-    zo.y = __shfl_sync(0xffffffffu, c[V - 1 - m].y, partner);
-    if (lane == 0) zo = c[(V - m) % V];
-    const cx<T> wk = zt.wk(tw, m);
-    const cx<T> A = c[m] + conjg(zo), B = c[m] - conjg(zo);
-    if (lane + 32 * m < kc) po[34 * m * LD] = scal(A + mul_mi(cmul(wk, B)), (T)0.5);
-  }
-}
-
-// Warps per z-cross block: 6 ZTX c2r lines and 3 ZTX r2c lines split evenly
-// (4 and 2 per warp).
-template <typename T, int N>
-struct ZCrossWarps {  // at most 12, so that two blocks share an SM and overlap load and transform
-  static constexpr int full = (3 * Geometry<T, N>::ZTX) / 2 >= 1 ? (3 * Geometry<T, N>::ZTX) / 2 : 1;
-  static constexpr int value = full > 12 ? 12 : full;
-};
-
-// Tile element walk for the z-cross block (load, cross product, store): one
-// warp instruction covers kz = 16 g + (ZTX/2) kq + c for kq = lane / ZTX and
-// x = lane % ZTX, which touches every shared-memory bank pair exactly twice
-// with the odd row stride ZLD, while each global access reads whole 32-byte
-// sectors of ZTX contiguous x.
-template <typename T, int N>
-struct ZWalk {
-  static constexpr int TX = Geometry<T, N>::ZTX;
-  static constexpr int S = TX / 2 > 0 ? TX / 2 : 1;  // values of c
-  static constexpr int G16 = (N / 2) / 16;           // values of g
-  static constexpr int ITEMS = G16 * S;              // per field
-};
-
-template <typename T, int N>
-__global__ void __launch_bounds__(32 * ZCrossWarps<T, N>::value, (ZCrossWarps<T, N>::value > 16 ? 1 : 2)) k_zcross(PassArgs a) {
-  using G = Geometry<T, N>;
-  using ZW = ZWalk<T, N>;
-  constexpr int M = G::M, TX = G::ZTX, LD = G::ZLD, V = M / 32;
-  constexpr int NW = ZCrossWarps<T, N>::value;
-  constexpr size_t FS = G::FS;
-  static_assert(32 % TX == 0 && (M % 16) == 0, "z-cross tile walk");
-  extern __shared__ unsigned char smraw[];
-  cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
-  const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
-  cx<T>* W = reinterpret_cast<cx<T>*>(a.W);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int x0 = blockIdx.x * TX, y = blockIdx.y;
-  int kc = (a.kmax3 + 2) / 3;
-  if (kc > M) kc = M;
-  const int tx = lane % TX, kq = lane / TX;
-  // lane part of the walk: k = 16 g + S kq + c  ->  padp(k) = 17 g + S kq + c
-  const cx<T>* gl = W + ((size_t)(ZW::S * kq) * N + y) * N + x0 + tx;
-  cx<T>* sl = s + (ZW::S * kq) * LD + tx;
-
-  if (rows_vanish(a)) {  // planes kz >= kc of a state that vanishes outside the 2/3 box: zeros
-    for (int it = w; it < 6 * ZW::ITEMS; it += NW) {
-      const int f = it / ZW::ITEMS, r = it % ZW::ITEMS, g = r / ZW::S, c = r % ZW::S;
-      sl[(17 * g + c) * LD + f * TX] =
-          16 * g + ZW::S * kq + c < kc ? gl[f * FS + (size_t)(16 * g + c) * N * N] : mk((T)0, (T)0);
-    }
-  } else {
-    for (int it = w; it < 6 * ZW::ITEMS; it += NW) {
-      const int f = it / ZW::ITEMS, r = it % ZW::ITEMS, g = r / ZW::S, c = r % ZW::S;
-      sl[(17 * g + c) * LD + f * TX] = gl[f * FS + (size_t)(16 * g + c) * N * N];
-    }
-  }
-  ZTw<T, N> zt;
-  zt.load(tw, lane);
-  __syncthreads();
-  // c2r of the 6 TX lines (u and omega of each column); physical pairs are
-  // written back into the same line at canonical positions
-  cx<T> v[V];
-#pragma unroll 1
-  for (int l = w; l < 6 * TX; l += NW) {
-    cx<T>* ln = s + l;
-    zc_c2r<T, N>(v, ln, zt, tw, lane);
-    cx<T>* pa = ln + padp(lane) * LD;
-#pragma unroll
-    for (int m = 0; m < V; ++m) pa[34 * m * LD] = v[m];
-  }
-  __syncthreads();
-  // u x omega at every point, into the u lines
-  for (int it = w; it < ZW::ITEMS; it += NW) {
-    const int g = it / ZW::S, c = it % ZW::S;
-    cx<T>* p = sl + (17 * g + c) * LD;
-    const cx<T> u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];
-    const cx<T> w0 = p[3 * TX], w1 = p[4 * TX], w2 = p[5 * TX];
-    p[0 * TX] = mk(u1.x * w2.x - u2.x * w1.x, u1.y * w2.y - u2.y * w1.y);
-    p[1 * TX] = mk(u2.x * w0.x - u0.x * w2.x, u2.y * w0.y - u0.y * w2.y);
-    p[2 * TX] = mk(u0.x * w1.x - u1.x * w0.x, u0.y * w1.y - u1.y * w0.y);
-  }
-  __syncthreads();
-  // r2c of the 3 TX product lines, X_k (k < kc) written back into the line
-#pragma unroll 1
-  for (int l = w; l < 3 * TX; l += NW) {
-    cx<T>* ln = s + l;
-    const cx<T>* pa = ln + padp(lane) * LD;
-#pragma unroll
-    for (int m = 0; m < V; ++m) v[m] = pa[34 * m * LD];
-    __syncwarp();
-    zc_r2c<T, N>(v, ln, ln, kc, zt, tw, lane);
-  }
-  __syncthreads();
-  cx<T>* gd = W + ((size_t)(ZW::S * kq) * N + y) * N + x0 + tx;
-  for (int it = w; it < 3 * ZW::ITEMS; it += NW) {
-    const int f = it / ZW::ITEMS, r = it % ZW::ITEMS, g = r / ZW::S, c = r % ZW::S;
-    if (16 * g + ZW::S * kq + c < kc) gd[f * FS + (size_t)(16 * g + c) * N * N] = sl[(17 * g + c) * LD + f * TX];
-  }
+__global__ void __launch_bounds__(ZP_THREADS<T>, (Geometry<T, N>::ZMIN)) k_zpass_b(const __grid_constant__ BatchArgs B) {
+  if constexpr (sizeof(T) == 8) zpass64_body<N, MODE, TXO, N, N, V>(B.a[blockIdx.z], blockIdx.x, blockIdx.y);
+  else zpass_body<T, N, MODE, TXO, N, N, V>(B.a[blockIdx.z], blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -1761,7 +1807,7 @@ struct SolverImpl {
   static constexpr int M = G::M;
   static constexpr bool ISO = NY == N && NZ == N;
   static constexpr int ROWS = M * NY;  // x-pass rows (kz, ky)
-  static constexpr bool BATCHED = ISO && N <= BATCH_MAX_N && !ZCross<T, N>::enabled;
+  static constexpr bool BATCHED = ISO && N <= BATCH_MAX_N;
   // non-cubic grids with 256-point FP32 z-lines use the quarter-warp z-pass of 256^3
   static constexpr bool Z8_BOX = !ISO && NZ == 256 && sizeof(T) == 4 && N % 16 == 0;
   // each direction's 2/3 cut-off (3|k_i| < kmax3 of that direction)
@@ -1784,15 +1830,14 @@ struct SolverImpl {
   // PLAN_Z (z-pass), PLAN_YF (y-forward).
   static constexpr int PLANS = (ISO && N <= BATCH_MAX_N) ? 2 : 1;
   // The handle's initial plan mask: AltPlan in the passes where it measured faster on
-  // GB300 (per-pass CUDA-event times of both schedules, 100 graph-replayed steps; FP64
-  // passes whose default has a radix-16 pass or radix-8 passes only run about twice as
-  // fast with radix 4). dns_tune_tiles re-measures on the machine at hand.
+  // GB300 (per-pass CUDA-event times of both schedules; FP64 at 64^3: 213 against 282 us a step, since
+  // two radix-8 passes of 64-point lines leave three lanes in four idle, and 3 - 15 % slower elsewhere). dns_tune_tiles re-measures on the machine at hand.
   static constexpr int default_plan() {
     if constexpr (PLANS == 1) {
       return 0;
     } else if constexpr (sizeof(T) == 8) {
       constexpr int XYY = (1 << PLAN_X) | (1 << PLAN_YI) | (1 << PLAN_YF);
-      return (N == 16 || N == 48 || N == 64 || N == 128) ? XYY : 0;
+      return (N == 16 || N == 64) ? XYY : 0;
     } else {
       switch (N) {
         case 48: return (1 << PLAN_X) | (1 << PLAN_YF);
@@ -1817,10 +1862,8 @@ struct SolverImpl {
     if (e == cudaSuccess) e = smem_attr(k_ypass<T, N, 1, 0, TXO, N, N, V>, YCfg<T, N, 1, TXO>::SMEM);
     if (e == cudaSuccess) e = smem_attr(k_ypass<T, N, 1, 0, TXO, N, N, V, 1>, YCfg<T, N, 1, TXO>::SMEM);
     if (e == cudaSuccess) e = smem_attr(k_ypass<T, N, 0, 1, TXO, N, N, V>, YCfg<T, N, 0, TXO>::SMEM);
-    if constexpr (!ZCross<T, N>::enabled) {
-      if (e == cudaSuccess) e = smem_attr(k_ypass_b<T, N, 1, 0, TXO, V>, YCfg<T, N, 1, TXO>::SMEM);
-      if (e == cudaSuccess) e = smem_attr(k_ypass_b<T, N, 0, 1, TXO, V>, YCfg<T, N, 0, TXO>::SMEM);
-    }
+    if (e == cudaSuccess) e = smem_attr(k_ypass_b<T, N, 1, 0, TXO, V>, YCfg<T, N, 1, TXO>::SMEM);
+    if (e == cudaSuccess) e = smem_attr(k_ypass_b<T, N, 0, 1, TXO, V>, YCfg<T, N, 0, TXO>::SMEM);
   }
   template <int TXO>
   static void tile_attr(cudaError_t& e) {
@@ -1837,8 +1880,8 @@ struct SolverImpl {
   }
   // z-pass tile widths offered besides the default (the generic z-pass of the small grids)
   static constexpr bool ztile_ok(int t) {
-    return ISO && N <= BATCH_MAX_N && !ZCross<T, N>::enabled && t >= 4 && t <= 32 && pow2_part(N) % t == 0 &&
-           G::zbytes(t) <= 112 * 1024;
+    return ISO && N <= BATCH_MAX_N && t >= 4 && t <= 32 && pow2_part(N) % t == 0 &&
+           (size_t)padded_len(M) * odd_ld(6 * t) * sizeof(cx<T>) <= 112 * 1024;
   }
   template <int TXO>
   static void ztile_attr(cudaError_t& e) {
@@ -1860,7 +1903,7 @@ struct SolverImpl {
   template <int TXO, int V = 0>
   static void z_go(const PassArgs& a, cudaStream_t st) {
     constexpr int TX = TXO > 0 ? TXO : G::ZTX;
-    k_zpass<T, N, ZM_CROSS, TXO, NY, NZ, V><<<dim3(N / TX, NY), ZP_THREADS, G::zbytes(TX), st>>>(a);
+    k_zpass<T, N, ZM_CROSS, TXO, NY, NZ, V><<<dim3(N / TX, NY), ZP_THREADS<T>, G::zbytes(TX), st>>>(a);
   }
   // PR: the y-inverse of a stage whose state vanishes outside the 2/3 box (k_ypass)
   template <int INV, int PRUNE, int TXO, int V = 0, int PR = 0>
@@ -1926,7 +1969,6 @@ struct SolverImpl {
       DNS_ATTR((k_ypass<T, N, 0, 1, 0, N, N, 1>), (YCfg<T, N, 0, 0>::SMEM));
       DNS_ATTR((k_zpass<T, N, ZM_CROSS, 0, N, N, 1>), G::ZSMEM);
     }
-    if constexpr (ISO && ZCross<T, N>::enabled) DNS_ATTR((k_zcross<T, N>), G::ZSMEM);
     if constexpr (ISO && N == 512 && sizeof(T) == 4) DNS_ATTR((k_zcross16p<T, N>), Z16P<T>::SMEM);
     if constexpr (ISO && N == 1024 && sizeof(T) == 4) DNS_ATTR((k_zcross32p<T, N>), Z32P<T>::SMEM);
     if constexpr (ISO && N == 256 && sizeof(T) == 4) DNS_ATTR((k_zcross8q<T, N>), Z8Q<T>::SMEM);
@@ -1959,14 +2001,10 @@ struct SolverImpl {
       z_go<0>(a, st);
     else if constexpr (N == 512 && sizeof(T) == 4)
       k_zcross16p<T, N><<<num_sms(), 32 * Z16P<T>::NW, Z16P<T>::SMEM, st>>>(a);
-    else if constexpr (N == 512)  // FP64: the generic z-pass, measured faster than a half-warp
-      z_go<0>(a, st);             // radix-16 kernel (38.2 against 41.2 ms per launch)
     else if constexpr (N == 1024 && sizeof(T) == 4)
       k_zcross32p<T, N><<<num_sms(), 32 * Z32P<T>::NW, Z32P<T>::SMEM, st>>>(a);
     else if constexpr (N == 256 && sizeof(T) == 4)
       k_zcross8q<T, N><<<dim3(N / Z8Q<T>::TX, N), 32 * Z8Q<T>::NW, Z8Q<T>::SMEM, st>>>(a);
-    else if constexpr (ZCross<T, N>::enabled)
-      k_zcross<T, N><<<dim3(N / G::ZTX, N), 32 * ZCrossWarps<T, N>::value, G::ZSMEM, st>>>(a);
     else {
       with_plan(bit(a.plan, PLAN_Z), [&](auto v) {
         constexpr int V = decltype(v)::value;
@@ -2075,7 +2113,7 @@ struct SolverImpl {
   template <int TXO, int V>
   static void zb_go(const BatchArgs& B, int count, cudaStream_t st) {
     constexpr int TX = TXO > 0 ? TXO : G::ZTX;
-    k_zpass_b<T, N, ZM_CROSS, TXO, V><<<dim3(N / TX, N, count), ZP_THREADS, G::zbytes(TX), st>>>(B);
+    k_zpass_b<T, N, ZM_CROSS, TXO, V><<<dim3(N / TX, N, count), ZP_THREADS<T>, G::zbytes(TX), st>>>(B);
   }
   template <int V>
   static void zb_stage(int tile, const BatchArgs& B, int count, cudaStream_t st) {
@@ -2133,7 +2171,7 @@ struct SolverImpl {
 
   static cudaError_t forward3d(const PassArgs& a, cudaStream_t st) {
     using Y = YCfg<T, N, 0, 0, NY>;
-    k_zpass<T, N, ZM_LOAD, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS, G::ZSMEM, st>>>(a);
+    k_zpass<T, N, ZM_LOAD, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS<T>, G::ZSMEM, st>>>(a);
     k_ypass<T, N, 0, 0, 0, NY, NZ><<<dim3(N / Y::TX, M, 3), Y::THREADS, Y::SMEM, st>>>(
         reinterpret_cast<cx<T>*>(a.U), reinterpret_cast<const cx<T>*>(a.tw), k3y(a));
     k_xpass<T, N, XM_FWD_STORE, NY, NZ><<<ROWS, XP_THREADS, G::XSMEM, st>>>(f32args(a));
@@ -2145,7 +2183,7 @@ struct SolverImpl {
     k_xpass<T, N, XM_INV_PLAIN, NY, NZ><<<ROWS, XP_THREADS, G::XSMEM, st>>>(f32args(a));
     k_ypass<T, N, 1, 0, 0, NY, NZ><<<dim3(N / Y::TX, M, 3), Y::THREADS, Y::SMEM, st>>>(
         reinterpret_cast<cx<T>*>(a.W), reinterpret_cast<const cx<T>*>(a.tw), k3y(a));
-    k_zpass<T, N, ZM_STORE, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS, G::ZSMEM, st>>>(a);
+    k_zpass<T, N, ZM_STORE, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS<T>, G::ZSMEM, st>>>(a);
     return cudaGetLastError();
   }
 
@@ -2157,7 +2195,7 @@ struct SolverImpl {
     k_ypass<T, N, 1, 0, 0, NY, NZ><<<dim3(N / Y::TX, M, 1), Y::THREADS, Y::SMEM, st>>>(
         reinterpret_cast<cx<T>*>(a.D), reinterpret_cast<const cx<T>*>(a.tw), k3y(a));
     cudaMemsetAsync(a.maxbits, 0, sizeof(unsigned long long), st);
-    k_zpass<T, N, ZM_MAXABS, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS, G::ZSMEM, st>>>(a);
+    k_zpass<T, N, ZM_MAXABS, 0, NY, NZ><<<dim3(N / G::ZTX, NY), ZP_THREADS<T>, G::ZSMEM, st>>>(a);
     return cudaGetLastError();
   }
 
