@@ -1,8 +1,7 @@
-// Pointwise subgrid-stress network 10 -> 64 (SiLU) -> 64 (SiLU) -> 6 on BF16
-// tensor cores with FP32 accumulation: inference on the 5th-generation tensor
-// cores (tcgen05.mma, accumulators in TMEM, k_mlp_tc), training (forward +
-// backward with the weight-gradient products also on the tensor cores, WMMA
-// m16n16k16 fragments, k_mlp<1>) and Adam on FP32 master weights.
+// Pointwise subgrid-stress network 10 -> 64 (SiLU) -> 64 (SiLU) -> 6 on the 5th-generation tensor
+// cores (tcgen05.mma, BF16 operands in shared memory, FP32 accumulators in TMEM): inference
+// (k_mlp_tc), the training pass (k_mlp_train: forward, backward and the weight gradients) and Adam on
+// FP32 master weights (k_reduce).
 //
 // Parameter vector (floats), in this order:
 //   in_shift[10] in_scale[10] W1[10][64] b1[64] W2[64][64] b2[64] W3[64][6]
@@ -13,11 +12,9 @@
 // out_scale)^2. Feature and stress arrays are planar: X[f * P + p], T[c * P + p].
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <mma.h>
 
 #include <cmath>
 #include <cstring>
-#include <vector>
 
 #include "../../include/dns.h"
 #include "dns_internal.h"
@@ -26,298 +23,65 @@ namespace dns {
 void set_error_message(const char* msg);
 }
 
-using namespace nvcuda;
-
 namespace {
 
 constexpr int NIN = 10, NH = 64, NOUT = 6;
 constexpr int O_INSH = 0, O_INSC = 10, O_W1 = 20, O_B1 = 660, O_W2 = 724, O_B2 = 4820, O_W3 = 4884, O_B3 = 5268,
               O_OUTSC = 5274, O_OUTSH = 5280, NPARAM = 5286;
 constexpr int TRAIN_BEGIN = O_W1, TRAIN_END = O_OUTSC;  // trainable range [W1 .. b3]
-constexpr int WARPS = 4, THREADS = 32 * WARPS;
-// packed BF16 weights: W1p[16][64] (rows >= 10 zero), W2[64][64], W3p[64][16] (cols >= 6 zero)
-constexpr int PW1 = 0, PW2 = 16 * 64, PW3 = PW2 + 64 * 64, NPACK = PW3 + 64 * 16;
+constexpr int NTRAIN = TRAIN_END - TRAIN_BEGIN;  // 5254
 
 typedef __nv_bfloat16 bf;
 
-// per-warp shared-memory work area (bytes, all offsets multiples of 32)
-constexpr int A0_B = 16 * 16 * 2, Z1_B = 16 * 64 * 4, H_B = 16 * 64 * 2, Y_B = 16 * 16 * 4, DY_B = 16 * 16 * 2,
-              G_B = 16 * 64 * 4, T_B = 16 * 16 * 4;
-constexpr int OFF_A0 = 0, OFF_Z1 = OFF_A0 + A0_B, OFF_H1 = OFF_Z1 + Z1_B, OFF_Z2 = OFF_H1 + H_B, OFF_H2 = OFF_Z2 + Z1_B,
-              OFF_Y = OFF_H2 + H_B, OFF_DY = OFF_Y + Y_B, OFF_G = OFF_DY + DY_B, OFF_DZ2 = OFF_G + G_B,
-              OFF_DZ1 = OFF_DZ2 + H_B, OFF_T = OFF_DZ1 + H_B, WARP_B = OFF_T + T_B;
-// block area: packed weights, then FP32 gradient accumulators (trainable range) and the loss
-constexpr int BLK_W_B = NPACK * 2, BLK_G = TRAIN_END - TRAIN_BEGIN;
-constexpr int SMEM_B = BLK_W_B + WARPS * WARP_B + (BLK_G + 8) * 4;
-
-
-// SiLU and its derivative with the fast exponential and division intrinsics (their
-// relative error, ~1e-6, is far below the BF16 rounding the activations then take)
-__device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.f + __expf(-z)); }
-__device__ __forceinline__ float dsilu(float z) {
-  const float s = __fdividef(1.f, 1.f + __expf(-z));
-  return s * (1.f + z * (1.f - s));
+// byte offset of element (r, k) of a K-major operand with K columns in the core-matrix layout
+__host__ __device__ constexpr int tc_off(int r, int k, int K) {
+  return ((r >> 3) * (K >> 3) + (k >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2;
 }
+// The BF16 weights as the B operands of the kernels, byte for byte the shared-memory image (made once
+// per change of the parameters, so that a block stages them by 16-byte copies; gathering them from
+// the row-major matrices in every block took 5 of the 17 us of a small inference): for the
+// forward products W1^T (64 x 16), W2^T (64 x 64), W3^T (16 x 64, rows >= 6 zero), for the backward
+// ones W2 (64 x 64) and W3 (64 x 16, columns >= 6 zero).
+constexpr int IMG_W1 = 0, IMG_W2 = IMG_W1 + 2048, IMG_W3 = IMG_W2 + 8192, IMG_FWD = IMG_W3 + 2048, IMG_W2B = IMG_FWD,
+              IMG_W3B = IMG_W2B + 8192, IMG_BYTES = IMG_W3B + 2048;
 
-__global__ void k_pack(const float* __restrict__ p, bf* __restrict__ w) {
-  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < NPACK; i += blockDim.x * gridDim.x) {
-    float v = 0.f;
-    if (i < PW2) {
-      const int k = i / 64, n = i % 64;
-      v = k < NIN ? p[O_W1 + k * 64 + n] : 0.f;
-    } else if (i < PW3) {
-      v = p[O_W2 + (i - PW2)];
-    } else {
-      const int k = (i - PW3) / 16, n = (i - PW3) % 16;
-      v = n < NOUT ? p[O_W3 + k * NOUT + n] : 0.f;
-    }
-    w[i] = __float2bfloat16(v);
+// puts parameter i (value v) where the image holds it
+__device__ __forceinline__ void pack_param(int i, float v, unsigned char* img) {
+  const bf w = __float2bfloat16(v);
+  auto put = [&](int at) { *reinterpret_cast<bf*>(img + at) = w; };
+  if (i >= O_W1 && i < O_B1) {
+    const int k = (i - O_W1) / NH, n = (i - O_W1) % NH;
+    put(IMG_W1 + tc_off(n, k, 16));
+  } else if (i >= O_W2 && i < O_B2) {
+    const int k = (i - O_W2) / NH, n = (i - O_W2) % NH;
+    put(IMG_W2 + tc_off(n, k, 64));
+    put(IMG_W2B + tc_off(k, n, 64));
+  } else if (i >= O_W3 && i < O_B3) {
+    const int k = (i - O_W3) / NOUT, c = (i - O_W3) % NOUT;
+    put(IMG_W3 + tc_off(c, k, 64));
+    put(IMG_W3B + tc_off(k, c, 16));
   }
 }
-
-typedef wmma::fragment<wmma::matrix_a, 16, 16, 16, bf, wmma::row_major> FragA;
-typedef wmma::fragment<wmma::matrix_a, 16, 16, 16, bf, wmma::col_major> FragAT;
-typedef wmma::fragment<wmma::matrix_b, 16, 16, 16, bf, wmma::row_major> FragB;
-typedef wmma::fragment<wmma::matrix_b, 16, 16, 16, bf, wmma::col_major> FragBT;
-typedef wmma::fragment<wmma::accumulator, 16, 16, 16, float> FragC;
-
-// Adds a 16x16 FP32 tile (row-major in `tile`) into acc[(r0 + r) * ld + c0 + c] (shared atomics).
-__device__ __forceinline__ void add_tile(float* acc, int ld, int r0, int c0, int rmax, int cmax, const float* tile,
-                                         int lane) {
-  for (int e = lane; e < 256; e += 32) {
-    const int r = e >> 4, c = e & 15;
-    if (r0 + r < rmax && c0 + c < cmax) atomicAdd(&acc[(r0 + r) * ld + c0 + c], tile[e]);
-  }
+__global__ void k_pack(const float* __restrict__ p, unsigned char* __restrict__ img) {
+  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < NPARAM; i += blockDim.x * gridDim.x) pack_param(i, p[i], img);
 }
 
-// TRAIN = 0: Y = network(X). TRAIN = 1: accumulate the loss and the gradients
-// of the trainable parameters into gsum (global, FP32) for targets T.
-template <int TRAIN>
-__global__ void __launch_bounds__(THREADS) k_mlp(const float* __restrict__ prm, const bf* __restrict__ wpack,
-                                                  const float* __restrict__ X, int P, float* __restrict__ Y,
-                                                  const float* __restrict__ T, float* __restrict__ gsum) {
-  extern __shared__ __align__(128) unsigned char sm[];
-  bf* sw = reinterpret_cast<bf*>(sm);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* wb = sm + BLK_W_B + warp * WARP_B;
-  bf* A0 = reinterpret_cast<bf*>(wb + OFF_A0);
-  float* Z1 = reinterpret_cast<float*>(wb + OFF_Z1);
-  bf* H1 = reinterpret_cast<bf*>(wb + OFF_H1);
-  float* Z2 = reinterpret_cast<float*>(wb + OFF_Z2);
-  bf* H2 = reinterpret_cast<bf*>(wb + OFF_H2);
-  float* Yt = reinterpret_cast<float*>(wb + OFF_Y);
-  bf* DY = reinterpret_cast<bf*>(wb + OFF_DY);
-  float* G = reinterpret_cast<float*>(wb + OFF_G);
-  bf* DZ2 = reinterpret_cast<bf*>(wb + OFF_DZ2);
-  bf* DZ1 = reinterpret_cast<bf*>(wb + OFF_DZ1);
-  float* TT = reinterpret_cast<float*>(wb + OFF_T);
-  float* acc = reinterpret_cast<float*>(sm + BLK_W_B + WARPS * WARP_B);  // [BLK_G] + loss
-
-  static_assert(NPACK % 8 == 0, "16-byte weight staging");
-  for (int i = threadIdx.x; i < NPACK / 8; i += THREADS)
-    reinterpret_cast<uint4*>(sw)[i] = reinterpret_cast<const uint4*>(wpack)[i];
-  if (TRAIN)
-    for (int i = threadIdx.x; i < BLK_G + 8; i += THREADS) acc[i] = 0.f;
-  __syncthreads();
-  const bf* W1p = sw + PW1;
-  const bf* W2s = sw + PW2;
-  const bf* W3p = sw + PW3;
-  float* gW1 = acc + (O_W1 - TRAIN_BEGIN);
-  float* gb1 = acc + (O_B1 - TRAIN_BEGIN);
-  float* gW2 = acc + (O_W2 - TRAIN_BEGIN);
-  float* gb2 = acc + (O_B2 - TRAIN_BEGIN);
-  float* gW3 = acc + (O_W3 - TRAIN_BEGIN);
-  float* gb3 = acc + (O_B3 - TRAIN_BEGIN);
-  float* gloss = acc + BLK_G;
-
-  const int ntiles = (P + 15) / 16;
-  for (int tile = blockIdx.x * WARPS + warp; tile < ntiles; tile += gridDim.x * WARPS) {
-    const int p0 = tile * 16;
-    // standardised inputs, BF16, features 10..15 zero
-    for (int e = lane; e < 256; e += 32) {
-      const int pt = e & 15, f = e >> 4;
-      float v = 0.f;
-      if (f < NIN && p0 + pt < P) v = (X[(size_t)f * P + p0 + pt] - prm[O_INSH + f]) * prm[O_INSC + f];
-      A0[pt * 16 + f] = __float2bfloat16(v);
-    }
-    __syncwarp();
-    FragA fa;
-    FragB fb;
-    FragC fc;
-    // layer 1: Z1 = A0 W1p (16 x 64)
-    wmma::load_matrix_sync(fa, A0, 16);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      wmma::fill_fragment(fc, 0.f);
-      wmma::load_matrix_sync(fb, W1p + nt * 16, 64);
-      wmma::mma_sync(fc, fa, fb, fc);
-      wmma::store_matrix_sync(Z1 + nt * 16, fc, 64, wmma::mem_row_major);
-    }
-    __syncwarp();
-    for (int e = lane; e < 1024; e += 32) {
-      const float z = Z1[e] + prm[O_B1 + (e & 63)];
-      if (TRAIN) Z1[e] = z;  // the backward pass reads the pre-activation
-      H1[e] = __float2bfloat16(silu(z));
-    }
-    __syncwarp();
-    // layer 2: Z2 = H1 W2 (16 x 64)
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      wmma::fill_fragment(fc, 0.f);
-#pragma unroll
-      for (int kt = 0; kt < 4; ++kt) {
-        wmma::load_matrix_sync(fa, H1 + kt * 16, 64);
-        wmma::load_matrix_sync(fb, W2s + kt * 16 * 64 + nt * 16, 64);
-        wmma::mma_sync(fc, fa, fb, fc);
-      }
-      wmma::store_matrix_sync(Z2 + nt * 16, fc, 64, wmma::mem_row_major);
-    }
-    __syncwarp();
-    for (int e = lane; e < 1024; e += 32) {
-      const float z = Z2[e] + prm[O_B2 + (e & 63)];
-      if (TRAIN) Z2[e] = z;
-      H2[e] = __float2bfloat16(silu(z));
-    }
-    __syncwarp();
-    // layer 3: Y = H2 W3p (16 x 16, columns >= 6 zero)
-    wmma::fill_fragment(fc, 0.f);
-#pragma unroll
-    for (int kt = 0; kt < 4; ++kt) {
-      wmma::load_matrix_sync(fa, H2 + kt * 16, 64);
-      wmma::load_matrix_sync(fb, W3p + kt * 16 * 16, 16);
-      wmma::mma_sync(fc, fa, fb, fc);
-    }
-    wmma::store_matrix_sync(Yt, fc, 16, wmma::mem_row_major);
-    __syncwarp();
-    if (!TRAIN) {
-      for (int e = lane; e < 16 * NOUT; e += 32) {
-        const int pt = e & 15, c = e >> 4;
-        if (p0 + pt < P) {
-          const float y = Yt[pt * 16 + c] + prm[O_B3 + c];
-          Y[(size_t)c * P + p0 + pt] = y * prm[O_OUTSC + c] + prm[O_OUTSH + c];
-        }
-      }
-      continue;
-    }
-    // ---- training: dY = 2 (y - t_n) / (P * 6)
-    float lsum = 0.f;
-    const float inv = 2.f / ((float)P * (float)NOUT);
-    for (int e = lane; e < 256; e += 32) {
-      const int pt = e >> 4, c = e & 15;
-      float d = 0.f;
-      if (c < NOUT && p0 + pt < P) {
-        const float tn = (T[(size_t)c * P + p0 + pt] - prm[O_OUTSH + c]) / prm[O_OUTSC + c];
-        const float dd = Yt[e] + prm[O_B3 + c] - tn;
-        lsum += dd * dd;
-        d = inv * dd;
-      }
-      Yt[e] = d;  // FP32 dY
-      DY[e] = __float2bfloat16(d);
-    }
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) atomicAdd(gloss, lsum);
-    __syncwarp();
-    if (lane < NOUT) {
-      float s = 0.f;
-      for (int pt = 0; pt < 16; ++pt) s += Yt[pt * 16 + lane];
-      atomicAdd(&gb3[lane], s);
-    }
-    // dH2 = dY W3^T (W3p read as a column-major B); dZ2 = dH2 * silu'(Z2)
-    wmma::load_matrix_sync(fa, DY, 16);
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      FragBT fbt;
-      wmma::fill_fragment(fc, 0.f);
-      wmma::load_matrix_sync(fbt, W3p + nt * 16 * 16, 16);
-      wmma::mma_sync(fc, fa, fbt, fc);
-      wmma::store_matrix_sync(G + nt * 16, fc, 64, wmma::mem_row_major);
-    }
-    __syncwarp();
-    for (int e = lane; e < 1024; e += 32) {
-      const float g = G[e] * dsilu(Z2[e]);
-      G[e] = g;
-      DZ2[e] = __float2bfloat16(g);
-    }
-    __syncwarp();
-    for (int n = lane; n < 64; n += 32) {
-      float s = 0.f;
-      for (int pt = 0; pt < 16; ++pt) s += G[pt * 64 + n];
-      atomicAdd(&gb2[n], s);
-    }
-    // dH1 = dZ2 W2^T (into G, free again); dZ1 = dH1 * silu'(Z1)
-    __syncwarp();
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      wmma::fill_fragment(fc, 0.f);
-#pragma unroll
-      for (int kt = 0; kt < 4; ++kt) {
-        FragBT fbt;
-        wmma::load_matrix_sync(fa, DZ2 + kt * 16, 64);
-        wmma::load_matrix_sync(fbt, W2s + nt * 16 * 64 + kt * 16, 64);
-        wmma::mma_sync(fc, fa, fbt, fc);
-      }
-      wmma::store_matrix_sync(G + nt * 16, fc, 64, wmma::mem_row_major);
-    }
-    __syncwarp();
-    for (int e = lane; e < 1024; e += 32) {
-      const float g = G[e] * dsilu(Z1[e]);
-      G[e] = g;
-      DZ1[e] = __float2bfloat16(g);
-    }
-    __syncwarp();
-    for (int n = lane; n < 64; n += 32) {
-      float s = 0.f;
-      for (int pt = 0; pt < 16; ++pt) s += G[pt * 64 + n];
-      atomicAdd(&gb1[n], s);
-    }
-    // weight gradients (sums over the 16 points of the tile) on the tensor cores
-#pragma unroll
-    for (int mt = 0; mt < 4; ++mt) {  // gW3 += H2^T dY
-      FragAT fat;
-      wmma::fill_fragment(fc, 0.f);
-      wmma::load_matrix_sync(fat, H2 + mt * 16, 64);
-      wmma::load_matrix_sync(fb, DY, 16);
-      wmma::mma_sync(fc, fat, fb, fc);
-      wmma::store_matrix_sync(TT, fc, 16, wmma::mem_row_major);
-      __syncwarp();
-      add_tile(gW3, NOUT, mt * 16, 0, NH, NOUT, TT, lane);
-      __syncwarp();
-    }
-#pragma unroll
-    for (int mt = 0; mt < 4; ++mt) {  // gW2 += H1^T dZ2
-      FragAT fat;
-      wmma::load_matrix_sync(fat, H1 + mt * 16, 64);
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        wmma::fill_fragment(fc, 0.f);
-        wmma::load_matrix_sync(fb, DZ2 + nt * 16, 64);
-        wmma::mma_sync(fc, fat, fb, fc);
-        wmma::store_matrix_sync(TT, fc, 16, wmma::mem_row_major);
-        __syncwarp();
-        add_tile(gW2, NH, mt * 16, nt * 16, NH, NH, TT, lane);
-        __syncwarp();
-      }
-    }
-    {  // gW1 += A0^T dZ1 (feature rows >= 10 are padding)
-      FragAT fat;
-      wmma::load_matrix_sync(fat, A0, 16);
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        wmma::fill_fragment(fc, 0.f);
-        wmma::load_matrix_sync(fb, DZ1 + nt * 16, 64);
-        wmma::mma_sync(fc, fat, fb, fc);
-        wmma::store_matrix_sync(TT, fc, 16, wmma::mem_row_major);
-        __syncwarp();
-        add_tile(gW1, NH, 0, nt * 16, NIN, NH, TT, lane);
-        __syncwarp();
-      }
-    }
-  }
-  if (TRAIN) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < BLK_G; i += THREADS) atomicAdd(&gsum[TRAIN_BEGIN + i], acc[i]);
-    if (threadIdx.x == 0) atomicAdd(&gsum[NPARAM], gloss[0]);
-  }
+// Logistic functions of two values, 1 / (1 + exp(-z)), with one reciprocal for both: 1 / a = b / (a b).
+// The multi-function unit (two exponentials and one reciprocal, 16 lanes per SM and clock) is what
+// bounds the activations. -z is capped at 60 ln 2 so that the product stays finite; below it the
+// logistic is under 1e-18. Relative error about 1e-6, far below the BF16 rounding that follows.
+__device__ __forceinline__ void logistic2(float z0, float z1, float& s0, float& s1) {
+  float e0, e1, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fminf(z0 * -1.4426950408889634f, 60.f)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fminf(z1 * -1.4426950408889634f, 60.f)));
+  const float a = 1.f + e0, b = 1.f + e1;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a * b));
+  s0 = r * b;
+  s1 = r * a;
+}
+__device__ __forceinline__ unsigned bf2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const unsigned*>(&v);
 }
 
 // ---------------------------------------------------------------------------
@@ -336,26 +100,23 @@ __global__ void __launch_bounds__(THREADS) k_mlp(const float* __restrict__ prm, 
 //   layer 3: D3 (TMEM columns 0..15)   = H2 (128 x 64) . W3 (64 x 16, columns >= 6 zero)
 // ---------------------------------------------------------------------------
 constexpr int TC_M = 128, TC_THREADS = 128, TC_TMEM_COLS = 128;
-// shared memory: A operands X (4 KB), H1, H2 (16 KB each); B operands W1^T (64 x 16, 2 KB),
-// W2^T (64 x 64, 8 KB), W3^T (16 x 64, 2 KB); then the mbarrier and the TMEM address
-constexpr int TC_X = 0, TC_H1 = TC_X + 128 * 16 * 2, TC_H2 = TC_H1 + 128 * 64 * 2, TC_W1 = TC_H2 + 128 * 64 * 2,
-              TC_W2 = TC_W1 + 64 * 16 * 2, TC_W3 = TC_W2 + 64 * 64 * 2, TC_BAR = TC_W3 + 16 * 64 * 2,
-              TC_SMEM = TC_BAR + 16;
+// shared memory: A operands X (4 KB), H1, H2 (16 KB each); the image of the forward weights; then the
+// mbarrier
+constexpr int TC_X = 0, TC_H1 = TC_X + 128 * 16 * 2, TC_H2 = TC_H1 + 128 * 64 * 2, TC_W = TC_H2 + 128 * 64 * 2,
+              TC_BAR = TC_W + IMG_FWD, TC_SMEM = TC_BAR + 16;
 constexpr unsigned long long TC_WAIT_NS = 1000000000ull;  // 1 s bound on every mbarrier wait
 
-// byte offset of element (r, k) of a K-major operand with K columns in the core-matrix layout
-__device__ __forceinline__ int tc_off(int r, int k, int K) {
-  return ((r >> 3) * (K >> 3) + (k >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
 // shared-memory matrix descriptor: start address, leading (K) and stride (row-group)
 // byte offsets, the fixed version bits 46-47 = 1, no swizzle
 __device__ __forceinline__ unsigned long long tc_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
   return (unsigned long long)((saddr & 0x3FFFF) >> 4) | ((unsigned long long)(lbo >> 4) << 16) |
          ((unsigned long long)(sbo >> 4) << 32) | (1ull << 46);
 }
-// instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major, M x N
-__host__ __device__ constexpr unsigned tc_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
+// instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, M x N; both K-major, or both
+// MN-major (mn = 1: the contraction runs over the rows of the stored operands)
+__host__ __device__ constexpr unsigned tc_idesc(int M, int N, int mn = 0) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)mn << 15) | ((unsigned)mn << 16) | ((unsigned)(N >> 3) << 17) |
+         ((unsigned)(M >> 4) << 24);
 }
 __device__ __forceinline__ void tc_mma(unsigned dt, unsigned long long ad, unsigned long long bd, unsigned idesc,
                                        int acc) {
@@ -411,17 +172,22 @@ __device__ __forceinline__ void tc_hidden(unsigned trow, int c0, const float* __
   for (int q = 0; q < 4; ++q) {
     float v[16];
     tc_ld16(trow + c0 + 16 * q, v);
+    unsigned o[8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {  // two 8-element core-matrix rows of 16 bytes
-      __align__(16) bf o[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] = __float2bfloat16(silu(v[8 * h + i] + bias[16 * q + 8 * h + i]));
-      *reinterpret_cast<uint4*>(dst + tc_off(row, 16 * q + 8 * h, 64)) = *reinterpret_cast<const uint4*>(o);
+    for (int i = 0; i < 8; ++i) {
+      const float z0 = v[2 * i] + bias[16 * q + 2 * i], z1 = v[2 * i + 1] + bias[16 * q + 2 * i + 1];
+      float s0, s1;
+      logistic2(z0, z1, s0, s1);
+      o[i] = bf2(z0 * s0, z1 * s1);
     }
+    // two 8-element core-matrix rows of 16 bytes
+    *reinterpret_cast<uint4*>(dst + tc_off(row, 16 * q, 64)) = make_uint4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<uint4*>(dst + tc_off(row, 16 * q + 8, 64)) = make_uint4(o[4], o[5], o[6], o[7]);
   }
 }
 
-__global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__ prm, const bf* __restrict__ wpack,
+__global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__ prm,
+                                                       const unsigned char* __restrict__ img,
                                                        const float* __restrict__ X, int P, float* __restrict__ Y,
                                                        int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char tsm[];
@@ -430,19 +196,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
   const int t = threadIdx.x, warp = t >> 5;
   const unsigned sbase = (unsigned)__cvta_generic_to_shared(tsm);
   const unsigned bar = sbase + TC_BAR;
-  // B operands from the packed weights: W^T rows n, columns k
-  for (int i = t; i < 64 * 16; i += TC_THREADS) {  // W1^T (64 x 16): W1p[k][n]
-    const int n = i >> 4, k = i & 15;
-    *reinterpret_cast<bf*>(tsm + TC_W1 + tc_off(n, k, 16)) = wpack[PW1 + k * 64 + n];
-  }
-  for (int i = t; i < 64 * 64; i += TC_THREADS) {  // W2^T (64 x 64): W2[k][n]
-    const int n = i >> 6, k = i & 63;
-    *reinterpret_cast<bf*>(tsm + TC_W2 + tc_off(n, k, 64)) = wpack[PW2 + k * 64 + n];
-  }
-  for (int i = t; i < 16 * 64; i += TC_THREADS) {  // W3^T (16 x 64): W3p[k][n]
-    const int n = i >> 6, k = i & 63;
-    *reinterpret_cast<bf*>(tsm + TC_W3 + tc_off(n, k, 64)) = wpack[PW3 + k * 16 + n];
-  }
+  for (int i = t; i < IMG_FWD / 16; i += TC_THREADS)
+    reinterpret_cast<uint4*>(tsm + TC_W)[i] = reinterpret_cast<const uint4*>(img)[i];
   for (int i = t; i < 2 * NH + 16; i += TC_THREADS)
     s_b[i] = i < NH ? prm[O_B1 + i] : (i < 2 * NH ? prm[O_B2 + i - NH] : (i - 2 * NH < NOUT ? prm[O_B3 + i - 2 * NH] : 0.f));
   if (t == 0) {
@@ -462,9 +217,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
   tc_fence_after();
   const unsigned tmem = s_taddr;
   const unsigned trow = tmem + ((unsigned)(32 * warp) << 16);  // this warp's 32 lanes
-  const unsigned long long dW1 = tc_desc(sbase + TC_W1, 128, 2 * 128);
-  const unsigned long long dW2 = tc_desc(sbase + TC_W2, 128, 8 * 128);
-  const unsigned long long dW3 = tc_desc(sbase + TC_W3, 128, 8 * 128);
+  const unsigned long long dW1 = tc_desc(sbase + TC_W + IMG_W1, 128, 2 * 128);
+  const unsigned long long dW2 = tc_desc(sbase + TC_W + IMG_W2, 128, 8 * 128);
+  const unsigned long long dW3 = tc_desc(sbase + TC_W + IMG_W3, 128, 8 * 128);
   const unsigned long long dX = tc_desc(sbase + TC_X, 128, 2 * 128);
   const unsigned long long dH1 = tc_desc(sbase + TC_H1, 128, 8 * 128);
   const unsigned long long dH2 = tc_desc(sbase + TC_H2, 128, 8 * 128);
@@ -544,17 +299,324 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
 }
 
-// Adam on the trainable range; moments m, v; step t >= 1; clears the gradient sums.
-__global__ void k_adam(float* __restrict__ prm, float* __restrict__ gsum, float* __restrict__ m,
-                       float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (int i = TRAIN_BEGIN + threadIdx.x + blockIdx.x * blockDim.x; i < TRAIN_END; i += blockDim.x * gridDim.x) {
-    const float g = gsum[i];
+// ---------------------------------------------------------------------------
+// Training pass: loss and gradient sums of the block's tiles of 128 points, all products on the tensor
+// cores. 8 warps: warp w reads the TMEM lanes (points) of quarter w & 3 and the columns of half
+// w >> 2. Per tile the scratch columns T take D1, D2, Y, dH2 and dH1 in turn; the slopes of the
+// activations stay in registers, so an activation costs one logistic for both directions. The
+// weight gradients contract over the points, i.e. over the rows of the operands that the other
+// products already have in shared memory, read as MN-major operands:
+//   columns 64 .. 143  (128 x 80) = [H1 | H2]^T [dZ2 | dY]: gW2 in rows < 64, gW3 in the last 16 columns
+//   columns 144 .. 159 (128 x 16) = [dZ1 | dZ2]^T X:        gW1^T in rows < 64
+// (the other blocks of these products are not read). They accumulate in TMEM over the block's tiles.
+// Bias gradients are FP32 sums of the unrounded dZ. Each block leaves its sums in its row of
+// `part`; k_reduce adds the rows in order, so the gradient is the same from run to run.
+// Bound by latency (five dependent products a tile) and instruction issue; 65536 points, one call
+// with its read-back 247 -> 54 us against warp-level products on 16-point tiles with shared-memory
+// atomics; a training step (k_mlp_train and k_reduce) 226 -> 30 us, 262144 points 820 -> 63 us.
+// ---------------------------------------------------------------------------
+constexpr int TR_THREADS = 256, TR_TMEM_COLS = 256, TR_T = 0, TR_GW = 64, TR_G1 = 144;
+constexpr int TR_EG = 18;  // groups of 8 columns of the array dZ1 (64) | dZ2 (64) | dY (16)
+constexpr int TR_X = 0, TR_H = TR_X + 128 * 16 * 2, TR_E = TR_H + 128 * 128 * 2, TR_W = TR_E + 128 * TR_EG * 16,
+              TR_BAR = TR_W + IMG_BYTES, TR_SMEM = TR_BAR + 16;
+constexpr int PART = 5264;  // floats of a row of partial sums: NTRAIN gradients, the loss, padding
+
+// sums over the warp's 32 lanes of v[i], i < 32: lane l returns the sum of v[l]
+__device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float mine = up ? v[i + o] : v[i], theirs = up ? v[i] : v[i + o];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+    }
+  }
+  return v[0];
+}
+
+__global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __restrict__ prm,
+                                                             const unsigned char* __restrict__ img,
+                                                             const float* __restrict__ X, const float* __restrict__ T,
+                                                             int P, float* __restrict__ part, int* __restrict__ err) {
+  extern __shared__ __align__(1024) unsigned char tsm[];
+  __shared__ unsigned s_taddr;
+  __shared__ float s_b[2 * NH + 16];           // b1, b2, b3
+  __shared__ float s_io[4][16];                // in_shift, in_scale, 1 / out_scale, out_shift
+  __shared__ float s_sum[4][2 * NH + 16];      // per quarter: gb1, gb2, gb3 and the loss
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, q = warp & 3, hf = warp >> 2, row = 32 * q + lane;
+  const unsigned sbase = (unsigned)__cvta_generic_to_shared(tsm);
+  const unsigned bar = sbase + TR_BAR;
+  for (int i = t; i < IMG_BYTES / 16; i += TR_THREADS)
+    reinterpret_cast<uint4*>(tsm + TR_W)[i] = reinterpret_cast<const uint4*>(img)[i];
+  if (t < 2 * NH + 16)
+    s_b[t] = t < NH ? prm[O_B1 + t] : (t < 2 * NH ? prm[O_B2 + t - NH] : (t - 2 * NH < NOUT ? prm[O_B3 + t - 2 * NH] : 0.f));
+  if (t < 16) {
+    s_io[0][t] = t < NIN ? prm[O_INSH + t] : 0.f;
+    s_io[1][t] = t < NIN ? prm[O_INSC + t] : 0.f;
+    s_io[2][t] = t < NOUT ? prm[O_OUTSC + t] : 1.f;
+    s_io[3][t] = t < NOUT ? prm[O_OUTSH + t] : 0.f;
+  }
+  if (t == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(&s_taddr)),
+                 "r"(TR_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  proxy_fence();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = s_taddr, trow = tmem + ((unsigned)(32 * q) << 16);
+  // A and B operands of the products over columns (K-major; rows of 8 points HS or ES bytes apart) ...
+  constexpr unsigned HS = 16 * 128, ES = TR_EG * 128;
+  const unsigned long long dX = tc_desc(sbase + TR_X, 128, 256), dW1 = tc_desc(sbase + TR_W + IMG_W1, 128, 256);
+  const unsigned long long dH1 = tc_desc(sbase + TR_H, 128, HS), dH2 = tc_desc(sbase + TR_H + 8 * 128, 128, HS);
+  const unsigned long long dW2 = tc_desc(sbase + TR_W + IMG_W2, 128, 1024), dW3 = tc_desc(sbase + TR_W + IMG_W3, 128, 1024);
+  const unsigned long long dDY = tc_desc(sbase + TR_E + 16 * 128, 128, ES), dDZ2 = tc_desc(sbase + TR_E + 8 * 128, 128, ES);
+  const unsigned long long dW2B = tc_desc(sbase + TR_W + IMG_W2B, 128, 1024), dW3B = tc_desc(sbase + TR_W + IMG_W3B, 128, 256);
+  // ... and over points (MN-major: 8 columns 128 bytes apart, 8 points HS, ES or 256 bytes apart)
+  const unsigned long long tH = tc_desc(sbase + TR_H, HS, 128), tE = tc_desc(sbase + TR_E, ES, 128),
+                           tE2 = tc_desc(sbase + TR_E + 8 * 128, ES, 128), tX = tc_desc(sbase + TR_X, 256, 128);
+  constexpr unsigned ID64 = tc_idesc(128, 64), ID16 = tc_idesc(128, 16), IDGW = tc_idesc(128, 80, 1), IDG1 = tc_idesc(128, 16, 1);
+  constexpr unsigned long long KSTEP = 256 >> 4;  // descriptor step of 16 columns
+  unsigned phase = 0;
+  bool ok = true;
+  float loss = 0.f, gb1 = 0.f, gb2 = 0.f, gb3[NOUT] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  const float inv = 2.f / ((float)P * (float)NOUT);
+  const int ntiles = (P + 127) / 128;
+  int done = 0;  // tiles of this block whose weight gradients are under way
+  auto publish = [&] {  // shared-memory operands written: visible to the tensor core
+    proxy_fence();
+    tc_fence_before();
+    __syncthreads();
+  };
+  auto wait = [&] {
+    ok = tc_wait(bar, phase) && ok;
+    phase ^= 1;
+    tc_fence_after();
+  };
+  // z = accumulator + bias of this thread's 32 units, h = SiLU(z) as BF16 into the columns c0 .. of H, slope into ds
+  auto hidden = [&](const float* bias, int c0, float (&ds)[32]) {
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      float v[16];
+      tc_ld16(trow + TR_T + 32 * hf + 16 * g, v);
+      unsigned o[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float z0 = v[2 * i] + bias[16 * g + 2 * i], z1 = v[2 * i + 1] + bias[16 * g + 2 * i + 1];
+        float s0, s1;
+        logistic2(z0, z1, s0, s1);
+        o[i] = bf2(z0 * s0, z1 * s1);
+        ds[16 * g + 2 * i] = s0 * (1.f + z0 * (1.f - s0));
+        ds[16 * g + 2 * i + 1] = s1 * (1.f + z1 * (1.f - s1));
+      }
+      *reinterpret_cast<uint4*>(tsm + TR_H + tc_off(row, c0 + 16 * g, 128)) = make_uint4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<uint4*>(tsm + TR_H + tc_off(row, c0 + 16 * g + 8, 128)) = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+  };
+  // dZ = accumulator * slope (into ds), as BF16 into the columns c0 .. of E; returns the bias gradient of unit `lane`
+  auto slope = [&](int c0, float (&ds)[32]) {
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      float v[16];
+      tc_ld16(trow + TR_T + 32 * hf + 16 * g, v);
+      unsigned o[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        ds[16 * g + 2 * i] *= v[2 * i];
+        ds[16 * g + 2 * i + 1] *= v[2 * i + 1];
+        o[i] = bf2(ds[16 * g + 2 * i], ds[16 * g + 2 * i + 1]);
+      }
+      *reinterpret_cast<uint4*>(tsm + TR_E + tc_off(row, c0 + 16 * g, 8 * TR_EG)) = make_uint4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<uint4*>(tsm + TR_E + tc_off(row, c0 + 16 * g + 8, 8 * TR_EG)) = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+  };
+  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const int p = tile * 128 + row;
+    float x[8], tn[NOUT];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int f = 8 * hf + i;
+      x[i] = (f < NIN && p < P) ? (X[(size_t)f * P + p] - s_io[0][f]) * s_io[1][f] : 0.f;
+    }
+    if (hf == 0)
+#pragma unroll
+      for (int c = 0; c < NOUT; ++c) tn[c] = p < P ? (T[(size_t)c * P + p] - s_io[3][c]) / s_io[2][c] : 0.f;
+    if (done > 0) wait();  // the operands of the tile before are free
+    *reinterpret_cast<uint4*>(tsm + TR_X + tc_off(row, 8 * hf, 16)) =
+        make_uint4(bf2(x[0], x[1]), bf2(x[2], x[3]), bf2(x[4], x[5]), bf2(x[6], x[7]));
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+      tc_mma(tmem + TR_T, dX, dW1, ID64, 0);
+      tc_commit(bar);
+    }
+    wait();
+    float ds1[32], ds2[32];
+    hidden(s_b + 32 * hf, 32 * hf, ds1);
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc_mma(tmem + TR_T, dH1 + k * KSTEP, dW2 + k * KSTEP, ID64, k);
+      tc_commit(bar);
+    }
+    wait();
+    hidden(s_b + NH + 32 * hf, NH + 32 * hf, ds2);
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc_mma(tmem + TR_T, dH2 + k * KSTEP, dW3 + k * KSTEP, ID16, k);
+      tc_commit(bar);
+    }
+    wait();
+    if (hf == 0) {  // dY = 2 (y - t) / (6 P)
+      float v[16], d[8];
+      tc_ld16(trow + TR_T, v);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        d[c] = 0.f;
+        if (c < NOUT && p < P) {
+          const float e = v[c] + s_b[2 * NH + c] - tn[c < NOUT ? c : 0];
+          loss += e * e;
+          d[c] = inv * e;
+          gb3[c < NOUT ? c : 0] += d[c];
+        }
+      }
+      *reinterpret_cast<uint4*>(tsm + TR_E + tc_off(row, 128, 8 * TR_EG)) =
+          make_uint4(bf2(d[0], d[1]), bf2(d[2], d[3]), bf2(d[4], d[5]), bf2(d[6], d[7]));
+      *reinterpret_cast<uint4*>(tsm + TR_E + tc_off(row, 136, 8 * TR_EG)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+      tc_mma(tmem + TR_T, dDY, dW3B, ID64, 0);
+      tc_commit(bar);
+    }
+    wait();
+    slope(NH + 32 * hf, ds2);
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) tc_mma(tmem + TR_T, dDZ2 + k * KSTEP, dW2B + k * KSTEP, ID64, k);
+      tc_commit(bar);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)  // 16 points a step
+        tc_mma(tmem + TR_GW, tH + k * (2 * HS >> 4), tE2 + k * (2 * ES >> 4), IDGW, done > 0 || k > 0);
+    }
+    gb2 += warp_column_sums(ds2, lane);
+    wait();
+    slope(32 * hf, ds1);
+    publish();
+    if (t == 0) {
+      tc_fence_after();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) tc_mma(tmem + TR_G1, tE + k * (2 * ES >> 4), tX + k * (512 >> 4), IDG1, done > 0 || k > 0);
+      tc_commit(bar);
+    }
+    gb1 += warp_column_sums(ds1, lane);
+    ++done;
+    ok = __syncthreads_and(ok);  // the block leaves the loop together
+  }
+  if (done > 0) wait();
+  // the block's sums: weights from TMEM, biases and loss through shared memory
+  s_sum[q][32 * hf + lane] = gb1;
+  s_sum[q][NH + 32 * hf + lane] = gb2;
+  if (hf == 0) {
+    for (int o = 16; o > 0; o >>= 1) {
+      loss += __shfl_xor_sync(0xffffffffu, loss, o);
+#pragma unroll
+      for (int c = 0; c < NOUT; ++c) gb3[c] += __shfl_xor_sync(0xffffffffu, gb3[c], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int c = 0; c < NOUT; ++c) s_sum[q][2 * NH + c] = gb3[c];
+      s_sum[q][2 * NH + NOUT] = loss;
+    }
+  }
+  float* out = part + (size_t)blockIdx.x * PART;
+  if (q < 2) {  // rows < 64 of both products
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      float v[16];
+      tc_ld16(trow + TR_GW + 32 * hf + 16 * g, v);
+      float4* d = reinterpret_cast<float4*>(out + (O_W2 - TRAIN_BEGIN) + row * NH + 32 * hf + 16 * g);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+    if (hf == 0) {
+      float v[16];
+      tc_ld16(trow + TR_G1, v);
+#pragma unroll
+      for (int f = 0; f < NIN; ++f) out[(O_W1 - TRAIN_BEGIN) + f * NH + row] = v[f];
+    }
+  } else if (hf == 0) {
+    float v[16];
+    tc_ld16(trow + TR_GW + NH, v);
+#pragma unroll
+    for (int c = 0; c < NOUT; ++c) out[(O_W3 - TRAIN_BEGIN) + (row - 64) * NOUT + c] = v[c];
+  }
+  if (!ok && t == 0) atomicExch(err, 1);
+  tc_fence_before();
+  __syncthreads();
+  if (t < 2 * NH + NOUT + 1) {
+    const float s = s_sum[0][t] + s_sum[1][t] + s_sum[2][t] + s_sum[3][t];
+    const int at = t < NH ? O_B1 + t : (t < 2 * NH ? O_B2 + t - NH : O_B3 + t - 2 * NH);  // the loss follows b3
+    out[at - TRAIN_BEGIN] = s;
+  }
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TR_TMEM_COLS) : "memory");
+}
+
+// The blocks' rows of partial sums added in order: gradients and loss into gsum (and, for the host, the
+// error flag behind them); ADAM: one Adam step on the trainable range (moments m, v; bias
+// corrections c1, c2) and the changed weights into the image.
+// 32 columns a block, 8 threads each on every eighth row.
+constexpr int RED_COLS = 32, RED_ROWS = 8;
+template <bool ADAM>
+__global__ void __launch_bounds__(RED_COLS * RED_ROWS) k_reduce(const float* __restrict__ part, int rows,
+                                                                float* __restrict__ gsum, float* __restrict__ prm,
+                                                                float* __restrict__ m, float* __restrict__ v,
+                                                                unsigned char* __restrict__ img, const int* __restrict__ err,
+                                                                float lr, float b1, float b2, float eps, float c1, float c2) {
+  __shared__ float red[RED_ROWS][RED_COLS];
+  const int x = threadIdx.x % RED_COLS, y = threadIdx.x / RED_COLS, j = blockIdx.x * RED_COLS + x;
+  float s = 0.f;
+  if (j <= NTRAIN) {
+#pragma unroll 8
+    for (int r = y; r < rows; r += RED_ROWS) s += part[(size_t)r * PART + j];
+  }
+  red[y][x] = s;
+  __syncthreads();
+  if (y != 0 || j > NTRAIN) return;
+  float g = 0.f;
+#pragma unroll
+  for (int r = 0; r < RED_ROWS; ++r) g += red[r][x];
+  if (j == NTRAIN) {
+    gsum[NPARAM] = g;
+    gsum[NPARAM + 1] = (float)*err;
+    return;
+  }
+  const int i = TRAIN_BEGIN + j;
+  if constexpr (ADAM) {
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
     v[i] = vi;
-    prm[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    gsum[i] = 0.f;
+    const float w = prm[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    prm[i] = w;
+    pack_param(i, w, img);
+  } else {
+    gsum[i] = g;
   }
 }
 
@@ -562,11 +624,13 @@ __global__ void k_adam(float* __restrict__ prm, float* __restrict__ gsum, float*
 
 struct dns_mlp {
   float* prm = nullptr;   // NPARAM (device)
-  float* gsum = nullptr;  // NPARAM + 1 (device): gradient sums and the loss sum
+  float* gsum = nullptr;  // NPARAM + 2 (device): gradient sums, the loss sum, the error flag; zeros where nothing is trained
+  float* host = nullptr;  // NPARAM + 2 (pinned): where a call reads them back
+  float* part = nullptr;  // partial sums of the training blocks (device)
   float* m = nullptr;
   float* v = nullptr;
-  bf* pack = nullptr;  // NPACK (device)
-  int* err = nullptr;  // device flag: a tensor-core wait of the inference kernel gave up
+  unsigned char* img = nullptr;  // the BF16 weights as the kernels' operands (device)
+  int* err = nullptr;  // device flag: a tensor-core wait gave up
   int t = 0;           // Adam steps taken
 };
 
@@ -583,29 +647,34 @@ int mlp_fail(int code, const char* msg) {
     if (e_ != cudaSuccess) return mlp_fail(DNS_ERR_CUDA, where); \
   } while (0)
 
-// inference grid: four blocks per SM (4 x 128 TMEM columns fill an SM's 512), each block
-// walking several 128-point tiles
-int mlp_blocks_tc(int P) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 148;
-  }
-  const int tiles = (P + TC_M - 1) / TC_M;
-  return tiles < 4 * sms ? (tiles < 1 ? 1 : tiles) : 4 * sms;
+int mlp_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 148;
+    return n;
+  }();
+  return sms;
 }
 
-int mlp_blocks(int P) {
-  int tiles = (P + 15) / 16;
-  int b = (tiles + WARPS - 1) / WARPS;
-  return b > 2048 ? 2048 : (b < 1 ? 1 : b);
+// grid of a kernel with `per_sm` blocks on an SM, each walking tiles of 128 points: four inference blocks
+// (4 x 128 TMEM columns fill an SM's 512), two training blocks (2 x 256)
+constexpr int TC_PER_SM = 4, TR_PER_SM = 2;
+int mlp_blocks(int P, int per_sm) {
+  const int tiles = (P + TC_M - 1) / TC_M;
+  return tiles < per_sm * mlp_sms() ? (tiles < 1 ? 1 : tiles) : per_sm * mlp_sms();
 }
 
 int mlp_run_grad(dns_mlp* net, const float* X, const float* T, int P, cudaStream_t st) {
-  MLP_CUDA(cudaMemsetAsync(net->gsum, 0, (NPARAM + 1) * sizeof(float), st), "dns_mlp: clear gradients");
-  k_mlp<1><<<mlp_blocks(P), THREADS, SMEM_B, st>>>(net->prm, net->pack, X, P, nullptr, T, net->gsum);
+  k_mlp_train<<<mlp_blocks(P, TR_PER_SM), TR_THREADS, TR_SMEM, st>>>(net->prm, net->img, X, T, P, net->part, net->err);
   MLP_CUDA(cudaGetLastError(), "dns_mlp: training kernel launch");
+  return DNS_OK;
+}
+template <bool ADAM>
+int mlp_reduce(dns_mlp* n, int P, float lr, float b1, float b2, float c1, float c2, cudaStream_t st) {
+  k_reduce<ADAM><<<(NTRAIN + RED_COLS) / RED_COLS, RED_COLS * RED_ROWS, 0, st>>>(
+      n->part, mlp_blocks(P, TR_PER_SM), n->gsum, n->prm, n->m, n->v, n->img, n->err, lr, b1, b2, 1e-8f, c1, c2);
+  MLP_CUDA(cudaGetLastError(), "dns_mlp: reduction launch");
   return DNS_OK;
 }
 
@@ -653,20 +722,20 @@ __global__ void __launch_bounds__(NORM_THREADS) k_norm(float* __restrict__ prm, 
   }
 }
 
-// Reports (and clears) a tensor-core wait of the inference kernel that gave up; synchronises.
+// Reports (and clears) a tensor-core wait that gave up; synchronises.
 int mlp_check_err(dns_mlp* n, const char* where) {
   int err = 0;
   MLP_CUDA(cudaMemcpy(&err, n->err, sizeof(int), cudaMemcpyDeviceToHost), where);
   if (!err) return DNS_OK;
   MLP_CUDA(cudaMemset(n->err, 0, sizeof(int)), where);
-  return mlp_fail(DNS_ERR_TIMEOUT, "dns_mlp: an inference kernel's tensor-core wait gave up after 1 s; its output is not valid");
+  return mlp_fail(DNS_ERR_TIMEOUT, "dns_mlp: a kernel's tensor-core wait gave up after 1 s; its output is not valid");
 }
 
 }  // namespace
 
 namespace dns {
 cudaError_t mlp_forward_async(::dns_mlp* n, const float* X, float* Y, int P, cudaStream_t st) {
-  k_mlp_tc<<<mlp_blocks_tc(P), TC_THREADS, TC_SMEM, st>>>(n->prm, n->pack, X, P, Y, n->err);
+  k_mlp_tc<<<mlp_blocks(P, TC_PER_SM), TC_THREADS, TC_SMEM, st>>>(n->prm, n->img, X, P, Y, n->err);
   return cudaGetLastError();
 }
 }  // namespace dns
@@ -687,18 +756,21 @@ int dns_mlp_create(dns_mlp** out) {
   *out = nullptr;
   dns_mlp* n = new dns_mlp();
   cudaError_t e = cudaMalloc(&n->prm, NPARAM * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&n->gsum, (NPARAM + 1) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&n->gsum, (NPARAM + 2) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMallocHost(&n->host, (NPARAM + 2) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&n->part, (size_t)TR_PER_SM * mlp_sms() * PART * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->m, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->v, NPARAM * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&n->pack, NPACK * sizeof(bf));
+  if (e == cudaSuccess) e = cudaMalloc(&n->img, IMG_BYTES);
+  if (e == cudaSuccess) e = cudaMemset(n->img, 0, IMG_BYTES);
   if (e == cudaSuccess) e = cudaMalloc(&n->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->prm, 0, NPARAM * sizeof(float));
-  if (e == cudaSuccess) e = cudaMemset(n->gsum, 0, (NPARAM + 1) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMemset(n->gsum, 0, (NPARAM + 2) * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(n->v, 0, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_B);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM);
   if (e != cudaSuccess) {
     dns_mlp_destroy(n);
     cudaGetLastError();
@@ -714,7 +786,9 @@ int dns_mlp_destroy(dns_mlp* n) {
   cudaFree(n->gsum);
   cudaFree(n->m);
   cudaFree(n->v);
-  cudaFree(n->pack);
+  cudaFree(n->img);
+  cudaFree(n->part);
+  if (n->host) cudaFreeHost(n->host);
   cudaFree(n->err);
   delete n;
   return DNS_OK;
@@ -726,7 +800,7 @@ int dns_mlp_set_params(dns_mlp* n, const float* host, int count) {
   MLP_CUDA(cudaMemset(n->m, 0, NPARAM * sizeof(float)), "dns_mlp_set_params");
   MLP_CUDA(cudaMemset(n->v, 0, NPARAM * sizeof(float)), "dns_mlp_set_params");
   n->t = 0;
-  k_pack<<<16, 256>>>(n->prm, n->pack);
+  k_pack<<<16, 256>>>(n->prm, n->img);
   MLP_CUDA(cudaGetLastError(), "dns_mlp_set_params pack");
   MLP_CUDA(cudaDeviceSynchronize(), "dns_mlp_set_params");
   return DNS_OK;
@@ -741,7 +815,7 @@ int dns_mlp_get_params(dns_mlp* n, float* host, int count) {
 
 int dns_mlp_forward(dns_mlp* n, const float* X, float* Y, int P, void* stream) {
   if (!n || !X || !Y || P < 1) return mlp_fail(DNS_ERR_ARG, "dns_mlp_forward: bad arguments");
-  k_mlp_tc<<<mlp_blocks_tc(P), TC_THREADS, TC_SMEM, (cudaStream_t)stream>>>(n->prm, n->pack, X, P, Y, n->err);
+  k_mlp_tc<<<mlp_blocks(P, TC_PER_SM), TC_THREADS, TC_SMEM, (cudaStream_t)stream>>>(n->prm, n->img, X, P, Y, n->err);
   MLP_CUDA(cudaGetLastError(), "dns_mlp_forward launch");
   return DNS_OK;
 }
@@ -752,13 +826,13 @@ int dns_mlp_loss_grad(dns_mlp* n, const float* X, const float* T, int P, float* 
   cudaStream_t st = (cudaStream_t)stream;
   int rc = mlp_run_grad(n, X, T, P, st);
   if (rc) return rc;
-  std::vector<float> g(NPARAM + 1);
-  MLP_CUDA(cudaMemcpyAsync(g.data(), n->gsum, (NPARAM + 1) * sizeof(float), cudaMemcpyDeviceToHost, st),
+  if ((rc = mlp_reduce<false>(n, P, 0.f, 0.f, 0.f, 1.f, 1.f, st))) return rc;
+  MLP_CUDA(cudaMemcpyAsync(n->host, n->gsum, (NPARAM + 2) * sizeof(float), cudaMemcpyDeviceToHost, st),
            "dns_mlp_loss_grad copy");
   MLP_CUDA(cudaStreamSynchronize(st), "dns_mlp_loss_grad");
-  if (grad_host) memcpy(grad_host, g.data(), NPARAM * sizeof(float));
-  if (loss_host) *loss_host = g[NPARAM] / ((float)P * (float)NOUT);
-  MLP_CUDA(cudaMemsetAsync(n->gsum, 0, (NPARAM + 1) * sizeof(float), st), "dns_mlp_loss_grad clear");
+  if (n->host[NPARAM + 1] != 0.f) return mlp_check_err(n, "dns_mlp_loss_grad");
+  if (grad_host) memcpy(grad_host, n->host, NPARAM * sizeof(float));
+  if (loss_host) *loss_host = n->host[NPARAM] / ((float)P * (float)NOUT);
   return DNS_OK;
 }
 
@@ -767,18 +841,16 @@ int dns_mlp_train_step(dns_mlp* n, const float* X, const float* T, int P, double
   cudaStream_t st = (cudaStream_t)stream;
   int rc = mlp_run_grad(n, X, T, P, st);
   if (rc) return rc;
-  float lsum = 0.f;
-  if (loss_host) MLP_CUDA(cudaMemcpyAsync(&lsum, n->gsum + NPARAM, sizeof(float), cudaMemcpyDeviceToHost, st),
-                          "dns_mlp_train_step loss copy");
   n->t += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)n->t), c2 = 1.f - std::pow(b2, (float)n->t);
-  k_adam<<<8, 256, 0, st>>>(n->prm, n->gsum, n->m, n->v, (float)lr, b1, b2, 1e-8f, c1, c2);
-  k_pack<<<16, 256, 0, st>>>(n->prm, n->pack);
-  MLP_CUDA(cudaGetLastError(), "dns_mlp_train_step update");
+  if ((rc = mlp_reduce<true>(n, P, (float)lr, b1, b2, c1, c2, st))) return rc;
   if (loss_host) {
+    MLP_CUDA(cudaMemcpyAsync(n->host + NPARAM, n->gsum + NPARAM, 2 * sizeof(float), cudaMemcpyDeviceToHost, st),
+             "dns_mlp_train_step loss copy");
     MLP_CUDA(cudaStreamSynchronize(st), "dns_mlp_train_step");
-    *loss_host = lsum / ((float)P * (float)NOUT);
+    if (n->host[NPARAM + 1] != 0.f) return mlp_check_err(n, "dns_mlp_train_step");
+    *loss_host = n->host[NPARAM] / ((float)P * (float)NOUT);
   }
   return DNS_OK;
 }
