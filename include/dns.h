@@ -376,6 +376,13 @@ int dns_ensemble_time_steps(dns_ensemble* e, int n, double* ms);
  *   synchronously; device input is read on the handle's stream. */
 int dns_transform_r2c(dns_handle* h, const void* phys3, void* spec3);
 int dns_transform_c2r(dns_handle* h, const void* spec3, void* phys3);
+/* The box-filtered velocity and products of the handle's state on an Nc^3 grid (Nc even, Nc <= N;
+ * cubic grids), as the closure's training data needs them: ubar3 (3,Nc,Nc,Nc/2+1) =
+ * dns_spectral_filter of the state, pbar6 (6,Nc,Nc,Nc/2+1) = dns_spectral_filter of F(u_i u_j) in the
+ * order of dns_pointwise_products. The same values as those separate calls give, without the physical
+ * fields and the modes that the filter drops. Device arrays, 16-byte aligned; the state is left alone;
+ * asynchronous on the handle's stream. Errors: DNS_ERR_ARG, DNS_ERR_UNSUPPORTED (not cubic). */
+int dns_filtered_products(dns_handle* h, int Nc, void* ubar3, void* pbar6);
 int dns_set_forcing(dns_handle* h, const void* f3, int on_device);
 
 /* ---- Learned subgrid-stress closure: spectral helpers ------------------------

@@ -78,6 +78,7 @@ SIGNATURES = {
     "dns_transform_r2c": (_I, [_P, _P, _P]),
     "dns_transform_c2r": (_I, [_P, _P, _P]),
     "dns_set_forcing": (_I, [_P, _P, _I]),
+    "dns_filtered_products": (_I, [_P, _I, _P, _P]),
     "dns_spectral_filter": (_I, [_P, _I, _P, _I, _I, _P]),
     "dns_spectral_gradient": (_I, [_P, _I, _P, _I, _P]),
     "dns_stress_force": (_I, [_P, _I, _P, _I, _P]),

@@ -1150,8 +1150,24 @@ int dns_transform_c2r(dns_handle* h, const void* spec3, void* phys3) {
   PassArgs a = base_args(h);
   a.U = h->US;
   a.out = phys3;
+  a.prune = PRUNE_NONE;  // the caller's fields, not the state
   DNS_CUDA(h->ops->inverse3d(a, h->stream), "dns_transform_c2r");
   h->w_valid = false;
+  return DNS_OK;
+}
+
+int dns_filtered_products(dns_handle* h, int Nc, void* ubar3, void* pbar6) {
+  int rc = check_handle(h);
+  if (rc) return rc;
+  if (h->Ny != h->N || h->Nz != h->N) return fail(DNS_ERR_UNSUPPORTED, "dns_filtered_products: cubic grids only");
+  if (Nc < 2 || Nc % 2 || Nc > h->N) return fail(DNS_ERR_ARG, "dns_filtered_products: Nc must be even, 2 .. N");
+  if (!ubar3 || !pbar6 || (uintptr_t)ubar3 % 16 || (uintptr_t)pbar6 % 16)
+    return fail(DNS_ERR_ARG, "dns_filtered_products: device pointers must be non-NULL and 16-byte aligned");
+  if ((rc = use_device(h))) return rc;
+  h->w_valid = false;
+  DNS_CUDA(filter_internal(h->U, h->N, ubar3, Nc, 3, h->dtype, h->stream), "dns_filtered_products filter");
+  DNS_CUDA(h->ops->products_low(base_args(h), Nc / 2, h->stream), "dns_filtered_products transforms");
+  DNS_CUDA(filter_internal(h->W, h->N, pbar6, Nc, 6, h->dtype, h->stream), "dns_filtered_products filter");
   return DNS_OK;
 }
 

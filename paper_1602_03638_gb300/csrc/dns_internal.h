@@ -54,6 +54,7 @@ struct PassArgs {
   // box as zeros, the z-pass reads only kz < kc. The results are those of the full
   // transforms (the skipped terms are zeros).
   int prune = 0;
+  int kz_keep = 0;  // planes of the products that products_low stores
   const void* in = nullptr;  // physical input (3,Nx,Ny,Nz) for set_state
   void* out = nullptr;       // physical output (3,Nx,Ny,Nz) / RHS output
   double* partials = nullptr;          // diagnostics block partials
@@ -95,6 +96,8 @@ struct DnsOps {
   int TW;      // length of the twiddle table exp(-2 pi i t / TW) (a multiple of N, NY, NZ)
   int plans;   // radix plan variants the stage launches offer (1: the default only, 2: AltPlan too)
   int default_plan;  // the plan mask a new handle starts with
+  // F(u_i u_j) (00 11 22 01 02 12) of the fields U, at |k_i| < half only, into W[0..5] (internal layout)
+  cudaError_t (*products_low)(const PassArgs& a, int half, cudaStream_t s);
 };
 
 // values of PassArgs::prune
@@ -121,6 +124,8 @@ const DnsOps* find_ops3(int dtype, int Nx, int Ny, int Nz);
 // float array.
 cudaError_t closure_gradient(const void* U, int N, int comp, void* G3, int dtype, cudaStream_t st);
 cudaError_t closure_force(const void* S6, int N, void* F3, int dtype, cudaStream_t st);
+// the filter of dns_spectral_filter on `fields` fields of the internal layout (cubic grid, Nc <= Nf)
+cudaError_t filter_internal(const void* fine, int Nf, void* coarse, int Nc, int fields, int dtype, cudaStream_t st);
 cudaError_t fill_f32(float* p, size_t n, float v, cudaStream_t st);
 
 }  // namespace dns

@@ -76,6 +76,12 @@ __device__ __forceinline__ int4 ldfx(const cx<double>* p) { return __ldg(reinter
 // a / 4 rounded
 __device__ __forceinline__ fx fx_quarter(fx a) { return mk((a.x + 2) >> 2, (a.y + 2) >> 2); }
 
+// a b 2^-62, rounded; |a|, |b| <= 2^61
+__device__ __forceinline__ ll fx_prod(ll a, ll b) {
+  const int al = (int)a, ah = fx_hi(a), bl = (int)b, bh = fx_hi(b);
+  const ll t = madw(ah, bl, madw(al, bh, 1ll << 29));
+  return fx_times4(fx_add_up(t, madw(ah, bh, 0)), t);
+}
 // (a b - c d) 2^-62, rounded; |a|, |b|, |c|, |d| <= 2^61
 __device__ __forceinline__ ll fx_cross(ll a, ll b, ll c, ll d) {
   const int al = (int)a, ah = fx_hi(a), bl = (int)b, bh = fx_hi(b);

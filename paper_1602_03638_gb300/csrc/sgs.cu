@@ -27,12 +27,13 @@ constexpr int SGS_THREADS = 256;
 __device__ __forceinline__ int fftk(int i, int N) { return i < N / 2 ? i : i - N; }
 __device__ __forceinline__ double sincd(double x) { return fabs(x) < 1e-12 ? 1.0 : sin(x) / x; }
 
-template <typename T>
-__global__ void k_filter_truncate(const cx<T>* __restrict__ fine, int Nf, cx<T>* __restrict__ coarse, int Nc,
+// INTERNAL: the fine fields in the solver's layout [c][kz][ky][kx] (kz < Nf/2) instead of the public one
+template <typename T, bool INTERNAL>
+__global__ void k_filter_truncate(const cx<T>* __restrict__ fine, int Nf, cx<T>* __restrict__ coarse, int Nc, int fields,
                                   double scale, double half_width) {
   const int M1c = Nc / 2 + 1, M1f = Nf / 2 + 1;
   const size_t per = (size_t)Nc * Nc * M1c;
-  for (size_t i = blockIdx.x * (size_t)SGS_THREADS + threadIdx.x; i < 3 * per; i += (size_t)gridDim.x * SGS_THREADS) {
+  for (size_t i = blockIdx.x * (size_t)SGS_THREADS + threadIdx.x; i < fields * per; i += (size_t)gridDim.x * SGS_THREADS) {
     const int c = (int)(i / per);
     const size_t r = i % per;
     const int kz = (int)(r % M1c), b = (int)((r / M1c) % Nc), a = (int)(r / ((size_t)M1c * Nc));
@@ -41,7 +42,8 @@ __global__ void k_filter_truncate(const cx<T>* __restrict__ fine, int Nf, cx<T>*
     if (2 * abs(kx) < Nc && 2 * abs(ky) < Nc && 2 * kz < Nc) {
       const double g = sincd(kx * half_width) * sincd(ky * half_width) * sincd(kz * half_width) * scale;
       const int af = (kx + Nf) % Nf, bf = (ky + Nf) % Nf;
-      const cx<T> u = fine[((size_t)c * Nf * Nf + (size_t)af * Nf + bf) * M1f + kz];
+      const cx<T> u = INTERNAL ? fine[(((size_t)c * (Nf / 2) + kz) * Nf + bf) * Nf + af]
+                               : fine[((size_t)c * Nf * Nf + (size_t)af * Nf + bf) * M1f + kz];
       v = mk((T)(g * (double)u.x), (T)(g * (double)u.y));
     }
     coarse[i] = v;
@@ -173,6 +175,18 @@ __global__ void k_force_internal(const cx<T>* __restrict__ th, int N, cx<T>* __r
   }
 }
 
+template <bool INTERNAL>
+void filter_launch(const void* fine, int Nf, void* coarse, int Nc, int fields, int dtype, cudaStream_t st) {
+  const double scale = std::pow((double)Nc / (double)Nf, 3.0), hw = 3.14159265358979323846 / Nc;
+  const size_t n = (size_t)fields * Nc * Nc * (Nc / 2 + 1);
+  if (dtype == DNS_F32)
+    k_filter_truncate<float, INTERNAL><<<grid_for(n), SGS_THREADS, 0, st>>>((const cx<float>*)fine, Nf, (cx<float>*)coarse,
+                                                                            Nc, fields, scale, hw);
+  else
+    k_filter_truncate<double, INTERNAL><<<grid_for(n), SGS_THREADS, 0, st>>>((const cx<double>*)fine, Nf,
+                                                                             (cx<double>*)coarse, Nc, fields, scale, hw);
+}
+
 __global__ void k_fill_f32(float* __restrict__ p, size_t n, float v) {
   for (size_t i = blockIdx.x * (size_t)SGS_THREADS + threadIdx.x; i < n; i += (size_t)gridDim.x * SGS_THREADS) p[i] = v;
 }
@@ -199,6 +213,11 @@ cudaError_t closure_force(const void* S6, int N, void* F3, int dtype, cudaStream
   return cudaGetLastError();
 }
 
+cudaError_t filter_internal(const void* fine, int Nf, void* coarse, int Nc, int fields, int dtype, cudaStream_t st) {
+  filter_launch<true>(fine, Nf, coarse, Nc, fields, dtype, st);
+  return cudaGetLastError();
+}
+
 cudaError_t fill_f32(float* p, size_t n, float v, cudaStream_t st) {
   k_fill_f32<<<grid_for(n), SGS_THREADS, 0, st>>>(p, n, v);
   return cudaGetLastError();
@@ -211,15 +230,7 @@ extern "C" {
 int dns_spectral_filter(const void* fine, int Nf, void* coarse, int Nc, int dtype, void* stream) {
   if (!fine || !coarse || !ok_n(Nf) || !ok_n(Nc) || Nc > Nf || (dtype != DNS_F32 && dtype != DNS_F64))
     return bad("dns_spectral_filter: bad arguments (need device arrays, even Nc <= Nf)");
-  const double scale = std::pow((double)Nc / (double)Nf, 3.0), hw = 3.14159265358979323846 / Nc;
-  const size_t n = 3ull * Nc * Nc * (Nc / 2 + 1);
-  cudaStream_t st = (cudaStream_t)stream;
-  if (dtype == DNS_F32)
-    k_filter_truncate<float><<<grid_for(n), SGS_THREADS, 0, st>>>((const cx<float>*)fine, Nf, (cx<float>*)coarse, Nc,
-                                                                  scale, hw);
-  else
-    k_filter_truncate<double><<<grid_for(n), SGS_THREADS, 0, st>>>((const cx<double>*)fine, Nf, (cx<double>*)coarse,
-                                                                   Nc, scale, hw);
+  filter_launch<false>(fine, Nf, coarse, Nc, 3, dtype, (cudaStream_t)stream);
   return launched("dns_spectral_filter: launch failed");
 }
 

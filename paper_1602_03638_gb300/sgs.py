@@ -9,7 +9,8 @@ transforms (dns_transform_r2c/c2r), box filter and truncation
 
 Workflow
   1. fine DNS (this solver) -> snapshots
-  2. filtered_training_data(): ubar, gradient features X (10 x P), stress T (6 x P)
+  2. filtered_training_data(): ubar, gradient features X (10 x P), stress T (6 x P); the products of the
+     fine velocity are formed inside the solver's z-pass (dns_filtered_products)
   3. MLP.fit(): Adam on the standardised stress, BF16 products, FP32 weights
   4. set_closure_force(): before each coarse step, f = -div(MLP(grad ubar))
 """
@@ -132,29 +133,16 @@ def filtered_training_data(fine: Solver, coarse: Solver):
     ubar = box filter (width 2 pi/Nc) + truncation of u; T = filter(u_i u_j) - ubar_i ubar_j
     on the coarse grid. The fine solver's state is not changed.
     """
-    Nf, Nc, dt = fine.N, coarse.N, fine.dtype
+    Nc, dt = coarse.N, fine.dtype
     dev = "cuda"
     on_torch_stream(fine, coarse)
-    uh = torch.empty(fine.spec_shape, dtype=_cdt(dt), device=dev)
-    fine.get_state_spectral(uh)
-    u = torch.empty(fine.phys_shape, dtype=_rdt(dt), device=dev)
-    fine.get_state(u)
-    torch.cuda.synchronize()
-    prod = pointwise_products(u, dt)
-    del u
-    torch.cuda.synchronize()
-    pbar_hat = torch.empty((6, Nc, Nc, Nc // 2 + 1), dtype=_cdt(dt), device=dev)
-    for i in (0, 3):
-        spec = r2c(fine, prod[i:i + 3])
-        torch.cuda.synchronize()
-        pbar_hat[i:i + 3] = spectral_filter(spec, Nc, dt)
-        del spec
-    del prod
-    ubar_hat = spectral_filter(uh, Nc, dt)
-    torch.cuda.synchronize()
+    shape = (Nc, Nc, Nc // 2 + 1)
+    ubar_hat = torch.empty((3,) + shape, dtype=_cdt(dt), device=dev)
+    pbar_hat = torch.empty((6,) + shape, dtype=_cdt(dt), device=dev)
+    _lib.check(_lib.lib().dns_filtered_products(fine.handle, Nc, _p(ubar_hat), _p(pbar_hat)), "dns_filtered_products")
+    torch.cuda.synchronize()  # on torch's default stream the solvers keep streams of their own
     tau = c2r(coarse, pbar_hat)
     ubar = c2r(coarse, ubar_hat)
-    torch.cuda.synchronize()
     subtract_products(tau, ubar, dt)
     X = gradient_features(coarse, ubar_hat)
     T = tau.reshape(6, -1).to(torch.float32)
