@@ -48,40 +48,61 @@ const DnsOps* find_ops3(int dtype, int Nx, int Ny, int Nz) {
   return nullptr;
 }
 
+// 32 lanes per sum, each over every 32nd block, then a fixed tree: one thread per sum took 6 us of additions
 __global__ void k_diag_final(double* partials, int nblocks) {
-  if (threadIdx.x < 4) {
-    double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += partials[b * 4 + threadIdx.x];
-    partials[nblocks * 4 + threadIdx.x] = t;
-  }
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double t = 0.0;
+  for (int b = lane; b < nblocks; b += 32) t += partials[b * 4 + q];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) partials[nblocks * 4 + q] = t;
 }
 
-// The row flag of the state U (3 fields of M x Ny rows of Nx values, internal layout):
-// bit 0 is set if a row (kz, ky) outside the 2/3 box (3 kz >= k3z or 3 |ky| >= k3y) holds a
-// nonzero value, bit 1 if a row inside it does at a column with 3 |kx| >= k3x (NaN counts as
-// nonzero, -0 as zero); the bits are only set here (the caller clears the flag).
+// The row flag of a state (internal layout): bit 0 is set if a row (kz, ky) outside the 2/3 box (3 kz >= k3z
+// or 3 |ky| >= k3y) holds a nonzero value, bit 1 if a row inside it does at a column with 3 |kx| >= k3x
+// (NaN counts as nonzero, -0 as zero); the bits are only set here (check_rows clears the flag).
+struct RowCheck {
+  int k3x, k3y, k3z;
+  int* flag;  // nullptr: no check
+};
 template <typename T>
-__global__ void k_rows_outside(const cx<T>* __restrict__ U, int Nx, int Ny, int M, int k3x, int k3y, int k3z,
-                               int* flag) {
-  const size_t rows = (size_t)3 * M * Ny;
-  for (size_t r = blockIdx.x; r < rows; r += gridDim.x) {
-    const int ky = (int)(r % Ny), kz = (int)((r / Ny) % M);
-    const int kf = ky < Ny / 2 ? ky : ky - Ny;
-    const bool inside = 3 * kz < k3z && 3 * (kf < 0 ? -kf : kf) < k3y;  // the same for the whole block
-    const cx<T>* p = U + r * Nx;
-    int nz = 0;
-    for (int j = threadIdx.x; j < Nx; j += blockDim.x) {
-      const int kx = j < Nx / 2 ? j : j - Nx;
-      if (!inside || 3 * (kx < 0 ? -kx : kx) >= k3x) nz |= (p[j].x != (T)0) | (p[j].y != (T)0);
-    }
-    if (__syncthreads_or(nz) && threadIdx.x == 0) atomicOr(flag, inside ? 2 : 1);
+__device__ __forceinline__ int row_bits(cx<T> v, int kx, int ky, int kz, int Nx, int Ny, const RowCheck& c) {
+  const int fx = kx < Nx / 2 ? kx : Nx - kx, fy = ky < Ny / 2 ? ky : Ny - ky;  // |k|
+  const bool nz = (v.x != (T)0) | (v.y != (T)0);
+  const bool inside = 3 * kz < c.k3z && 3 * fy < c.k3y;
+  return !nz ? 0 : (!inside ? 1 : (3 * fx >= c.k3x ? 2 : 0));
+}
+__device__ __forceinline__ void put_row_bits(int bits, int* flag) {  // whole warps
+  bits = __reduce_or_sync(0xffffffffu, (unsigned)bits);
+  if ((threadIdx.x + threadIdx.y * blockDim.x) % 32 == 0 && (bits & ~*(volatile int*)flag)) atomicOr(flag, bits);
+}
+constexpr int ROWS_THREADS = 256;
+template <typename T>
+__global__ void __launch_bounds__(ROWS_THREADS) k_rows_outside(const cx<T>* __restrict__ U, int Nx, int Ny, int M,
+                                                               RowCheck c) {
+  // 16 bytes a thread and step: one or two columns of a row (Nx is even)
+  constexpr int V = 16 / (int)sizeof(cx<T>);
+  struct __align__(16) Pack {
+    cx<T> v[V];
+  };
+  const size_t n = (size_t)3 * M * Ny * Nx / V;
+  int bits = 0;
+  for (size_t i = (size_t)blockIdx.x * ROWS_THREADS + threadIdx.x; i < n; i += (size_t)gridDim.x * ROWS_THREADS) {
+    const Pack p = reinterpret_cast<const Pack*>(U)[i];
+    const unsigned per = (unsigned)(Nx / V);
+    const size_t r = i / per;
+    const int kx = (int)(i % per) * V, ky = (int)(r % Ny), kz = (int)((r / Ny) % M);
+#pragma unroll
+    for (int j = 0; j < V; ++j) bits |= row_bits(p.v[j], kx + j, ky, kz, Nx, Ny, c);
   }
+  put_row_bits(bits, c.flag);
 }
 
 // Paper order P[c][kx][ky][kz'] (kz' <= Nz/2)  <->  internal O[c][kz][ky][kx] (kz < Nz/2).
-// grid = (ceil(Nx/32), ceil(kzcount/32), 3*Ny), block = (32, 8)
+// grid = (ceil(Nx/32), ceil(kzcount/32), 3*Ny), block = (32, 8). Into the internal layout with the row
+// check of the values on the way (a pass over the new state saved: 0.25 ms at 512^3, 9 us at 64^3).
 template <typename T>
-__global__ void k_paper_to_internal(const cx<T>* __restrict__ P, cx<T>* __restrict__ O, int Nx, int Ny, int Nz) {
+__global__ void k_paper_to_internal(const cx<T>* __restrict__ P, cx<T>* __restrict__ O, int Nx, int Ny, int Nz,
+                                    RowCheck check) {
   __shared__ cx<T> tile[32][33];
   const int M = Nz / 2;
   const int c = blockIdx.z / Ny, ky = blockIdx.z % Ny;
@@ -91,14 +112,17 @@ __global__ void k_paper_to_internal(const cx<T>* __restrict__ P, cx<T>* __restri
     if (kx < Nx && kz < M) tile[i][threadIdx.x] = P[(((size_t)c * Nx + kx) * Ny + ky) * (M + 1) + kz];
   }
   __syncthreads();
+  int bits = 0;
   for (int i = threadIdx.y; i < 32; i += 8) {
     const int kz = kz0 + i, kx = kx0 + threadIdx.x;
     if (kx < Nx && kz < M) {
       cx<T> v = tile[threadIdx.x][i];
       if (kx == Nx / 2 || ky == Ny / 2) v = mk((T)0, (T)0);
       O[(((size_t)c * M + kz) * Ny + ky) * Nx + kx] = v;
+      if (check.flag) bits |= row_bits(v, kx, ky, kz, Nx, Ny, check);
     }
   }
+  if (check.flag) put_row_bits(bits, check.flag);
 }
 
 template <typename T>
@@ -290,6 +314,8 @@ struct dns_handle {
   cudaEvent_t cl_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   void* tw = nullptr;
   double* diag = nullptr;
+  int* host_flag = nullptr;  // pinned: where the row flag is read back to
+  bool flag_set = false;     // the row flag may hold bits
   size_t bytes = 0;
   size_t fs = 0;  // complex values per field
   bool w_valid = false;
@@ -332,6 +358,7 @@ void release(dns_handle* h) {
     if (ev) cudaEventDestroy(ev);
   for (cudaStream_t cs : h->cl_side)
     if (cs) cudaStreamDestroy(cs);
+  if (h->host_flag) cudaFreeHost(h->host_flag);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->own_stream) cudaStreamDestroy(h->own_stream);
 }
@@ -363,26 +390,26 @@ PassArgs base_args(const dns_handle* h) {
   return a;
 }
 
-// Where the state now in U vanishes (h->support, PRUNE_*): the row flag, bit 0 unless U
-// vanishes on every row (kz, ky) outside the handle's 2/3 box, bit 1 unless it also vanishes
-// at the columns |kx| >= N/3 of the rows inside, computed on the handle's stream and read
-// back (synchronises). A change re-captures the step graph.
-cudaError_t check_rows(dns_handle* h) {
-  int* flag = row_flag(h);
-  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), h->stream);
-  if (e != cudaSuccess) return e;
-  const int k3x = h->N + 2 * h->variant, k3y = h->Ny + 2 * h->variant, k3z = h->Nz + 2 * h->variant;
-  const int M = h->Nz / 2, blocks = 1024;
-  if (h->dtype == DNS_F32)
-    k_rows_outside<float><<<blocks, 256, 0, h->stream>>>((const cx<float>*)h->U, h->N, h->Ny, M, k3x, k3y, k3z, flag);
-  else
-    k_rows_outside<double><<<blocks, 256, 0, h->stream>>>((const cx<double>*)h->U, h->N, h->Ny, M, k3x, k3y, k3z,
-                                                          flag);
-  int f = 3;
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&f, flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+// Starts the check of a state against the handle's 2/3 box: what the kernels that set the flag take. The flag
+// is cleared on their stream, where the check before left bits in it.
+cudaError_t start_check(dns_handle* h, RowCheck* c) {
+  *c = RowCheck{h->N + 2 * h->variant, h->Ny + 2 * h->variant, h->Nz + 2 * h->variant, row_flag(h)};
+  const cudaError_t e = h->flag_set ? cudaMemsetAsync(row_flag(h), 0, sizeof(int), h->stream) : cudaSuccess;
+  h->flag_set = true;
+  return e;
+}
+
+// Where the state now in U vanishes (h->support, PRUNE_*), from the row flag that the kernels before on the
+// stream have set (synchronises): bit 0 unless U vanishes on every row (kz, ky) outside the handle's 2/3
+// box, bit 1 unless it also vanishes at the columns |kx| >= N/3 of the rows inside. A change
+// re-captures the step graph.
+cudaError_t read_rows(dns_handle* h) {
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h->host_flag, row_flag(h), sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return e;
+  const int f = *h->host_flag;
+  h->flag_set = f != 0;
   const int support = (f & 1) ? PRUNE_NONE : ((f & 2) ? PRUNE_ROWS : PRUNE_BOX);
   if (support != h->support) {
     h->support = support;
@@ -390,6 +417,21 @@ cudaError_t check_rows(dns_handle* h) {
     ++h->epoch;
   }
   return cudaSuccess;
+}
+
+// the same for a state that is in U already: a pass over it
+cudaError_t check_rows(dns_handle* h) {
+  const int M = h->Nz / 2;
+  const size_t n = 3 * h->fs * h->ops->elem_bytes / 16;
+  const int blocks = (int)std::min<size_t>((n + ROWS_THREADS - 1) / ROWS_THREADS, 2048);
+  RowCheck c;
+  const cudaError_t e = start_check(h, &c);
+  if (e != cudaSuccess) return e;
+  if (h->dtype == DNS_F32)
+    k_rows_outside<float><<<blocks, ROWS_THREADS, 0, h->stream>>>((const cx<float>*)h->U, h->N, h->Ny, M, c);
+  else
+    k_rows_outside<double><<<blocks, ROWS_THREADS, 0, h->stream>>>((const cx<double>*)h->U, h->N, h->Ny, M, c);
+  return read_rows(h);
 }
 
 int rk_stages(const dns_handle* h) { return h->rk.stages; }
@@ -489,18 +531,18 @@ size_t paper_spec_bytes(const dns_handle* h) {
   return (size_t)3 * h->N * h->Ny * (h->Nz / 2 + 1) * h->ops->elem_bytes;
 }
 
-cudaError_t launch_transpose(dns_handle* h, const void* src, void* dst, bool to_internal) {
+cudaError_t launch_transpose(dns_handle* h, const void* src, void* dst, bool to_internal, RowCheck check = RowCheck{}) {
   const int Nx = h->N, Ny = h->Ny, Nz = h->Nz, M = Nz / 2;
   dim3 block(32, 8);
   dim3 grid((Nx + 31) / 32, ((to_internal ? M : M + 1) + 31) / 32, 3 * Ny);
   if (h->dtype == 0) {
     if (to_internal)
-      k_paper_to_internal<float><<<grid, block, 0, h->stream>>>((const cx<float>*)src, (cx<float>*)dst, Nx, Ny, Nz);
+      k_paper_to_internal<float><<<grid, block, 0, h->stream>>>((const cx<float>*)src, (cx<float>*)dst, Nx, Ny, Nz, check);
     else
       k_internal_to_paper<float><<<grid, block, 0, h->stream>>>((const cx<float>*)src, (cx<float>*)dst, Nx, Ny, Nz);
   } else {
     if (to_internal)
-      k_paper_to_internal<double><<<grid, block, 0, h->stream>>>((const cx<double>*)src, (cx<double>*)dst, Nx, Ny, Nz);
+      k_paper_to_internal<double><<<grid, block, 0, h->stream>>>((const cx<double>*)src, (cx<double>*)dst, Nx, Ny, Nz, check);
     else
       k_internal_to_paper<double><<<grid, block, 0, h->stream>>>((const cx<double>*)src, (cx<double>*)dst, Nx, Ny, Nz);
   }
@@ -592,6 +634,8 @@ int dns_create3(int Nx, int Ny, int Nz, double nu, double dt, int dtype, dns_han
       ce = cudaMemcpy(h->tw, tfx.data(), tfx.size() * sizeof(int), cudaMemcpyHostToDevice);
     }
     if (ce == cudaSuccess) ce = cudaMemset(h->U, 0, 3 * h->fs * cb);
+    if (ce == cudaSuccess) ce = cudaMemset(row_flag(h), 0, sizeof(int));
+    if (ce == cudaSuccess) ce = cudaMallocHost(&h->host_flag, sizeof(int));
     if (ce != cudaSuccess) rc = cuda_fail(ce, "dns_create initialisation");
   }
   if (rc != DNS_OK) {
@@ -1005,8 +1049,10 @@ int dns_set_state_spectral(dns_handle* h, const void* uhat, int on_device) {
              "dns_set_state_spectral copy");
     src = h->W;
   }
-  DNS_CUDA(launch_transpose(h, src, h->U, true), "dns_set_state_spectral transpose");
-  DNS_CUDA(check_rows(h), "dns_set_state_spectral row check");
+  RowCheck check;
+  DNS_CUDA(start_check(h, &check), "dns_set_state_spectral row check");
+  DNS_CUDA(launch_transpose(h, src, h->U, true, check), "dns_set_state_spectral transpose");
+  DNS_CUDA(read_rows(h), "dns_set_state_spectral row check");
   h->w_valid = false;
   h->t = 0.0;
   return DNS_OK;

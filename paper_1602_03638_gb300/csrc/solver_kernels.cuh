@@ -2337,7 +2337,7 @@ struct SolverImpl {
 
   static cudaError_t diag(const PassArgs& a, cudaStream_t st) {
     k_diag<T, N, NY, NZ><<<DIAG_BLOCKS, DG_THREADS, 0, st>>>(a);
-    k_diag_final<<<1, 32, 0, st>>>(a.partials, DIAG_BLOCKS);
+    k_diag_final<<<1, 128, 0, st>>>(a.partials, DIAG_BLOCKS);
     k_xpass<T, N, XM_INV_DIV, NY, NZ><<<ROWS, XP_THREADS, G::XSMEM, st>>>(f32args(a));
     y_go<1, 0, 0>(reinterpret_cast<cx<T>*>(a.D), reinterpret_cast<const cx<T>*>(a.tw), k3y(a), M, 1, st);
     cudaMemsetAsync(a.maxbits, 0, sizeof(unsigned long long), st);
