@@ -19,6 +19,8 @@
 // [component][kz][ky][kx], kz < N/2, kx and ky in FFT order.
 #pragma once
 
+#include <cuda.h>  // CUtensorMap
+
 #include <type_traits>
 
 #include "dns_internal.h"
@@ -1126,15 +1128,10 @@ __global__ void __launch_bounds__(ZP_THREADS<T>, (Geometry<T, N>::ZMIN)) k_zpass
 }
 
 // ---------------------------------------------------------------------------
-// Half-warp 256-point FFT of the N = 512 z-pass (lines of M = 256 values): each
-// line belongs to one half-warp, lane h holding positions h + 16 m (m < 16),
-// and the 256-point DFT is two radix-16 passes with a single shared-memory
-// exchange whose stores (17 h + r) and loads (h + 17 m) are free of bank
-// conflicts.
+// Line transforms of k_ztma. A line of M = 128 or 256 values belongs to M / 16 lanes, lane h holding positions
+// h + (M / 16) m (m < 16). HwTwL, per lane: the twiddle powers exp(-2 pi i h r / M) between its two passes, and the
+// pair twiddle exp(-2 pi i (h + (M / 16) m) / 2M), formed on use as tl exp(-2 pi i m / 32) with a constant factor.
 // ---------------------------------------------------------------------------
-// Leaner per-lane twiddles for the FP32 pipelined z-pass: the second-pass powers
-// p2[r] as in HwTw, and exp(-2 pi i (h + 16 m) / 512) formed on use as
-// tl * exp(-2 pi i m / 32) with the second factor a compile-time constant.
 struct HwTwL {
   cx<float> p2[16];
   cx<float> tl;
@@ -1143,7 +1140,7 @@ struct HwTwL {
     twiddle_powers<16>(ldro(tw + 2 * h * ts), p2);
     tl = ldro(tw + h * ts);
   }
-  __device__ __forceinline__ cx<float> wk(const cx<float>* __restrict__, int, int m) const {
+  __device__ __forceinline__ cx<float> wk(int m) const {
     constexpr float c[16][2] = {
         {1.0f, -0.0f},
         {0.9807852804032304f, -0.19509032201612825f},
@@ -1166,228 +1163,11 @@ struct HwTwL {
   }
 };
 
-template <typename T, int TWN, int ES, class HT>
-__device__ __forceinline__ void hw_fft256(cx<T> (&v)[16], cx<T>* ln, const HT& ht, const cx<T>* __restrict__ tw,
-                                          int h) {
-  dft16(v);
-  cx<T>* q = ln + 17 * h * ES;
-#pragma unroll
-  for (int r = 0; r < 16; ++r) q[r * ES] = v[r];
-  __syncwarp();
-  const cx<T>* rb = ln + h * ES;
-#pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = rb[17 * m * ES];
-  __syncwarp();
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], ht.p2[r]);
-  } else {
-    constexpr int C = TWN / 256;
-#pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], ldro(tw + h * r * C));
-  }
-  dft16(v);
-}
-
-// ---------------------------------------------------------------------------
-// Pipelined z-pass for N = 512: one persistent block per SM walks tiles of
-// 128-byte rows (16 adjacent x in FP32, 8 in FP64) at fixed y. The whole tile
-// (6 fields x 256 kz) sits in shared memory and arrives by cp.async straight
-// into the padded layout; the next tile's omega fields are fetched while the
-// products are transformed and stored, its u fields while the omega lines are
-// transformed, so HBM traffic overlaps the shared-memory-bound transforms.
-// Line transforms, cross product and walks are those of k_zcross16. FP32 only:
-// the FP64 form (8 x per row) would spill and keeps k_zcross16.
-// ---------------------------------------------------------------------------
-template <typename T>
-struct Z16P {
-  static constexpr int M = 256;
-  static constexpr int TX = 128 / (int)sizeof(cx<T>);  // 128-byte rows
-  static constexpr int LD = odd_ld(6 * TX);
-  static constexpr int NW = 24;                        // warps per block
-  static constexpr int ITEMS = (M / 32) * TX;          // walk items per field
-  static constexpr size_t SMEM = (size_t)padded_len(M) * LD * sizeof(cx<T>);
-};
-
-template <typename T, int N>
-__global__ void __launch_bounds__(32 * Z16P<T>::NW, 1) k_zcross16p(PassArgs a) {
-  using P = Z16P<T>;
-  constexpr int M = P::M, TX = P::TX, LD = P::LD, NW = P::NW, ITEMS = P::ITEMS;
-  constexpr size_t FS = Geometry<T, N>::FS;
-  constexpr int XT = N / TX, NT = XT * N;  // tiles: x-tiles times y
-  static_assert(N == 512 && (TX == 8 || TX == 16), "k_zcross16p is the N = 512 z-pass");
-  static_assert((3 * ITEMS) % NW == 0, "z tile load split");
-    extern __shared__ unsigned char smraw[];
-  cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
-  const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
-  cx<T>* W = reinterpret_cast<cx<T>*>(a.W);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = lane & 15, half = lane >> 4;
-  int kc = (a.kmax3 + 2) / 3;
-  if (kc > M) kc = M;
-  const int tx = lane % TX, kq = lane / TX;
-  // lane part of the walk kz = 32 g + TX kq + c: padp(kz) = 34 g + padp(TX kq) + c
-  cx<T>* const sl = s + padp(TX * kq) * LD + tx;
-  const size_t lane_g = ((size_t)(TX * kq) * N) * N + tx;
-
-  // asynchronous fetch of fields f0 .. f0+2 of tile t into their lines. Warp w takes the
-  // 16 consecutive walk items 16 w + j: with ITEMS = 8 TX = 128 its field (w / 8) and row
-  // group g = w % 8 are fixed and j is the row offset c, so the addresses are a per-warp
-  // base plus j times a constant stride.
-  static_assert(TX == 16 && ITEMS == 128 && 3 * ITEMS == 16 * NW, "z tile chunking");
-  auto fetch = [&](int t, int f0) {
-    // a stage whose state vanishes outside the 2/3 box: the planes kz >= kc hold zeros (the
-    // y-inverse left them alone) and are filled with zeros instead of read
-    const int f = f0 + w / 8, g = w % 8;
-    const cx<T>* gl = W + lane_g + (size_t)(t / XT) * N + (t % XT) * TX + (size_t)f * FS + (size_t)(32 * g) * N * N;
-    cx<T>* sd = sl + 34 * g * LD + f * TX;
-    if (rows_vanish(a)) {
-      const int nv = kc - (32 * g + TX * kq);  // rows of this lane's chunk below kc
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        if (j < nv) cp_async<sizeof(cx<T>)>(sd + j * LD, gl + (size_t)j * N * N);
-        else sd[j * LD] = mk((T)0, (T)0);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) cp_async<sizeof(cx<T>)>(sd + j * LD, gl + (size_t)j * N * N);
-    }
-  };
-  // c2r of the TX lines of fields f0 .. f0+2, two lines per warp at a time
-  HwTwL ht;
-  ht.init(tw, h);
-  // partner X_{M-k} of k = h + 16 m sits at padded row padp(M - k) = pb0 + 17 (15 - m)
-  // with pb0 = 16 - h for h > 0 and 17 for h = 0 (k = 0 has no partner: X_M = 0)
-  const int pb0 = (h == 0) ? 17 : 16 - h;
-  // The inputs of modes k and M - k come from one pair (X_k, X_{M-k}): with
-  // A = X_k + conj X_{M-k}, B = X_k - conj X_{M-k} and P = i conj(w_k) B,
-  // z_k = A + P and z_{M-k} = conj(A - P). Lane h forms the pairs of its slots
-  // m < 8 (k = h + 16 m); the mirror M - k = (16 - h) + 16 (15 - m) is slot
-  // 15 - m of lane 16 - h, which receives it by a shuffle. Lane 0 pairs its slots
-  // m and 16 - m, takes the self-paired k = M/2 at m = 0 and forms k = 0 apart.
-  auto c2r_lines = [&](int f0) {
-    cx<T> v[16];
-#pragma unroll 1
-    for (int l = f0 * TX + 2 * w + half; l < (f0 + 3) * TX; l += 2 * NW) {
-      cx<T>* ln = s + l;
-      const cx<T>* pa = ln + h * LD;
-      const cx<T>* pb = ln + pb0 * LD;
-      const cx<T> x0 = ln[0];
-      cx<T> zq[8];
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        cx<T> xk, xm, wk;
-        if (m == 0) {
-          const cx<T>* ph = ln + padp(M / 2) * LD;
-          xk = (h == 0) ? *ph : pa[0];
-          xm = (h == 0) ? xk : pb[17 * 15 * LD];
-          wk = (h == 0) ? mk((T)0, (T)-1) : ht.wk(tw, h, 0);  // w_{M/2} = -i
-        } else {
-          xk = pa[17 * m * LD];
-          xm = pb[17 * (15 - m) * LD];
-          wk = ht.wk(tw, h, m);
-        }
-        const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
-        const cx<T> P = mul_pi(cmul(conjg(wk), B));
-        v[m] = conjg(A + P);
-        zq[m] = A - P;  // conj of z_{M-k}
-      }
-      const int src = (16 - h) & 15;
-#pragma unroll
-      for (int q = 8; q < 16; ++q) {
-        v[q].x = __shfl_sync(0xffffffffu, zq[15 - q].x, src, 16);
-        v[q].y = __shfl_sync(0xffffffffu, zq[15 - q].y, src, 16);
-      }
-      if (h == 0) {
-        v[8] = v[0];
-#pragma unroll
-        for (int q = 9; q < 16; ++q) v[q] = zq[16 - q];
-        v[0] = mk(x0.x, -x0.x);  // z_0 = (1 + i) Re X_0: Im X_0 ignored, X_M = 0
-      }
-      __syncwarp();
-      hw_fft256<T, N, LD>(v, ln, ht, tw, h);
-      cx<T>* pw = ln + h * LD;
-#pragma unroll
-      for (int m = 0; m < 16; ++m) pw[17 * m * LD] = conjg(v[m]);
-    }
-  };
-
-  int t = blockIdx.x;
-  if (t < NT) fetch(t, 3);
-  cp_async_commit();
-  if (t < NT) fetch(t, 0);
-  cp_async_commit();
-#pragma unroll 1
-  for (; t < NT; t += gridDim.x) {
-    const int x0 = (t % XT) * TX, y = t / XT, tn = t + gridDim.x;
-    cp_async_wait<1>();  // omega fields of tile t
-    __syncthreads();
-    c2r_lines(3);
-    cp_async_wait<0>();  // u fields of tile t
-    __syncthreads();
-    c2r_lines(0);
-    __syncthreads();
-    // u x omega at every point, into the u lines
-    for (int it = w; it < ITEMS; it += NW) {
-      const int g = it / TX, c = it % TX;
-      cx<T>* p = sl + (34 * g + c) * LD;
-      const cx<T> u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];
-      const cx<T> w0 = p[3 * TX], w1v = p[4 * TX], w2 = p[5 * TX];
-      p[0 * TX] = mk(u1.x * w2.x - u2.x * w1v.x, u1.y * w2.y - u2.y * w1v.y);
-      p[1 * TX] = mk(u2.x * w0.x - u0.x * w2.x, u2.y * w0.y - u0.y * w2.y);
-      p[2 * TX] = mk(u0.x * w1v.x - u1.x * w0.x, u0.y * w1v.y - u1.y * w0.y);
-    }
-    __syncthreads();
-    if (tn < NT) fetch(tn, 3);  // the omega lines are free
-    cp_async_commit();
-    // r2c of the 3 TX product lines; X_k (k < kc) back into the line
-    {
-      cx<T> v[16];
-#pragma unroll 1
-      for (int l = 2 * w + half; l < 3 * TX; l += 2 * NW) {
-        cx<T>* ln = s + l;
-        const cx<T>* pa = ln + h * LD;
-#pragma unroll
-        for (int m = 0; m < 16; ++m) v[m] = pa[17 * m * LD];
-        __syncwarp();
-        hw_fft256<T, N, LD>(v, ln, ht, tw, h);
-        cx<T>* po = ln + h * LD;
-        const int partner = (16 - h) & 15;
-#pragma unroll
-        for (int m = 0; m < 16; ++m) {
-          if (16 * m >= kc) break;  // slots m and above hold modes past the 2/3 cut
-          cx<T> zo;
-          zo.x = __shfl_sync(0xffffffffu, v[15 - m].x, partner, 16);
-          zo.y = __shfl_sync(0xffffffffu, v[15 - m].y, partner, 16);
-          if (h == 0) zo = v[(16 - m) & 15];
-          const cx<T> wk = ht.wk(tw, h, m);
-          const cx<T> A = v[m] + conjg(zo), B = v[m] - conjg(zo);
-          if (h + 16 * m < kc) po[17 * m * LD] = scal(A + mul_mi(cmul(wk, B)), (T)0.5);
-        }
-      }
-    }
-    __syncthreads();
-    {  // the same chunks as the fetch: field w / 8, rows 32 (w % 8) + TX kq + j
-      const int f = w / 8, g = w % 8, k0 = 32 * g + TX * kq;
-      cx<T>* gd = W + lane_g + (size_t)y * N + x0 + (size_t)f * FS + (size_t)(32 * g) * N * N;
-      const cx<T>* sd = sl + 34 * g * LD + f * TX;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (k0 + j < kc) gd[(size_t)j * N * N] = sd[j * LD];
-    }
-    __syncthreads();  // the u lines have been read out
-    if (tn < NT) fetch(tn, 0);
-    cp_async_commit();
-  }
-  cp_async_wait<0>();
-}
-
 // ---------------------------------------------------------------------------
 // Half-warp 512-point FFT for the N = 1024 z-pass (FP32). Lane h of a half-warp
 // holds v[m] = x[h + 16 m], m < 32. With k = k1 + 32 k2: a 32-point DFT over m in
 // each lane gives Y[h][k1]; after the twiddle exp(-2 pi i h k1 / 512) one
-// shared-memory exchange (stores at 33 h + k1, loads at 33 h + h' and
-// 33 h + h' + 16: conflict-free for any odd element stride) gives lane h' the
+// shared-memory exchange gives lane h' the
 // 16-point columns k1 = h' and h' + 16, whose DFTs over h leave
 // v[j] = X[h' + 16 j] in the lane: the input layout again.
 // ---------------------------------------------------------------------------
@@ -1395,13 +1175,13 @@ struct HwTw32 {
   cx<float> p[16];  // w^r, w = exp(-2 pi i h / 512), r < 16
   cx<float> q[16];  // w^(16 + r)
   cx<float> tl;     // exp(-2 pi i h / 1024)
-  __device__ __forceinline__ void init(const cx<float>* __restrict__ tw, int h) {
-    twiddle_powers<16>(ldro(tw + 2 * h), p);
+  __device__ __forceinline__ void init(const cx<float>* __restrict__ tw, int h, int ts) {
+    twiddle_powers<16>(ldro(tw + 2 * h * ts), p);
     p[0] = mk(1.f, 0.f);
     const cx<float> w16 = cmul(p[8], p[8]);
 #pragma unroll
     for (int r = 0; r < 16; ++r) q[r] = r == 0 ? w16 : cmul(w16, p[r]);
-    tl = ldro(tw + h);
+    tl = ldro(tw + h * ts);
   }
   // exp(-2 pi i (h + 16 m) / 1024) = tl * exp(-2 pi i m / 64)
   __device__ __forceinline__ cx<float> wk(int m) const {
@@ -1442,394 +1222,313 @@ struct HwTw32 {
   }
 };
 
-template <int ES>
-__device__ __forceinline__ void hw_fft512(cx<float> (&v)[32], cx<float>* ln, const HwTw32& ht, int h) {
-  dft32(v);
-#pragma unroll
-  for (int k = 1; k < 32; ++k) v[k] = cmul(v[k], k < 16 ? ht.p[k] : ht.q[k - 16]);
-  cx<float>* q = ln + 33 * h * ES;
-#pragma unroll
-  for (int k = 0; k < 32; ++k) q[k * ES] = v[k];
-  __syncwarp();
-  cx<float> a[16], b[16];
-  const cx<float>* rb = ln + h * ES;
-#pragma unroll
-  for (int g = 0; g < 16; ++g) {
-    a[g] = rb[33 * g * ES];
-    b[g] = rb[(33 * g + 16) * ES];
-  }
-  __syncwarp();
-  dft16(a);
-  dft16(b);
-#pragma unroll
-  for (int k2 = 0; k2 < 16; ++k2) {
-    v[2 * k2] = a[k2];
-    v[2 * k2 + 1] = b[k2];
+// ---------------------------------------------------------------------------
+// Pipelined z-pass of the FP32 grids with z-lines of 256, 512 or 1024 points: one persistent block per SM walks
+// tiles of TX adjacent x at fixed y, the whole tile (6 fields x M kz, 192 KB) in shared memory. Tensor copies (TMA)
+// fill it with whole rows and drain the products' rows, the planes past the cut-off filled with zeros or left out
+// by the bounds of the tensor; the next tile's omega arrives while the products are transformed, its u while
+// omega is.
+//
+// Bound by the shared-memory pipe (12.7 k of its cycles a tile, two thirds busy at 512). Rows arrive in the copies'
+// swizzle (16-byte chunks of a row permuted by the row number), so a warp takes pairs of adjacent columns: its
+// half-warps' accesses are eight rows of a column pair, 128 bytes of distinct banks, and the exchange inside a line
+// goes through rows permuted the same way (an address is one XOR). Against tiles moved in 8-byte pieces by cp.async
+// and drained by the threads (each 32 pieces took six cycles of that pipe, a quarter of all; an address and an
+// instruction each): 512^3 1476 -> 1059 us, 1024^3 15.99 -> 13.33 ms, 256^3 167 -> 144 us, 1024 x 512 x 256
+// 1271 -> 1065 us. Shorter lines keep k_zpass (tiles of their own width, batched members).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ cx<float> lds(unsigned p) {
+  cx<float> v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(p));
+  return v;
+}
+__device__ __forceinline__ void sts(unsigned p, cx<float> v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y));
+}
+__device__ __forceinline__ float4 lds4(unsigned p) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(p));
+  return v;
+}
+__device__ __forceinline__ void sts4(unsigned p, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+}
+// what threads did to shared memory before the copies that follow a barrier
+__device__ __forceinline__ void fence_copies() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// waits for the phase `parity` of the mbarrier; false if it did not complete within a second
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+  unsigned long long t0 = 0;
+  for (int it = 0;; ++it) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (it == 0) t0 = t;
+    else if (t - t0 > 1000000000ull) return false;
   }
 }
 
-// Pipelined z-pass for N = 1024, FP32, with half-warp lines: the schedule of
-// k_zcross16p (persistent block, whole tile in shared memory, next tile's omega
-// fields fetched during the product transforms, its u fields during the omega
-// transforms) on tiles of 8 adjacent x (64-byte rows) and 512-value lines.
-template <typename T>
-struct Z32P {
-  static constexpr int M = 512;
-  static constexpr int TX = 64 / (int)sizeof(cx<T>);
-  static constexpr int LD = odd_ld(6 * TX);
-  static constexpr int NW = 12;
-  static constexpr int ITEMS = (M / 32) * TX;
-  static constexpr size_t SMEM = (size_t)padded_len(M) * LD * sizeof(cx<T>);
+template <int M>
+struct ZTma {
+  static constexpr int TX = 4096 / M;                    // columns of a tile (32 KB a field)
+  static constexpr int CX = TX < 16 ? TX : 16;           // columns of a copy: a field is TX / CX blocks of M rows
+  static constexpr int ROWB = CX * 8, CB = M * ROWB, FB = 32768;  // bytes of a row (128 or 64), of a block, of a field
+  static constexpr int HL = M == 128 ? 8 : 16, VALS = M / HL;  // lanes of a line, values of a line in a lane
+  static constexpr int GL = 32 / HL;                     // columns of a warp
+  static constexpr int NW = VALS == 16 ? 24 : 12;        // warps: 80 or 168 registers a thread
+  static constexpr int BOX = M < 256 ? M : 256;          // rows of a copy
+  static constexpr size_t SMEM = 6 * FB + 2048;          // 2 KB alignment: the address bits that are XORed
+  using Tw = std::conditional_t<M == 512, HwTw32, HwTwL>;
+  // swizzle of the copies: chunk ^ (row / (128 / ROWB)) % (ROWB / 16)
+  static constexpr int SH = ROWB == 128 ? 0 : 1, MASK = ROWB / 16 - 1;
+  static constexpr CUtensorMapSwizzle SWIZZLE = ROWB == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+  // row r of a line and its chunk, to be XORed into the address of chunk p of row 0 (r < 2048 / ROWB)
+  __host__ __device__ static constexpr unsigned at(unsigned r) { return r * ROWB | ((r >> SH) & MASK) * 16; }
 };
 
-template <typename T, int N>
-__global__ void __launch_bounds__(32 * Z32P<T>::NW, 1) k_zcross32p(PassArgs a) {
-  using P = Z32P<T>;
-  using G = Geometry<T, N>;
-  constexpr int M = P::M, TX = P::TX, LD = P::LD, NW = P::NW, ITEMS = P::ITEMS;
-  constexpr size_t FS = G::FS;
-  constexpr int XT = N / TX, NT = XT * N;
-  static_assert(N == 1024 && sizeof(T) == 4 && TX == 8, "k_zcross32p is the FP32 N = 1024 z-pass");
-  static_assert((3 * ITEMS) % NW == 0 && (3 * TX) % (2 * NW) == 0, "z tile split");
-  extern __shared__ unsigned char smraw[];
-  cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
-  const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
-  cx<T>* W = reinterpret_cast<cx<T>*>(a.W);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = lane & 15, half = lane >> 4;
-  int kc = (a.kmax3 + 2) / 3;
-  if (kc > M) kc = M;
-  const int tx = lane % TX, kq = lane / TX;
-  // walk kz = 32 g + TX kq + c: padp(kz) = 34 g + padp(TX kq) + c
-  cx<T>* const sl = s + padp(TX * kq) * LD + tx;
-  const size_t lane_g = ((size_t)(TX * kq) * N) * N + tx;
-  // warp w takes the 32 consecutive walk items 32 w + j (j = 8 a + b): field f0 + w / 4, row
-  // group g = 4 (w % 4) + a, row offset c = b, so the addresses are a per-warp base plus
-  // compile-time offsets
-  static_assert(TX == 8 && ITEMS == 128 && 3 * ITEMS == 32 * NW, "z tile chunking");
-  auto fetch = [&](int t, int f0) {
-    // planes kz >= kc of a stage whose state vanishes outside the 2/3 box: zeros, not read
-    const int f = f0 + w / 4, q = w % 4;
-    const cx<T>* gl = W + lane_g + (size_t)(t / XT) * N + (t % XT) * TX + (size_t)f * FS + (size_t)(128 * q) * N * N;
-    cx<T>* sd = sl + 136 * q * LD + f * TX;
-    if (rows_vanish(a)) {
-      const int nv = kc - (128 * q + TX * kq);  // this lane's rows below kc: 32 (j / 8) + j % 8 < nv
+// The M-point DFT of a line of HL lanes, lane h holding x[h + HL m] and then X[h + HL m]. Value r of lane h crosses
+// in row R h + (r ^ h) of the line (R rows a lane). la: address of the line's row h.
+//   M = 128: 16-point DFTs, two 8-point ones;  256: 16 x 16;  512: 32-point DFTs, two 16-point ones (HwTw32)
+template <int M>
+__device__ __forceinline__ void zt_fft(cx<float> (&v)[ZTma<M>::VALS], unsigned la, const typename ZTma<M>::Tw& ht, int h) {
+  using Z = ZTma<M>;
+  const unsigned we = la + h * Z::VALS * Z::ROWB;
+  if constexpr (M == 256) {
+    dft16(v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        if (32 * (j / 8) + j % 8 < nv)
-          cp_async<sizeof(cx<T>)>(sd + (34 * (j / 8) + j % 8) * LD, gl + (size_t)(32 * (j / 8) + j % 8) * N * N);
-        else
-          sd[(34 * (j / 8) + j % 8) * LD] = mk((T)0, (T)0);
-      }
+    for (int r = 0; r < 16; ++r) sts(we ^ Z::at(r), v[r]);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = lds((la ^ Z::at(m)) + m * 16 * Z::ROWB);
+    __syncwarp();
+#pragma unroll
+    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], ht.p2[r]);
+    dft16(v);
+  } else {
+    constexpr int R = Z::VALS;
+    if constexpr (M == 128) {
+      dft16(v);
+#pragma unroll
+      for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], ht.p2[k]);
     } else {
+      dft32(v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j)
-        cp_async<sizeof(cx<T>)>(sd + (34 * (j / 8) + j % 8) * LD, gl + (size_t)(32 * (j / 8) + j % 8) * N * N);
+      for (int k = 1; k < 32; ++k) v[k] = cmul(v[k], k < 16 ? ht.p[k] : ht.q[k - 16]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) sts(we ^ Z::at(r), v[r]);
+    __syncwarp();
+    cx<float> a[R / 2], b[R / 2];
+#pragma unroll
+    for (int g = 0; g < R / 2; ++g) {
+      const unsigned q = (la ^ Z::at(g)) + g * R * Z::ROWB;
+      a[g] = lds(q);
+      b[g] = lds(q + R / 2 * Z::ROWB);
+    }
+    __syncwarp();
+    dft<R / 2>(a);
+    dft<R / 2>(b);
+#pragma unroll
+    for (int k2 = 0; k2 < R / 2; ++k2) {
+      v[2 * k2] = a[k2];
+      v[2 * k2 + 1] = b[k2];
+    }
+  }
+}
+
+// in: W as (x, y, kz, field), kz bounded by the planes that hold values; out: by the planes kept
+template <int N, int NY, int NZ>
+__global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
+    k_ztma(int kmax3, const void* __restrict__ twp, const __grid_constant__ CUtensorMap in,
+           const __grid_constant__ CUtensorMap out) {
+  constexpr int M = NZ / 2;
+  using Z = ZTma<M>;
+  constexpr int TX = Z::TX, CX = Z::CX, NW = Z::NW, FB = Z::FB, HL = Z::HL, V = Z::VALS, STEP = HL * Z::ROWB;
+  constexpr int XT = N / TX, NT = XT * NY;  // tiles: x-tiles times y
+  static_assert(N % TX == 0, "whole tiles");
+  extern __shared__ unsigned char smraw[];
+  __shared__ unsigned long long bars[2];
+  const unsigned s = ((unsigned)__cvta_generic_to_shared(smraw) + 2047u) & ~2047u;
+  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(bars), bar1 = bar0 + 8;
+  const cx<float>* tw = reinterpret_cast<const cx<float>*>(twp);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // lane: column bit 3 of a pair; row h < HL in bits 0-2 and, of 16, 4 (of 8: the second pair)
+  const int h = HL == 16 ? (lane & 7) | ((lane >> 4) << 3) : lane & 7, cb = (lane >> 3) & 1;
+  const int hp = (HL - h) & (HL - 1);
+  const int partner = HL == 16 ? (hp & 7) | (cb << 3) | ((hp >> 3) << 4) : (lane & 24) | hp;  // the lane of row HL - h
+  const int kc = min((kmax3 + 2) / 3, M);
+
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar1) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  auto fetch = [&](int t, int f0, unsigned bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(3 * FB) : "memory");
+    for (int b = f0 * (TX / CX); b < (f0 + 3) * (TX / CX); ++b) {
+      for (int k = 0; k < M; k += Z::BOX)
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+            ::"r"(s + b * Z::CB + k * Z::ROWB), "l"(&in), "r"((t % XT) * TX + (b % (TX / CX)) * CX), "r"(t / XT), "r"(k),
+            "r"(b / (TX / CX)), "r"(bar)
+            : "memory");
     }
   };
-  HwTw32 ht;
-  ht.init(tw, h);
-  // partner X_{M-k} of k = h + 16 m at padded row pb0 + 17 (31 - m), pb0 = 16 - h (h > 0), 17 (h = 0)
-  const int pb0 = (h == 0) ? 17 : 16 - h;
+  typename Z::Tw ht;
+  ht.init(tw, h, Geometry<float, N, NY, NZ>::TW / NZ);
+  // address of row r (the row h or HL - h of this lane) of this lane's column, the warp's columns starting at line l
+  auto row = [&](int l, int r) {
+    const int x = l + (HL == 8 ? (lane >> 4) * 2 : 0);
+    return s + (x / CX) * Z::CB + r * Z::ROWB + (((x % CX) / 2) ^ ((r >> Z::SH) & Z::MASK)) * 16 + cb * 8;
+  };
+
+  // c2r of the TX lines of fields f0 .. f0+2, GL lines per warp at a time.
+  // The inputs of modes k and M - k come from one pair (X_k, X_{M-k}): with
+  // A = X_k + conj X_{M-k}, B = X_k - conj X_{M-k} and P = i conj(w_k) B,
+  // z_k = A + P and z_{M-k} = conj(A - P). Lane h forms the pairs of its slots
+  // m < V/2 (k = h + HL m); the mirror M - k = (HL - h) + HL (V - 1 - m) is slot
+  // V - 1 - m of lane HL - h, which receives it by a shuffle. Lane 0 pairs its slots
+  // m and V - m, takes the self-paired k = M/2 at m = 0 and forms k = 0 apart.
   auto c2r_lines = [&](int f0) {
-    cx<T> v[32];
+    cx<float> v[V];
 #pragma unroll 1
-    for (int l = f0 * TX + 2 * w + half; l < (f0 + 3) * TX; l += 2 * NW) {
-      cx<T>* ln = s + l;
-      const cx<T>* pa = ln + h * LD;
-      const cx<T>* pb = ln + pb0 * LD;
-      const cx<T> x0 = ln[0];
-      // modes k = h + 16 m (m < 16) and M - k = (16 - h) + 16 (31 - m) from one pair:
-      // z_k = A + P, z_{M-k} = conj(A - P), the mirror going to slot 31 - m of lane
-      // 16 - h; lane 0 pairs its slots m and 32 - m and takes k = M/2 at m = 0
-      cx<T> zq[16];
+    for (int l = f0 * TX + Z::GL * w; l < (f0 + 3) * TX; l += Z::GL * NW) {
+      const unsigned pa = row(l, h), pb = row(l, HL - h);
+      const cx<float> x0 = lds(pa);
+      cx<float> zq[V / 2];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        cx<T> xk, xm, wk;
+      for (int m = 0; m < V / 2; ++m) {
+        cx<float> xk, xm, w1;
         if (m == 0) {
-          const cx<T>* ph = ln + padp(M / 2) * LD;
-          xk = (h == 0) ? *ph : pa[0];
-          xm = (h == 0) ? xk : pb[17 * 31 * LD];
-          wk = (h == 0) ? mk((T)0, (T)-1) : ht.wk(0);  // w_{M/2} = -i
+          const cx<float> y = lds(h == 0 ? pa + V / 2 * STEP : pb + (V - 1) * STEP);  // X_{M/2}, X_{M-h}
+          xk = h == 0 ? y : x0;
+          xm = y;
+          w1 = h == 0 ? mk(0.f, -1.f) : ht.wk(0);  // w_{M/2} = -i
         } else {
-          xk = pa[17 * m * LD];
-          xm = pb[17 * (31 - m) * LD];
-          wk = ht.wk(m);
+          xk = lds(pa + m * STEP);
+          xm = lds(pb + (V - 1 - m) * STEP);
+          w1 = ht.wk(m);
         }
-        const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
-        const cx<T> P = mul_pi(cmul(conjg(wk), B));
+        const cx<float> A = xk + conjg(xm), B = xk - conjg(xm);
+        const cx<float> P = mul_pi(cmul(conjg(w1), B));
         v[m] = conjg(A + P);
         zq[m] = A - P;  // conj of z_{M-k}
       }
-      const int src = (16 - h) & 15;
 #pragma unroll
-      for (int q = 16; q < 32; ++q) {
-        v[q].x = __shfl_sync(0xffffffffu, zq[31 - q].x, src, 16);
-        v[q].y = __shfl_sync(0xffffffffu, zq[31 - q].y, src, 16);
+      for (int q = V / 2; q < V; ++q) {
+        v[q].x = __shfl_sync(0xffffffffu, zq[V - 1 - q].x, partner);
+        v[q].y = __shfl_sync(0xffffffffu, zq[V - 1 - q].y, partner);
       }
       if (h == 0) {
-        v[16] = v[0];
+        v[V / 2] = v[0];
 #pragma unroll
-        for (int q = 17; q < 32; ++q) v[q] = zq[32 - q];
+        for (int q = V / 2 + 1; q < V; ++q) v[q] = zq[V - q];
         v[0] = mk(x0.x, -x0.x);  // z_0 = (1 + i) Re X_0: Im X_0 ignored, X_M = 0
       }
       __syncwarp();
-      hw_fft512<LD>(v, ln, ht, h);
-      cx<T>* pw = ln + h * LD;
+      zt_fft<M>(v, pa, ht, h);
 #pragma unroll
-      for (int m = 0; m < 32; ++m) pw[17 * m * LD] = conjg(v[m]);
+      for (int m = 0; m < V; ++m) sts(pa + m * STEP, conjg(v[m]));
     }
   };
 
   int t = blockIdx.x;
-  if (t < NT) fetch(t, 3);
-  cp_async_commit();
-  if (t < NT) fetch(t, 0);
-  cp_async_commit();
+  if (threadIdx.x == 0 && t < NT) {
+    fetch(t, 3, bar0);
+    fetch(t, 0, bar1);
+  }
+  bool ok = true;  // a copy that does not arrive leaves NaN, which the checks of the state report
+  unsigned phase = 0;
 #pragma unroll 1
-  for (; t < NT; t += gridDim.x) {
-    const int x0 = (t % XT) * TX, y = t / XT, tn = t + gridDim.x;
-    cp_async_wait<1>();  // omega fields of tile t
-    __syncthreads();
+  for (; t < NT; t += gridDim.x, phase ^= 1) {
+    const int tn = t + gridDim.x;
+    ok = ok && mbar_wait(bar0, phase);  // omega fields of tile t
     c2r_lines(3);
-    cp_async_wait<0>();  // u fields of tile t
-    __syncthreads();
+    ok = ok && mbar_wait(bar1, phase);  // u fields of tile t
     c2r_lines(0);
     __syncthreads();
-    for (int it = w; it < ITEMS; it += NW) {
-      const int g = it / TX, c = it % TX;
-      cx<T>* p = sl + (34 * g + c) * LD;
-      const cx<T> u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];
-      const cx<T> w0 = p[3 * TX], w1v = p[4 * TX], w2 = p[5 * TX];
-      p[0 * TX] = mk(u1.x * w2.x - u2.x * w1v.x, u1.y * w2.y - u2.y * w1v.y);
-      p[1 * TX] = mk(u2.x * w0.x - u0.x * w2.x, u2.y * w0.y - u0.y * w2.y);
-      p[2 * TX] = mk(u0.x * w1v.x - u1.x * w0.x, u0.y * w1v.y - u1.y * w0.y);
+    // u x omega at every point, into the u lines: all fields are permuted alike
+    for (int i = threadIdx.x; i < FB / 16; i += 32 * NW) {
+      const unsigned p = s + i * 16;
+      const float4 u0 = lds4(p), u1 = lds4(p + FB), u2 = lds4(p + 2 * FB);
+      const float4 w0 = lds4(p + 3 * FB), w1 = lds4(p + 4 * FB), w2 = lds4(p + 5 * FB);
+      sts4(p, make_float4(u1.x * w2.x - u2.x * w1.x, u1.y * w2.y - u2.y * w1.y, u1.z * w2.z - u2.z * w1.z,
+                          u1.w * w2.w - u2.w * w1.w));
+      sts4(p + FB, make_float4(u2.x * w0.x - u0.x * w2.x, u2.y * w0.y - u0.y * w2.y, u2.z * w0.z - u0.z * w2.z,
+                               u2.w * w0.w - u0.w * w2.w));
+      sts4(p + 2 * FB, make_float4(u0.x * w1.x - u1.x * w0.x, u0.y * w1.y - u1.y * w0.y, u0.z * w1.z - u1.z * w0.z,
+                                   u0.w * w1.w - u1.w * w0.w));
     }
+    fence_copies();
     __syncthreads();
-    if (tn < NT) fetch(tn, 3);  // the omega lines are free
-    cp_async_commit();
+    if (threadIdx.x == 0 && tn < NT) fetch(tn, 3, bar0);  // the omega lines are free
+    // r2c of the 3 TX product lines; X_k (k < kc) back into the line
     {
-      cx<T> v[32];
+      const float half = ok ? 0.5f : __int_as_float(0x7fffffff);
+      cx<float> v[V];
 #pragma unroll 1
-      for (int l = 2 * w + half; l < 3 * TX; l += 2 * NW) {
-        cx<T>* ln = s + l;
-        const cx<T>* pa = ln + h * LD;
+      for (int l = Z::GL * w; l < 3 * TX; l += Z::GL * NW) {
+        const unsigned pa = row(l, h);
 #pragma unroll
-        for (int m = 0; m < 32; ++m) v[m] = pa[17 * m * LD];
+        for (int m = 0; m < V; ++m) v[m] = lds(pa + m * STEP);
         __syncwarp();
-        hw_fft512<LD>(v, ln, ht, h);
-        cx<T>* po = ln + h * LD;
-        const int partner = (16 - h) & 15;
+        zt_fft<M>(v, pa, ht, h);
 #pragma unroll
-        for (int m = 0; m < 32; ++m) {
-          if (16 * m >= kc) break;  // slots m and above hold modes past the 2/3 cut
-          cx<T> zo;
-          zo.x = __shfl_sync(0xffffffffu, v[31 - m].x, partner, 16);
-          zo.y = __shfl_sync(0xffffffffu, v[31 - m].y, partner, 16);
-          if (h == 0) zo = v[(32 - m) & 31];
-          const cx<T> wk = ht.wk(m);
-          const cx<T> A = v[m] + conjg(zo), B = v[m] - conjg(zo);
-          if (h + 16 * m < kc) po[17 * m * LD] = scal(A + mul_mi(cmul(wk, B)), (T)0.5);
+        for (int m = 0; m < V; ++m) {
+          if (HL * m >= kc) break;  // slots m and above hold modes past the 2/3 cut
+          cx<float> zo;
+          zo.x = __shfl_sync(0xffffffffu, v[V - 1 - m].x, partner);
+          zo.y = __shfl_sync(0xffffffffu, v[V - 1 - m].y, partner);
+          if (h == 0) zo = v[(V - m) & (V - 1)];
+          const cx<float> A = v[m] + conjg(zo), B = v[m] - conjg(zo);
+          if (h + HL * m < kc) sts(pa + m * STEP, scal(A + mul_mi(cmul(ht.wk(m), B)), half));
         }
       }
     }
+    fence_copies();
     __syncthreads();
-    {  // the same chunks as the fetch: field w / 4, rows 128 (w % 4) + 32 a + TX kq + b
-      const int f = w / 4, q = w % 4, k0 = 128 * q + TX * kq;
-      cx<T>* gd = W + lane_g + (size_t)y * N + x0 + (size_t)f * FS + (size_t)(128 * q) * N * N;
-      const cx<T>* sd = sl + 136 * q * LD + f * TX;
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (k0 + 32 * (j / 8) + j % 8 < kc) gd[(size_t)(32 * (j / 8) + j % 8) * N * N] = sd[(34 * (j / 8) + j % 8) * LD];
+    if (threadIdx.x == 0) {
+      for (int b = 0; b < 3 * (TX / CX); ++b) {
+        for (int k = 0; k < kc; k += Z::BOX)
+          asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
+                       ::"l"(&out), "r"((t % XT) * TX + (b % (TX / CX)) * CX), "r"(t / XT), "r"(k), "r"(b / (TX / CX)),
+                       "r"(s + b * Z::CB + k * Z::ROWB)
+                       : "memory");
+      }
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the u lines have been read out
+      if (tn < NT) fetch(tn, 0, bar1);
     }
-    __syncthreads();  // the u lines have been read out
-    if (tn < NT) fetch(tn, 0);
-    cp_async_commit();
   }
-  cp_async_wait<0>();
+  if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// ---------------------------------------------------------------------------
-// Quarter-warp 128-point FFT for the N = 256 z-pass (FP32): lane h < 8 of a
-// quarter-warp holds v[m] = x[h + 8 m], m < 16; a 16-point DFT in each lane, the
-// twiddle exp(-2 pi i h k1 / 128), one exchange through positions 17 h + k1 and two
-// 8-point DFTs per lane leave v[j] = X[h + 8 j] in the lane. The two quarter-warps of
-// a half-warp work on lines l and l + 8, whose banks are disjoint. The twiddles are
-// those of the 256-point half-warp transform (HwTwL) on the N = 256 table.
-// ---------------------------------------------------------------------------
-template <int ES>
-__device__ __forceinline__ void qw_fft128(cx<float> (&v)[16], cx<float>* ln, const HwTwL& qt, int h) {
-  dft16(v);
-#pragma unroll
-  for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], qt.p2[k]);
-  cx<float>* q = ln + 17 * h * ES;
-#pragma unroll
-  for (int k = 0; k < 16; ++k) q[k * ES] = v[k];
-  __syncwarp();
-  cx<float> a[8], b[8];
-  const cx<float>* rb = ln + h * ES;
-#pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    a[g] = rb[17 * g * ES];
-    b[g] = rb[(17 * g + 8) * ES];
-  }
-  __syncwarp();
-  dft8(a);
-  dft8(b);
-#pragma unroll
-  for (int k2 = 0; k2 < 8; ++k2) {
-    v[2 * k2] = a[k2];
-    v[2 * k2 + 1] = b[k2];
-  }
-}
-
-template <typename T>
-struct Z8Q {
-  static constexpr int M = 128;
-  static constexpr int TX = 128 / (int)sizeof(cx<T>);  // 128-byte rows
-  static constexpr int LD = odd_ld(6 * TX);
-  static constexpr int NW = 12;
-  static constexpr int ITEMS = (M / 32) * TX;
-  static constexpr size_t SMEM = (size_t)padded_len(M) * LD * sizeof(cx<T>);
-};
-
-// z-pass for N = 256, FP32: one tile (16 adjacent x at fixed y, 6 fields of 128
-// values) per block, fetched whole by cp.async, two blocks per SM; each warp
-// transforms four lines at once as quarter-warps (lines b, b + 8, b + 1, b + 9).
-// NY, NZ: counts along y and z where they differ from N (NZ = 256; N a multiple of 16).
-template <typename T, int N, int NY = N, int NZ = N>
-__global__ void __launch_bounds__(32 * Z8Q<T>::NW, 2) k_zcross8q(PassArgs a) {
-  using P = Z8Q<T>;
-  using G = Geometry<T, N, NY, NZ>;
-  constexpr int M = P::M, TX = P::TX, LD = P::LD, NW = P::NW, ITEMS = P::ITEMS;
-  constexpr size_t FS = G::FS;
-  constexpr size_t PL = (size_t)NY * N;  // one kz plane
-  static_assert(NZ == 256 && N % TX == 0 && sizeof(T) == 4 && TX == 16, "k_zcross8q is the FP32 256-point z-pass");
-  static_assert((6 * ITEMS) % NW == 0, "z tile split");
-  extern __shared__ unsigned char smraw[];
-  cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
-  const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
-  cx<T>* W = reinterpret_cast<cx<T>*>(a.W);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = lane & 7, qw = lane >> 3;
-  const int x0 = blockIdx.x * TX, y = blockIdx.y;
-  int kc = ((NZ == N ? a.kmax3 : a.kmax3z) + 2) / 3;
-  if (kc > M) kc = M;
-  const int tx = lane % TX, kq = lane / TX;
-  // walk kz = 32 g + TX kq + c: padp(kz) = 34 g + padp(TX kq) + c
-  cx<T>* const sl = s + padp(TX * kq) * LD + tx;
-  const cx<T>* gl = W + ((size_t)(TX * kq) * NY + y) * N + x0 + tx;
-  // warp w takes the 32 consecutive walk items 32 w + j (j = 16 a + b): field w / 2, row group
-  // g = 2 (w % 2) + a, row offset c = b: a per-warp base plus compile-time offsets
-  static_assert(TX == 16 && ITEMS == 64 && 6 * ITEMS == 32 * NW && 3 * ITEMS == 16 * NW, "z tile chunking");
-  {
-    const int f = w / 2, q = w % 2;
-    const cx<T>* gf = gl + (size_t)f * FS + (size_t)(64 * q) * PL;
-    cx<T>* sd = sl + 68 * q * LD + f * TX;
-    if (rows_vanish(a)) {  // planes kz >= kc of a state that vanishes outside the 2/3 box: zeros
-      const int nv = kc - (64 * q + TX * kq);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        if (32 * (j / 16) + j % 16 < nv)
-          cp_async<sizeof(cx<T>)>(sd + (34 * (j / 16) + j % 16) * LD, gf + (size_t)(32 * (j / 16) + j % 16) * PL);
-        else
-          sd[(34 * (j / 16) + j % 16) * LD] = mk((T)0, (T)0);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        cp_async<sizeof(cx<T>)>(sd + (34 * (j / 16) + j % 16) * LD, gf + (size_t)(32 * (j / 16) + j % 16) * PL);
-    }
-  }
-  cp_async_commit();
-  HwTwL qt;  // w = exp(-2 pi i h / 128), tl = exp(-2 pi i h / 256)
-  qt.init(tw, h, G::TW / NZ);
-  // quarter-warp line of group gi (groups of 4 lines b, b + 8, b + 1, b + 9 with b = 16 f + 2 i)
-  auto line_of = [&](int gi) { return 16 * (gi >> 2) + 2 * (gi & 3) + (qw & 1) * 8 + (qw >> 1); };
-  cp_async_wait<0>();
-  __syncthreads();
-  {
-    cx<T> v[16];
-#pragma unroll 1
-    for (int gi = w; gi < 6 * 4; gi += NW) {  // c2r of the 96 lines
-      cx<T>* ln = s + line_of(gi);
-      const cx<T> x0 = ln[0];
-      // modes k = h + 8 m (m < 8) and M - k = (8 - h) + 8 (15 - m) from one pair:
-      // z_k = A + P, z_{M-k} = conj(A - P), the mirror going to slot 15 - m of lane
-      // 8 - h; lane 0 pairs its slots m and 16 - m and takes k = M/2 at m = 0
-      cx<T> zq[8];
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int k = (m == 0 && h == 0) ? M / 2 : h + 8 * m;
-        const cx<T> xk = ln[padp(k) * LD];
-        const cx<T> xm = (m == 0 && h == 0) ? xk : ln[padp(M - k) * LD];
-        const cx<T> wk = (m == 0 && h == 0) ? mk((T)0, (T)-1) : qt.wk(tw, h, m);  // w_{M/2} = -i
-        const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
-        const cx<T> P = mul_pi(cmul(conjg(wk), B));
-        v[m] = conjg(A + P);
-        zq[m] = A - P;  // conj of z_{M-k}
-      }
-      const int src = (8 - h) & 7;
-#pragma unroll
-      for (int q = 8; q < 16; ++q) {
-        v[q].x = __shfl_sync(0xffffffffu, zq[15 - q].x, src, 8);
-        v[q].y = __shfl_sync(0xffffffffu, zq[15 - q].y, src, 8);
-      }
-      if (h == 0) {
-        v[8] = v[0];
-#pragma unroll
-        for (int q = 9; q < 16; ++q) v[q] = zq[16 - q];
-        v[0] = mk(x0.x, -x0.x);  // z_0 = (1 + i) Re X_0: Im X_0 ignored, X_M = 0
-      }
-      __syncwarp();
-      qw_fft128<LD>(v, ln, qt, h);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) ln[padp(h + 8 * m) * LD] = conjg(v[m]);
-    }
-  }
-  __syncthreads();
-  for (int it = w; it < ITEMS; it += NW) {
-    const int g = it / TX, c = it % TX;
-    cx<T>* p = sl + (34 * g + c) * LD;
-    const cx<T> u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];
-    const cx<T> w0 = p[3 * TX], w1v = p[4 * TX], w2 = p[5 * TX];
-    p[0 * TX] = mk(u1.x * w2.x - u2.x * w1v.x, u1.y * w2.y - u2.y * w1v.y);
-    p[1 * TX] = mk(u2.x * w0.x - u0.x * w2.x, u2.y * w0.y - u0.y * w2.y);
-    p[2 * TX] = mk(u0.x * w1v.x - u1.x * w0.x, u0.y * w1v.y - u1.y * w0.y);
-  }
-  __syncthreads();
-  {
-    cx<T> v[16];
-    const int partner = (8 - h) & 7;
-#pragma unroll 1
-    for (int gi = w; gi < 3 * 4; gi += NW) {  // r2c of the 48 product lines
-      cx<T>* ln = s + line_of(gi);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) v[m] = ln[padp(h + 8 * m) * LD];
-      __syncwarp();
-      qw_fft128<LD>(v, ln, qt, h);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        if (8 * m >= kc) break;  // slots m and above hold modes past the 2/3 cut
-        cx<T> zo;
-        zo.x = __shfl_sync(0xffffffffu, v[15 - m].x, partner, 8);
-        zo.y = __shfl_sync(0xffffffffu, v[15 - m].y, partner, 8);
-        if (h == 0) zo = v[(16 - m) & 15];
-        const cx<T> wk = qt.wk(tw, h, m);
-        const cx<T> A = v[m] + conjg(zo), B = v[m] - conjg(zo);
-        if (h + 8 * m < kc) ln[padp(h + 8 * m) * LD] = scal(A + mul_mi(cmul(wk, B)), (T)0.5);
-      }
-    }
-  }
-  __syncthreads();
-  {  // warp w stores items 16 w + j: field w / 4, rows 32 (w % 4) + TX kq + j
-    const int f = w / 4, g = w % 4, k0 = 32 * g + TX * kq;
-    cx<T>* gd = W + ((size_t)(TX * kq) * NY + y) * N + x0 + tx + (size_t)f * FS + (size_t)(32 * g) * PL;
-    const cx<T>* sd = sl + 34 * g * LD + f * TX;
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (k0 + j < kc) gd[(size_t)j * PL] = sd[j * LD];
-  }
+// The tensor (x, y, kz < planes, field < fields) at W, and the box of a copy
+template <int N, int NY, int NZ>
+inline cudaError_t ztma_map(CUtensorMap* map, void* W, int planes, int fields) {
+  using Z = ZTma<NZ / 2>;
+  typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const Encode encode = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess
+               ? (Encode)f : (Encode) nullptr;
+  }();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t dims[4] = {N, NY, (cuuint64_t)planes, (cuuint64_t)fields};
+  const cuuint64_t strides[3] = {N * 8ull, (cuuint64_t)N * NY * 8, (cuuint64_t)N * NY * (NZ / 2) * 8};
+  const cuuint32_t box[4] = {Z::CX, 1, Z::BOX, 1}, step[4] = {1, 1, 1, 1};
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, W, dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            Z::SWIZZLE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------
@@ -1906,8 +1605,8 @@ struct SolverImpl {
   static constexpr bool ISO = NY == N && NZ == N;
   static constexpr int ROWS = M * NY;  // x-pass rows (kz, ky)
   static constexpr bool BATCHED = ISO && N <= BATCH_MAX_N;
-  // non-cubic grids with 256-point FP32 z-lines use the quarter-warp z-pass of 256^3
-  static constexpr bool Z8_BOX = !ISO && NZ == 256 && sizeof(T) == 4 && N % 16 == 0;
+  // FP32 z-lines of 256 to 1024 points: k_ztma
+  static constexpr bool ZTMA = sizeof(T) == 4 && (NZ == 256 || NZ == 512 || NZ == 1024);
   // each direction's 2/3 cut-off (3|k_i| < kmax3 of that direction)
   static int k3y(const PassArgs& a) { return NY == N ? a.kmax3 : a.kmax3y; }
   static int k3z(const PassArgs& a) { return NZ == N ? a.kmax3 : a.kmax3z; }
@@ -2084,10 +1783,7 @@ struct SolverImpl {
       DNS_ATTR((k_ypass<T, N, 0, 1, 0, N, N, 1>), (YCfg<T, N, 0, 0>::SMEM));
       DNS_ATTR((k_zpass<T, N, ZM_CROSS, 0, N, N, 1>), G::ZSMEM);
     }
-    if constexpr (ISO && N == 512 && sizeof(T) == 4) DNS_ATTR((k_zcross16p<T, N>), Z16P<T>::SMEM);
-    if constexpr (ISO && N == 1024 && sizeof(T) == 4) DNS_ATTR((k_zcross32p<T, N>), Z32P<T>::SMEM);
-    if constexpr (ISO && N == 256 && sizeof(T) == 4) DNS_ATTR((k_zcross8q<T, N>), Z8Q<T>::SMEM);
-    if constexpr (Z8_BOX) DNS_ATTR((k_zcross8q<T, N, NY, NZ>), Z8Q<T>::SMEM);
+    if constexpr (ZTMA) DNS_ATTR((k_ztma<N, NY, NZ>), ZTma<M>::SMEM);
     DNS_ATTR((k_zpass<T, N, ZM_STORE, 0, NY, NZ>), G::ZSMEM);
     DNS_ATTR((k_zpass<T, N, ZM_LOAD, 0, NY, NZ>), G::ZSMEM);
     DNS_ATTR((k_zpass<T, N, ZM_MAXABS, 0, NY, NZ>), G::ZSMEM);
@@ -2110,18 +1806,17 @@ struct SolverImpl {
     return e;
   }
 
-  static void z_cross(const PassArgs& a, cudaStream_t st) {
-    if constexpr (Z8_BOX)
-      k_zcross8q<T, N, NY, NZ><<<dim3(N / Z8Q<T>::TX, NY), 32 * Z8Q<T>::NW, Z8Q<T>::SMEM, st>>>(a);
-    else if constexpr (!ISO)
+  static cudaError_t z_cross(const PassArgs& a, cudaStream_t st) {
+    if constexpr (ZTMA) {
+      CUtensorMap in, out;
+      const int kc = kc_of(k3z(a));
+      cudaError_t e = ztma_map<N, NY, NZ>(&in, a.W, a.prune >= PRUNE_ROWS ? kc : M, 6);
+      if (e == cudaSuccess) e = ztma_map<N, NY, NZ>(&out, a.W, kc, 3);
+      if (e != cudaSuccess) return e;
+      k_ztma<N, NY, NZ><<<num_sms(), 32 * ZTma<M>::NW, ZTma<M>::SMEM, st>>>(k3z(a), a.tw, in, out);
+    } else if constexpr (!ISO) {
       z_go<0>(a, st);
-    else if constexpr (N == 512 && sizeof(T) == 4)
-      k_zcross16p<T, N><<<num_sms(), 32 * Z16P<T>::NW, Z16P<T>::SMEM, st>>>(a);
-    else if constexpr (N == 1024 && sizeof(T) == 4)
-      k_zcross32p<T, N><<<num_sms(), 32 * Z32P<T>::NW, Z32P<T>::SMEM, st>>>(a);
-    else if constexpr (N == 256 && sizeof(T) == 4)
-      k_zcross8q<T, N><<<dim3(N / Z8Q<T>::TX, N), 32 * Z8Q<T>::NW, Z8Q<T>::SMEM, st>>>(a);
-    else {
+    } else {
       with_plan(bit(a.plan, PLAN_Z), [&](auto v) {
         constexpr int V = decltype(v)::value;
         if constexpr (ztile_ok(4)) if (a.ztile == 4) return z_go<4, V>(a, st);
@@ -2131,6 +1826,7 @@ struct SolverImpl {
         z_go<0, V>(a, st);
       });
     }
+    return cudaGetLastError();
   }
 
   // shared memory of a stage-update launch: with the wide layout only the rows
@@ -2174,12 +1870,14 @@ struct SolverImpl {
                   reinterpret_cast<const cx<T>*>(a.tw), k3y(a), pr ? kc_of(k3z(a)) : M, 6, st, pr);
   }
 
-  static void rhs_front(const PassArgs& a, cudaStream_t st) {
+  static cudaError_t rhs_front(const PassArgs& a, cudaStream_t st) {
     cx<T>* W = reinterpret_cast<cx<T>*>(a.W);
     const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
     y_inverse(a, st);
-    z_cross(a, st);
+    const cudaError_t e = z_cross(a, st);
+    if (e != cudaSuccess) return e;
     y_stage<0, 1>(a.ytile[1], bit(a.plan, PLAN_YF), W, tw, k3y(a), kc_of(k3z(a)), 3, st);
+    return cudaGetLastError();
   }
 
   // the x-stage launch of a stage, in the form of the stage's scheme
@@ -2194,7 +1892,8 @@ struct SolverImpl {
   }
 
   static cudaError_t rk_stage(const PassArgs& a, cudaStream_t st) {
-    rhs_front(a, st);
+    const cudaError_t e = rhs_front(a, st);
+    if (e != cudaSuccess) return e;
     x_stage(a, st);
     return cudaGetLastError();
   }
@@ -2204,7 +1903,7 @@ struct SolverImpl {
     const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
     switch (part) {
       case 0: y_inverse(a, st); break;
-      case 1: z_cross(a, st); break;
+      case 1: return z_cross(a, st);
       case 2: y_stage<0, 1>(a.ytile[1], bit(a.plan, PLAN_YF), W, tw, k3y(a), kc_of(k3z(a)), 3, st); break;
       default: x_stage(a, st); break;
     }
@@ -2277,7 +1976,8 @@ struct SolverImpl {
   static cudaError_t rhs(const PassArgs& a, cudaStream_t st) {
     cudaError_t e = x_inverse_curl(a, 0, st);
     if (e != cudaSuccess) return e;
-    rhs_front(a, st);
+    e = rhs_front(a, st);
+    if (e != cudaSuccess) return e;
     PassArgs b = a;
     b.stage = 0;
     with_plan(bit(b.plan, PLAN_X), [&](auto v) {
