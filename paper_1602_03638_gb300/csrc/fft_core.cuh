@@ -268,6 +268,44 @@ template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING) : "memory"); }
 
 // ---------------------------------------------------------------------------
+// Bulk copies (contiguous ranges, tensor boxes) that report to an mbarrier.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+// makes the initialised barriers known to the copies; a block barrier follows
+__device__ __forceinline__ void mbar_init_done() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// bytes (a multiple of 16) of contiguous memory; both addresses 16-byte aligned
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* gmem_src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(smem_dst)), "l"(gmem_src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// what threads did to shared memory before the copies that follow a barrier
+__device__ __forceinline__ void fence_copies() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// waits for the phase `parity` of the mbarrier; false if it did not complete within a second
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+  unsigned long long t0 = 0;
+  for (int it = 0;; ++it) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (it == 0) t0 = t;
+    else if (t - t0 > 1000000000ull) return false;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Shared-memory line layout: element p sits at padded position p + p/16. With
 // this padding both the contiguous accesses (j + r*L/R over lanes j) and the
 // stride-R Stockham stores of every pass used here touch each bank pair at

@@ -57,7 +57,7 @@ struct Geometry {
   // x-pass: one row (fixed kz, ky) per block, 6 padded line buffers. The
   // stage update (XPRE, where it fits in 100 KB) uses 3 padded lines (the
   // nonlinear term, then u) and 9 unpadded rows that receive the stage's state
-  // rows by cp.async (then omega in rows 0-2 and the padded work lines of the
+  // rows by asynchronous copies (then omega in rows 0-2 and the padded work lines of the
   // omega transforms over rows 3-8).
   // Where 6 padded lines and the 9 rows fit in 64 KB (XWIDE), omega keeps
   // its own 3 padded lines instead (faster at N = 512 FP32).
@@ -65,6 +65,11 @@ struct Geometry {
   static constexpr bool XWIDE = (size_t)((6 * XLS + 1) / 2 * 2 + 9 * N) * CB <= 64 * 1024;
   static constexpr int XST = ((XWIDE ? 6 : 3) * XLS + 1) / 2 * 2;  // 16-byte aligned start of the state rows
   static constexpr bool XPRE = CB == 8 && (size_t)(XST + 9 * N) * CB <= 100 * 1024;
+  // Rows of 2 KB and more arrive by bulk copies instead (one thread issues them; no asynchronous copy per value:
+  // those took a quarter of the shared-memory pipe's cycles): x-stage 512^3 816 -> 689 us (its bytes: 670 at the
+  // copy bandwidth), 1024^3 8.02 -> 7.19 ms, 1024 x 512 x 256 1022 -> 913 us, 256^3 103 -> 94 us; 128^3, whose
+  // rows are 1 KB, the same within the noise.
+  static constexpr bool XBULK = XPRE && N >= 128;
   static constexpr size_t XSMEM = (size_t)6 * XLS * CB;
   static constexpr size_t XSMEM_ST = XPRE ? (size_t)(XST + 9 * N) * CB : XSMEM;  // XM_STAGE, XM_RHS
   // z-pass: ZTX adjacent x at fixed y, 6 fields of M values each, <= 112 KB
@@ -246,7 +251,8 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
 
   if constexpr (STAGE || MODE == XM_RHS) {
     // rows outside the box: skip their forward transform
-    const T nu = par<T>(a.nu, a.f_nu), cA = par<T>(a.cA, a.f_cA), cB = par<T>(a.cB, a.f_cB);
+    T nu = par<T>(a.nu, a.f_nu);
+    const T cA = par<T>(a.cA, a.f_cA), cB = par<T>(a.cB, a.f_cB);
     const int stage = a.stage, last = a.last;
     // Williamson 2N stages keep the stage state in U (updated in place) and dU in U1
     constexpr bool lsrk = MODE == XM_STAGE2N;
@@ -260,7 +266,47 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
     // the columns |kx| >= N/3 of this row too: its rows are read and written at the kept
     // columns only, the others give u = omega = 0
     const bool xbox = STAGE && box_vanish(a);
-    if constexpr (G::XPRE) {
+    if constexpr (G::XBULK) {
+      // rows of W where the lines lie (unpadded, from an even value on; a line's first pass takes it all before
+      // it stores), rows of the state: whole, or the kept columns' two ranges
+      __shared__ unsigned long long bars[2];
+      const unsigned bw = smem_addr(bars), bs = bw + 8;
+      if (threadIdx.x == 0) {
+        mbar_init(bw);
+        mbar_init(bs);
+        mbar_init_done();
+        if (row_kept) {
+          mbar_expect(bw, 3 * N * 8);
+#pragma unroll 1
+          for (int f = 0; f < 3; ++f) bulk_load(s + (f * LS + 1) / 2 * 2, W + f * FS + rb, N * 8, bw);
+        }
+        const int R = (a.kmax3 + 2) / 3 - 1;  // the last kept column
+        int lo = (R + 2) / 2 * 2, hi = (N - R) / 2 * 2;
+        if (!xbox || lo >= hi) lo = hi = N;
+        const int rows = 3 * (1 + need1 + need0);
+        mbar_expect(bs, rows * (lo + N - hi) * 8);
+#pragma unroll 1
+        for (int f = 0; f < 3; ++f) {
+          auto fetch_row = [&](const cx<T>* src, cx<T>* dst) {
+            bulk_load(dst + f * N, src + f * FS + rb, lo * 8, bs);
+            if (hi < N) bulk_load(dst + f * N + hi, src + f * FS + rb + hi, (N - hi) * 8, bs);
+          };
+          fetch_row(Sst, st);
+          if (need1) fetch_row(U1, st + 3 * N);
+          if (need0) fetch_row(U, st + 6 * N);
+        }
+      }
+      __syncthreads();
+      bool ok = true;
+      if (row_kept && warp < 3) {
+        ok = mbar_wait(bw, 0);
+        const SLine<T, 1> line{s + warp * LS};
+        line_fft<T, N, TW, V>(SRow<T>{s + (warp * LS + 1) / 2 * 2}, line, line, tw, lane);
+      }
+      ok = mbar_wait(bs, 0) && ok;
+      if (!ok) nu = (T)__int_as_float(0x7fffffff);  // a copy that does not arrive: NaN, which the checks of the state report
+      __syncthreads();
+    } else if constexpr (G::XPRE) {
       if (row_kept) {
         for (int e = threadIdx.x; e < 3 * N; e += NT) {
           const int f = e / N, j = e % N;
@@ -295,7 +341,7 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
         line_fft<T, N, TW, V>(GLoad<T, false>{W + warp * FS + rb}, line, line, tw, lane);
       }
     }
-    __syncthreads();
+    if constexpr (!G::XBULK) __syncthreads();
     // state values of component c at column j: staged rows or global memory
     auto ld_s = [&](int c, int j) -> cx<T> { return G::XPRE ? st[c * N + j] : Sst[c * FS + rb + j]; };
     auto ld_1 = [&](int c, int j) -> cx<T> { return G::XPRE ? st[(3 + c) * N + j] : U1[c * FS + rb + j]; };
@@ -1253,26 +1299,6 @@ __device__ __forceinline__ float4 lds4(unsigned p) {
 __device__ __forceinline__ void sts4(unsigned p, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
 }
-// what threads did to shared memory before the copies that follow a barrier
-__device__ __forceinline__ void fence_copies() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// waits for the phase `parity` of the mbarrier; false if it did not complete within a second
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-  unsigned long long t0 = 0;
-  for (int it = 0;; ++it) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    if (it == 0) t0 = t;
-    else if (t - t0 > 1000000000ull) return false;
-  }
-}
-
 template <int M>
 struct ZTma {
   static constexpr int TX = 4096 / M;                    // columns of a tile (32 KB a field)
@@ -1353,8 +1379,8 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
   static_assert(N % TX == 0, "whole tiles");
   extern __shared__ unsigned char smraw[];
   __shared__ unsigned long long bars[2];
-  const unsigned s = ((unsigned)__cvta_generic_to_shared(smraw) + 2047u) & ~2047u;
-  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(bars), bar1 = bar0 + 8;
+  const unsigned s = (smem_addr(smraw) + 2047u) & ~2047u;
+  const unsigned bar0 = smem_addr(bars), bar1 = bar0 + 8;
   const cx<float>* tw = reinterpret_cast<const cx<float>*>(twp);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // lane: column bit 3 of a pair; row h < HL in bits 0-2 and, of 16, 4 (of 8: the second pair)
@@ -1364,13 +1390,13 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
   const int kc = min((kmax3 + 2) / 3, M);
 
   if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar1) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_init(bar0);
+    mbar_init(bar1);
+    mbar_init_done();
   }
   __syncthreads();
   auto fetch = [&](int t, int f0, unsigned bar) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(3 * FB) : "memory");
+    mbar_expect(bar, 3 * FB);
     for (int b = f0 * (TX / CX); b < (f0 + 3) * (TX / CX); ++b) {
       for (int k = 0; k < M; k += Z::BOX)
         asm volatile(
