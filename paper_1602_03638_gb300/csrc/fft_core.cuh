@@ -321,6 +321,9 @@ __host__ __device__ constexpr int padt(int p) { return sizeof(T) == 8 ? p + (p >
 template <typename T>
 __host__ __device__ constexpr int padt_len(int L) { return sizeof(T) == 8 ? padt<T>(L - 1) + 1 : padded_len(L); }
 
+template <int PAD>
+__host__ __device__ constexpr int padrow(int p) { return PAD ? p + p / (PAD ? PAD : 1) : p; }
+
 constexpr int ilog2c(int x) {
   int r = 0;
   while (x > 1) { x >>= 1; ++r; }
@@ -544,7 +547,7 @@ __device__ __forceinline__ void warp_fft(const Src& src, const Work& work, const
 
 // ---------------------------------------------------------------------------
 // Several short lines per warp: G lines at s0 + g (g < G), element p of every
-// line at padded position padp(p) * LD, transformed in place. The butterflies
+// line at row padrow<PAD>(p) of LD values, transformed in place. The butterflies
 // of all G lines of a pass are spread over the lanes (virtual butterfly
 // g * NB + j), so short lines whose passes have fewer butterflies than lanes
 // still keep the warp busy. Same radix plan and twiddles as warp_fft.
@@ -555,8 +558,11 @@ struct LinesPerWarp {  // largest power of two G with G * (butterflies of pass 0
   static constexpr int value = nb0 >= 32 ? 1 : (nb0 >= 16 ? 2 : (nb0 >= 8 ? 4 : (nb0 >= 4 ? 8 : 16)));
 };
 
-template <typename T, int L, int TWN, int G, int LD, int P, int V>
-__device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __restrict__ tw, int lane) {
+// C2R: pass 0 takes the half spectrum X_k (k < klim, zeros above) of 2L real values and forms the input of the
+// L-point DFT on the way, conj Z'_k with Z'_k = (X_k + conj X_{L-k}) + i e^{+2 pi i k / 2L} (X_k - conj X_{L-k}), so that
+// the forward DFT gives the inverse one (Im X_0 ignored, X_L = 0). PAD: position p lies in row p + p / PAD (0: p).
+template <typename T, int L, int TWN, int G, int LD, int PAD, int P, int V, bool C2R>
+__device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int klim) {
   using PL = LinePlanV<L, V>;
   constexpr int R = PL::radix(P);
   constexpr int NS = PL::ns(P);
@@ -572,8 +578,23 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
     if (TOT % 32 == 0 || vj < TOT) {
       const int g = vj / NB, j = vj % NB;
       const cx<T>* ln = s0 + g;
+      if constexpr (C2R && P == 0) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[b][r] = ln[padp(j + r * NB) * LD];
+        for (int r = 0; r < R; ++r) {
+          const int k = j + r * NB;
+          cx<T> x = mk((T)0, (T)0), m = x;
+          if (k < klim) x = ln[padrow<PAD>(k) * LD];
+          if (k > 0 && L - k < klim) m = ln[padrow<PAD>(L - k) * LD];
+          const bool low = k <= L / 2;
+          const cx<T> w1 = ldro(tw + (low ? k : L - k) * (TWN / (2 * L)));
+          const cx<T> A = x + conjg(m), B = x - conjg(m);  // e^{+2 pi i k / 2L} = -w1 above the middle
+          v[b][r] = low ? conjg(A + mul_pi(cmul(conjg(w1), B))) : conjg(A - mul_pi(cmul(w1, B)));
+          if (r == 0 && j == 0) v[b][r] = mk(x.x, -x.x);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[b][r] = ln[padrow<PAD>(j + r * NB) * LD];
+      }
       if constexpr (NS > 1) {
         cx<T> w[R];
         twiddle_powers<R>(ldro(tw + (j % NS) * TWC), w);
@@ -592,17 +613,17 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
       cx<T>* ln = s0 + g;
       const int base = (j / NS) * NS * R + (j % NS);
 #pragma unroll
-      for (int r = 0; r < R; ++r) ln[padp(base + r * NS) * LD] = v[b][r];
+      for (int r = 0; r < R; ++r) ln[padrow<PAD>(base + r * NS) * LD] = v[b][r];
     }
   }
   __syncwarp();
-  if constexpr (!LAST) warp_fft_lines_pass<T, L, TWN, G, LD, P + 1, V>(s0, tw, lane);
+  if constexpr (!LAST) warp_fft_lines_pass<T, L, TWN, G, LD, PAD, P + 1, V, C2R>(s0, tw, lane, klim);
 }
 
 // Forward DFT, in place, of the G lines s0 + g (see above) by one warp (V: plan variant).
-template <typename T, int L, int TWN, int G, int LD, int V = 0>
-__device__ __forceinline__ void warp_fft_lines(cx<T>* s0, const cx<T>* __restrict__ tw, int lane) {
-  warp_fft_lines_pass<T, L, TWN, G, LD, 0, V>(s0, tw, lane);
+template <typename T, int L, int TWN, int G, int LD, int PAD, int V, bool C2R>
+__device__ __forceinline__ void warp_fft_lines(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int klim = 0) {
+  warp_fft_lines_pass<T, L, TWN, G, LD, PAD, 0, V, C2R>(s0, tw, lane, klim);
 }
 
 }  // namespace dns

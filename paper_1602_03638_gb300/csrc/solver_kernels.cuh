@@ -46,6 +46,21 @@ constexpr int odd_ld(int lines) { return (lines % 2) ? lines : lines + 1; }
 constexpr int igcd(int a, int b) { return b == 0 ? a : igcd(b, a % b); }
 constexpr int ilcm(int a, int b) { return a / igcd(a, b) * b; }
 
+// Tile layout of k_zpass for lines of M values in FP32: row p + p / PAD of LD values, LD = RES modulo 16 (a row
+// of 16 values meets every bank), chosen by counting the bank conflicts of the passes of warp_fft_lines over
+// all (PAD, RES) and the tile widths 4 to 32. Shared-memory cycles of a line's transform, PAD 16 and odd rows -> these:
+// M = 64 32 -> 16, 48 24 -> 12.4, 32 20 -> 12, 24 13.5 -> 8.1, 16 (4 x 4) 13 -> 4, 12 9.8 -> 4.5; the others keep
+// the former. Even rows are filled by 16-byte copies.
+// z-pass, with the c2r pairs formed in the first pass of the line transforms (one pass over the tile less):
+// 128^3 36.8 -> 26.6 us, 64^3 12.3 -> 10.3, 96^3 22.9 -> 20.5; a step of 128 runs of 32^3 .. 96^3 9.05 -> 8.26 ms.
+template <int M>
+struct ZLay {
+  static constexpr int PAD = M == 12 || M == 16 ? 4 : (M == 24 || M == 32 || M == 64 ? 8 : 16);
+  static constexpr int RES = M == 12 || M == 16 ? 4 : (M == 24 ? 6 : (M == 32 || M == 64 ? 2 : (M == 48 ? 11 : -1)));
+  static constexpr int ROWS = padrow<PAD>(M - 1) + 1;
+  static constexpr int ld(int lines) { return RES < 0 ? lines | 1 : lines + (RES - lines % 16 + 16) % 16; }
+};
+
 // Grid of N x NY x NZ points (x, y, z); the spectral fields hold kz < NZ/2.
 template <typename T, int N, int NY = N, int NZ = N>
 struct Geometry {
@@ -74,7 +89,9 @@ struct Geometry {
   static constexpr size_t XSMEM_ST = XPRE ? (size_t)(XST + 9 * N) * CB : XSMEM;  // XM_STAGE, XM_RHS
   // z-pass: ZTX adjacent x at fixed y, 6 fields of M values each, <= 112 KB
   // (two blocks per SM); rows narrower than one 32-byte sector may use up to 200 KB.
-  static constexpr size_t zbytes(int t) { return (size_t)padt_len<T>(M) * odd_ld(6 * t) * CB; }
+  static constexpr size_t zbytes(int t) {
+    return CB == 8 ? (size_t)ZLay<M>::ROWS * ZLay<M>::ld(6 * t) * CB : (size_t)padt_len<T>(M) * odd_ld(6 * t) * CB;
+  }
   static constexpr size_t ZBLOCK = (CB == 16 ? 113 : 112) * 1024;  // half an SM's shared memory
   static constexpr int ztx() {
     int t = cmin(16, pow2_part(N));
@@ -86,7 +103,7 @@ struct Geometry {
   // hold 32+ registers of data per lane in the warp FFT, so allow more registers.
   static constexpr int LINE_BYTES = N * CB;
   static constexpr int XMIN = CB == 16 ? (N <= 256 ? 4 : (N <= 512 ? 3 : 2)) : (LINE_BYTES > 4096 ? 2 : 4);
-  static constexpr int ZMIN = (M * CB > 4096) ? 1 : 2;
+  static constexpr int ZMIN = (M * CB > 4096) ? 1 : (CB == 8 && M <= 64 ? (M == 48 ? 3 : 4) : 2);
   static constexpr int ZLD = odd_ld(6 * ZTX);
   static constexpr size_t ZSMEM = zbytes(ZTX);
 };
@@ -218,7 +235,7 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
   constexpr int LS = G::XLS;
   constexpr size_t FS = G::FS;
   constexpr int TW = G::TW;
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
   cx<T>* U = reinterpret_cast<cx<T>*>(a.U);
@@ -596,7 +613,7 @@ __device__ __forceinline__ void ypass_tile(cx<T>* __restrict__ base, const cx<T>
   using Y = YCfg<T, N, INV, TXO>;
   constexpr int TX = Y::TX;
   constexpr int LD = Y::LD;
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the whole tile in flight at once (cp.async, no register staging); the
@@ -642,7 +659,7 @@ __global__ void __launch_bounds__(YCfg<T, N, INV, TXO, NY>::THREADS, (YCfg<T, N,
   constexpr int TX = Y::TX;
   constexpr int LD = Y::LD;
   constexpr int NT = Y::THREADS;  // warps loop over the columns
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   cx<T>* base = F + blockIdx.z * G::FS + (size_t)blockIdx.y * NY * N + blockIdx.x * TX;
@@ -706,7 +723,7 @@ __global__ void __launch_bounds__(YReg<NY>::THREADS, YReg<NY>::BLOCKS)
     k_yreg(cx<float>* __restrict__ F, const cx<float>* __restrict__ tw, size_t FS, int rd, int wr) {
   using Y = YReg<NY>;
   constexpr int E = Y::E, T = Y::T, TX = Y::TX, B = E / T;
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   cx<float>* s = reinterpret_cast<cx<float>*>(smraw);
   const int c = threadIdx.x % TX, l = threadIdx.x / TX;
   cx<float>* base = F + blockIdx.z * FS + (size_t)blockIdx.y * NY * N + blockIdx.x * TX + c;
@@ -789,7 +806,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   constexpr size_t FS = G::FS;
   constexpr int NF = MODE == ZM_CROSS ? 6 : (MODE == ZM_MAXABS ? 1 : 3), NL = NF * TX;
   constexpr int GL = cmin(FxLinesPerWarp<M, V>::value, TX);  // lines per warp
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int sK[NL];        // scale of a line
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
@@ -1000,10 +1017,10 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
   constexpr int M = G::M;
   constexpr int TW = G::TW, TS = TW / NZ;  // exp(-2 pi i k / NZ) = tw[k * TS]
   constexpr int TX = TXO > 0 ? TXO : G::ZTX;  // TXO: a tuned tile width of the small grids
-  constexpr int LD = odd_ld(6 * TX);
+  constexpr int LD = ZLay<M>::ld(6 * TX), PAD = ZLay<M>::PAD;
   constexpr size_t FS = G::FS;
   constexpr int NF = (MODE == ZM_CROSS) ? 6 : (MODE == ZM_MAXABS ? 1 : 3);
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const cx<T>* tw = reinterpret_cast<const cx<T>*>(a.tw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1016,7 +1033,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     const cx<T>* in = reinterpret_cast<const cx<T>*>(a.in);
     for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<T>) {
       const int n = e % M, x = (e / M) % TX, c = e / (M * TX);
-      cp_async<sizeof(cx<T>)>(s + padp(n) * LD + c * TX + x, in + ((size_t)(c * N + x0 + x) * NY + y) * M + n);
+      cp_async<sizeof(cx<T>)>(s + padrow<PAD>(n) * LD + c * TX + x, in + ((size_t)(c * N + x0 + x) * NY + y) * M + n);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -1032,49 +1049,44 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
         if (klim > M) klim = M;
       }
     }
-    if (klim < M) {  // the walk of the full fill (compile-time divisors), planes past klim as zeros
-      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS<T>) {
-        const int x = e % TX, k = (e / TX) % M, f = e / (TX * M);
-        if (k < klim)
-          cp_async<sizeof(cx<T>)>(s + padp(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
-        else
-          s[padp(k) * LD + f * TX + x] = mk((T)0, (T)0);
-      }
-    } else {
-      for (int e = threadIdx.x; e < NF * TX * M; e += ZP_THREADS<T>) {
-        const int x = e % TX, k = (e / TX) % M, f = e / (TX * M);
-        cp_async<sizeof(cx<T>)>(s + padp(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
-      }
+    constexpr int VX = LD % 2 == 0 && TX % 2 == 0 ? 2 : 1;  // values of a copy
+    for (int e = threadIdx.x; e < NF * TX / VX * M; e += ZP_THREADS<T>) {
+      const int x = e % (TX / VX) * VX, k = (e / (TX / VX)) % M, f = e / (TX / VX * M);
+      if (k < klim)
+        cp_async<VX * (int)sizeof(cx<T>)>(s + padrow<PAD>(k) * LD + f * TX + x, src + f * FS + ((size_t)k * NY + y) * N + x0 + x);
     }
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    // c2r pre-processing: Z'_k = (X_k + conj X_{M-k}) + i e^{+2 pi i k/N} (X_k - conj X_{M-k}),
-    // stored conjugated so that a forward DFT gives the inverse one.
     constexpr int NL = NF * TX;
-    for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<T>) {
-      const int l = e % NL, k = e / NL;
-      if (k == 0) {
-        const T r0 = s[l].x;  // Im X_0 ignored, X_M = 0
-        s[l] = mk(r0, -r0);
-      } else {
-        cx<T>* pk = s + padp(k) * LD + l;
-        cx<T>* pm = s + padp(M - k) * LD + l;
-        const cx<T> xk = *pk, xm = *pm;
-        const cx<T> wk = ldro(tw + k * TS);  // exp(-2 pi i k / NZ)
-        const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
-        *pk = conjg(A + mul_pi(cmul(conjg(wk), B)));
-        if (k != M - k) {
-          // partner M-k: e^{+2 pi i (M-k)/N} = -wk
-          const cx<T> A2 = xm + conjg(xk), B2 = xm - conjg(xk);
-          *pm = conjg(A2 - mul_pi(cmul(wk, B2)));
+    // c2r pre-processing: Z'_k = (X_k + conj X_{M-k}) + i e^{+2 pi i k/N} (X_k - conj X_{M-k}),
+    // stored conjugated so that a forward DFT gives the inverse one. The stage forms it in the first pass of the
+    // line transforms; here apart, so that the filtered stresses, small differences of products, keep their rounding.
+    if constexpr (MODE != ZM_CROSS) {
+      for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<T>) {
+        const int l = e % NL, k = e / NL;
+        if (k == 0) {
+          const T r0 = s[l].x;  // Im X_0 ignored, X_M = 0
+          s[l] = mk(r0, -r0);
+        } else {
+          cx<T>* pk = s + padrow<PAD>(k) * LD + l;
+          cx<T>* pm = s + padrow<PAD>(M - k) * LD + l;
+          const cx<T> zero = mk((T)0, (T)0), xk = k < klim ? *pk : zero, xm = M - k < klim ? *pm : zero;
+          const cx<T> wk = ldro(tw + k * TS);  // exp(-2 pi i k / NZ)
+          const cx<T> A = xk + conjg(xm), B = xk - conjg(xm);
+          *pk = conjg(A + mul_pi(cmul(conjg(wk), B)));
+          if (k != M - k) {
+            // partner M-k: e^{+2 pi i (M-k)/N} = -wk
+            const cx<T> A2 = xm + conjg(xk), B2 = xm - conjg(xk);
+            *pm = conjg(A2 - mul_pi(cmul(wk, B2)));
+          }
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;  // lines per warp
 #pragma unroll 1
-    for (int l = warp * GL; l < NL; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
+    for (int l = warp * GL; l < NL; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, MODE == ZM_CROSS>(s + l, tw, lane, klim);
     __syncthreads();
     // now conj(s) = x_{2n} + i x_{2n+1} (physical values, unnormalised c2r)
   }
@@ -1082,7 +1094,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
   if constexpr (MODE == ZM_CROSS) {
     for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<T>) {
       const int x = e % TX, n = e / TX;
-      cx<T>* p = s + padp(n) * LD + x;
+      cx<T>* p = s + padrow<PAD>(n) * LD + x;
       const cx<T> u0 = conjg(p[0 * TX]), u1 = conjg(p[1 * TX]), u2 = conjg(p[2 * TX]);
       const cx<T> w0 = conjg(p[3 * TX]), w1 = conjg(p[4 * TX]), w2 = conjg(p[5 * TX]);
       // u x omega on both packed points (real and imaginary parts)
@@ -1096,7 +1108,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
   if constexpr (MODE == ZM_PRODUCTS) {
     for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<T>) {
       const int x = e % TX, n = e / TX;
-      cx<T>* p = s + padp(n) * LD + x;
+      cx<T>* p = s + padrow<PAD>(n) * LD + x;
       const cx<T> u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];  // conjugated: the products are the same
       p[0 * TX] = pmul(u0, u0);
       p[1 * TX] = pmul(u1, u1);
@@ -1112,7 +1124,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines per column
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;
 #pragma unroll 1
-    for (int l = warp * GL; l < NP * TX; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, V>(s + l, tw, lane);
+    for (int l = warp * GL; l < NP * TX; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, false>(s + l, tw, lane);
     __syncthreads();
     // r2c post-processing: X_k = 1/2 [(Z_k + conj Z_{M-k}) - i e^{-2 pi i k/N} (Z_k - conj Z_{M-k})]
     cx<T>* dst = reinterpret_cast<cx<T>*>(MODE == ZM_LOAD ? a.U : a.W);
@@ -1130,7 +1142,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
       for (int e = threadIdx.x; e < NP * TX * kk; e += ZP_THREADS<T>) {
         const int x = e % TX, k = (e / TX) % kk, c = e / (TX * kk);
         const int l = c * TX + x;
-        const cx<T> zk = s[padp(k) * LD + l], zm = s[padp((M - k) % M) * LD + l];
+        const cx<T> zk = s[padrow<PAD>(k) * LD + l], zm = s[padrow<PAD>((M - k) % M) * LD + l];
         const cx<T> wk = ldro(tw + k * TS);
         const cx<T> A = zk + conjg(zm), B = zk - conjg(zm);
         dst[c * FS + ((size_t)k * NY + y) * N + x0 + x] = scal(A + mul_mi(cmul(wk, B)), (T)0.5);
@@ -1147,13 +1159,13 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     cx<T>* out = reinterpret_cast<cx<T>*>(a.out);
     for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<T>) {
       const int n = e % M, x = (e / M) % TX, c = e / (M * TX);
-      out[((size_t)(c * N + x0 + x) * NY + y) * M + n] = conjg(s[padp(n) * LD + c * TX + x]);
+      out[((size_t)(c * N + x0 + x) * NY + y) * M + n] = conjg(s[padrow<PAD>(n) * LD + c * TX + x]);
     }
   } else if constexpr (MODE == ZM_MAXABS) {
     double m = 0.0;
     for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<T>) {
       const int x = e % TX, n = e / TX;
-      const cx<T> v = s[padp(n) * LD + x];
+      const cx<T> v = s[padrow<PAD>(n) * LD + x];
       m = fmax(m, fmax(fabs((double)v.x), fabs((double)v.y)));
     }
     zpass_block_max<ZP_THREADS<T>>(m, a.maxbits);
@@ -1377,7 +1389,7 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
   constexpr int TX = Z::TX, CX = Z::CX, NW = Z::NW, FB = Z::FB, HL = Z::HL, V = Z::VALS, STEP = HL * Z::ROWB;
   constexpr int XT = N / TX, NT = XT * NY;  // tiles: x-tiles times y
   static_assert(N % TX == 0, "whole tiles");
-  extern __shared__ unsigned char smraw[];
+  extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned long long bars[2];
   const unsigned s = (smem_addr(smraw) + 2047u) & ~2047u;
   const unsigned bar0 = smem_addr(bars), bar1 = bar0 + 8;

@@ -1,4 +1,4 @@
-"""The FP32 z-pass of 256-, 512- and 1024-point lines inside the right-hand side, against u x omega, its projection
+"""The FP32 z-pass, small grids and 256- to 1024-point lines, inside the right-hand side, against u x omega, its projection
 and the viscous term in plain FP64 transforms, with states inside and outside the 2/3 box (planes read as zeros, and
 all planes). Tolerance: three FP32 inverse and three forward passes keep 1e-6 relative L2 (the bound of the y-pass
 test, for three); six and a product whose projection halves it at most: 4e-6."""
@@ -18,7 +18,7 @@ def _k(shape):
     return f[0][:, None, None], f[1][None, :, None], f[2][None, None, :]
 
 
-@pytest.mark.parametrize("shape", [(256, 256, 256), (512, 512, 512), (1024, 512, 256), (1024, 1024, 1024)])
+@pytest.mark.parametrize("shape", [(n, n, n) for n in (8, 12, 16, 24, 32, 48, 64, 96, 128)] + [(256, 256, 256), (512, 512, 512), (1024, 512, 256), (1024, 1024, 1024)])
 @pytest.mark.parametrize("full", [True, False])
 def test_right_hand_side(shape, full):
     nu = 1e-6  # the viscous term small beside the products
