@@ -558,11 +558,13 @@ struct LinesPerWarp {  // largest power of two G with G * (butterflies of pass 0
   static constexpr int value = nb0 >= 32 ? 1 : (nb0 >= 16 ? 2 : (nb0 >= 8 ? 4 : (nb0 >= 4 ? 8 : 16)));
 };
 
-// C2R: pass 0 takes the half spectrum X_k (k < klim, zeros above) of 2L real values and forms the input of the
+// IN, what pass 0 takes: LINES_CONJ conj of the line, the rows r0 <= p < r1 as zeros (not read);
+// LINES_C2R the half spectrum X_k (k < r0, zeros above) of 2L real values and forms the input of the
 // L-point DFT on the way, conj Z'_k with Z'_k = (X_k + conj X_{L-k}) + i e^{+2 pi i k / 2L} (X_k - conj X_{L-k}), so that
 // the forward DFT gives the inverse one (Im X_0 ignored, X_L = 0). PAD: position p lies in row p + p / PAD (0: p).
-template <typename T, int L, int TWN, int G, int LD, int PAD, int P, int V, bool C2R>
-__device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int klim) {
+enum LinesIn { LINES_PLAIN = 0, LINES_CONJ = 1, LINES_C2R = 2 };
+template <typename T, int L, int TWN, int G, int LD, int PAD, int P, int V, int IN>
+__device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int r0, int r1) {
   using PL = LinePlanV<L, V>;
   constexpr int R = PL::radix(P);
   constexpr int NS = PL::ns(P);
@@ -578,18 +580,24 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
     if (TOT % 32 == 0 || vj < TOT) {
       const int g = vj / NB, j = vj % NB;
       const cx<T>* ln = s0 + g;
-      if constexpr (C2R && P == 0) {
+      if constexpr (IN == LINES_C2R && P == 0) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int k = j + r * NB;
           cx<T> x = mk((T)0, (T)0), m = x;
-          if (k < klim) x = ln[padrow<PAD>(k) * LD];
-          if (k > 0 && L - k < klim) m = ln[padrow<PAD>(L - k) * LD];
+          if (k < r0) x = ln[padrow<PAD>(k) * LD];
+          if (k > 0 && L - k < r0) m = ln[padrow<PAD>(L - k) * LD];
           const bool low = k <= L / 2;
           const cx<T> w1 = ldro(tw + (low ? k : L - k) * (TWN / (2 * L)));
           const cx<T> A = x + conjg(m), B = x - conjg(m);  // e^{+2 pi i k / 2L} = -w1 above the middle
           v[b][r] = low ? conjg(A + mul_pi(cmul(conjg(w1), B))) : conjg(A - mul_pi(cmul(w1, B)));
           if (r == 0 && j == 0) v[b][r] = mk(x.x, -x.x);
+        }
+      } else if constexpr (IN == LINES_CONJ && P == 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int k = j + r * NB;
+          v[b][r] = conjg(k >= r0 && k < r1 ? mk((T)0, (T)0) : ln[padrow<PAD>(k) * LD]);
         }
       } else {
 #pragma unroll
@@ -617,13 +625,13 @@ __device__ __forceinline__ void warp_fft_lines_pass(cx<T>* s0, const cx<T>* __re
     }
   }
   __syncwarp();
-  if constexpr (!LAST) warp_fft_lines_pass<T, L, TWN, G, LD, PAD, P + 1, V, C2R>(s0, tw, lane, klim);
+  if constexpr (!LAST) warp_fft_lines_pass<T, L, TWN, G, LD, PAD, P + 1, V, IN>(s0, tw, lane, r0, r1);
 }
 
 // Forward DFT, in place, of the G lines s0 + g (see above) by one warp (V: plan variant).
-template <typename T, int L, int TWN, int G, int LD, int PAD, int V, bool C2R>
-__device__ __forceinline__ void warp_fft_lines(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int klim = 0) {
-  warp_fft_lines_pass<T, L, TWN, G, LD, PAD, 0, V, C2R>(s0, tw, lane, klim);
+template <typename T, int L, int TWN, int G, int LD, int PAD, int V, int IN>
+__device__ __forceinline__ void warp_fft_lines(cx<T>* s0, const cx<T>* __restrict__ tw, int lane, int r0 = 0, int r1 = 0) {
+  warp_fft_lines_pass<T, L, TWN, G, LD, PAD, 0, V, IN>(s0, tw, lane, r0, r1);
 }
 
 }  // namespace dns

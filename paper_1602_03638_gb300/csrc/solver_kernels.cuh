@@ -119,10 +119,11 @@ template <typename T, int N, int INV, int TXO = 0, int NY = N>
 struct YCfg {
   static constexpr int CB = (int)sizeof(cx<T>);
   static constexpr int TX = TXO > 0 ? TXO : cmin(((INV || CB == 16) && NY <= 512 ? 128 : 64) / CB, pow2_part(N));
-  static constexpr int THREADS = cmin(32 * TX, 256);
-  static constexpr int LD = odd_ld(TX);
-  static constexpr size_t SMEM = (size_t)padt_len<T>(NY) * LD * CB;
-  static constexpr int MINB = CB == 16 ? (NY <= 256 ? 3 : 2) : (NY <= 512 ? (INV ? 3 : 4) : 2);
+  static constexpr bool SHORT = CB == 8 && NY <= 128;  // yshort_tile
+  static constexpr int THREADS = cmin(32 * TX, SHORT ? 128 : 256);
+  static constexpr int LD = SHORT ? ZLay<NY>::ld(TX) : odd_ld(TX);
+  static constexpr size_t SMEM = (size_t)(SHORT ? ZLay<NY>::ROWS : padt_len<T>(NY)) * LD * CB;
+  static constexpr int MINB = SHORT ? 6 : (CB == 16 ? (NY <= 256 ? 3 : 2) : (NY <= 512 ? (INV ? 3 : 4) : 2));
 };
 
 __device__ __forceinline__ int kfreq(int i, int N) { return i < N / 2 ? i : i - N; }
@@ -604,6 +605,51 @@ __device__ __noinline__ void ytile_fill_kept(cx<T>* s, const cx<T>* __restrict__
   }
 }
 
+// The y tile of FP32 lines of up to 128 points (INV, PRUNE, vanish as in ypass_tile; L points, row stride N). A line has
+// fewer radix-8 butterflies than a warp has lanes, so a warp takes several columns at once (a quarter of the tile at
+// most), in the layout of the z-pass tiles (ZLay), filled and drained 16 bytes at a time. Against one column per warp
+// (8 to 12 lanes of 32 busy in the first pass at 64 and 96 points): a step of 128 runs of 32^3 .. 96^3 7.14 -> 6.02 ms
+// with the default tiles, the y-passes of 128^3 20.3 + 14.8 -> 18.0 + 13.1 us (29.0 + 13.9 -> 25.8 + 13.3 with every row).
+template <int N, int L, int TWN, int INV, int PRUNE, int TX, int NT, int V>
+__device__ __forceinline__ void yshort_tile(cx<float>* __restrict__ base, const cx<float>* __restrict__ tw, int kmax3,
+                                            bool vanish) {
+  constexpr int LD = ZLay<L>::ld(TX), PAD = ZLay<L>::PAD;
+  constexpr int G = cmin(LinesPerWarp<L, V>::value, TX >= 4 ? TX / 4 : 1);
+  constexpr int VX = LD % 2 == 0 && TX % 2 == 0 ? 2 : 1;  // values of a copy
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cx<float>* s = reinterpret_cast<cx<float>*>(smraw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // rows inside the box: [0, lo) and [lo + gap, L)
+  const int R = min((kmax3 - 1) / 3, L / 2 - 1), lo = R + 1, gap = 3 * (L / 2) < kmax3 ? 0 : L - 2 * R - 1;
+  const int skip = INV && vanish ? gap : 0;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < TX / VX * (L - skip); e += NT) {
+    const int x = e % (TX / VX) * VX, r = e / (TX / VX), y = r < lo ? r : r + skip;
+    cp_async<VX * 8>(s + padrow<PAD>(y) * LD + x, base + (size_t)y * N + x);
+  }
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+#pragma unroll 1
+  for (int c = warp * G; c < TX; c += NT / 32 * G)
+    warp_fft_lines<float, L, TWN, G, LD, PAD, V, INV ? LINES_CONJ : LINES_PLAIN>(s + c, tw, lane, lo, lo + skip);
+  __syncthreads();
+  const int drop = PRUNE ? gap : 0;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < TX / VX * (L - drop); e += NT) {
+    const int x = e % (TX / VX) * VX, r = e / (TX / VX), y = r < lo ? r : r + drop;
+    const cx<float>* q = s + padrow<PAD>(y) * LD + x;
+    cx<float>* o = base + (size_t)y * N + x;
+    if constexpr (VX == 2) {
+      float4 v = *reinterpret_cast<const float4*>(q);
+      if (INV) v = make_float4(v.x, -v.y, v.z, -v.w);
+      *reinterpret_cast<float4*>(o) = v;
+    } else {
+      *o = INV ? conjg(*q) : *q;
+    }
+  }
+}
+
 // One y tile: TX adjacent columns starting at `base` (field, kz plane and first
 // column already applied), transformed along y in place. NT: threads of the block.
 // vanish (inverse only): the rows with |ky| >= N/3 are zeros, not read.
@@ -613,6 +659,10 @@ __device__ __forceinline__ void ypass_tile(cx<T>* __restrict__ base, const cx<T>
   using Y = YCfg<T, N, INV, TXO>;
   constexpr int TX = Y::TX;
   constexpr int LD = Y::LD;
+  if constexpr (Y::SHORT) {
+    yshort_tile<N, N, N, INV, PRUNE, TX, NT, V>(base, tw, kmax3, vanish);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -663,6 +713,10 @@ __global__ void __launch_bounds__(YCfg<T, N, INV, TXO, NY>::THREADS, (YCfg<T, N,
   cx<T>* s = reinterpret_cast<cx<T>*>(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   cx<T>* base = F + blockIdx.z * G::FS + (size_t)blockIdx.y * NY * N + blockIdx.x * TX;
+  if constexpr (Y::SHORT) {
+    yshort_tile<N, NY, G::TW, INV, PRUNE, TX, NT, V>(base, tw, kmax3, INV && PR);
+    return;
+  }
   // the whole tile in flight at once (cp.async, no register staging); the
   // inverse's conjugation is applied when the first pass reads it
   if constexpr (INV && PR) {
@@ -1086,7 +1140,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     }
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;  // lines per warp
 #pragma unroll 1
-    for (int l = warp * GL; l < NL; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, MODE == ZM_CROSS>(s + l, tw, lane, klim);
+    for (int l = warp * GL; l < NL; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, MODE == ZM_CROSS ? LINES_C2R : LINES_PLAIN>(s + l, tw, lane, klim);
     __syncthreads();
     // now conj(s) = x_{2n} + i x_{2n+1} (physical values, unnormalised c2r)
   }
@@ -1124,7 +1178,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines per column
     constexpr int GL = LinesPerWarp<M, V>::value <= TX ? LinesPerWarp<M, V>::value : TX;
 #pragma unroll 1
-    for (int l = warp * GL; l < NP * TX; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, false>(s + l, tw, lane);
+    for (int l = warp * GL; l < NP * TX; l += (ZP_THREADS<T> / 32) * GL) warp_fft_lines<T, M, TW, GL, LD, PAD, V, LINES_PLAIN>(s + l, tw, lane);
     __syncthreads();
     // r2c post-processing: X_k = 1/2 [(Z_k + conj Z_{M-k}) - i e^{-2 pi i k/N} (Z_k - conj Z_{M-k})]
     cx<T>* dst = reinterpret_cast<cx<T>*>(MODE == ZM_LOAD ? a.U : a.W);
