@@ -276,9 +276,9 @@ int dns_profile_steps(dns_handle* h, int n, double* ms, int* launches, int nclas
 
 /* Measured FP64 FMA throughput of the current device in TFLOP/s (2 flops per
  * FMA): independent chains of dependent FMAs on 4 blocks of 256 threads per SM,
- * best of three CUDA-event-timed launches after one warm-up. The denominator of
- * the FP64 form's arithmetic roofline (its step is bound by FP64 arithmetic, not
- * HBM). Allocates 8 bytes; synchronous. The paper has no counterpart. */
+ * best of three CUDA-event-timed launches after one warm-up. The rate that bounded
+ * the FP64 form's transforms while they ran on the FP64 pipe (they run in 64-bit
+ * integers). Allocates 8 bytes; synchronous. The paper has no counterpart. */
 int dns_measure_fp64_peak(double* tflops);
 
 /* Bytes of device memory the handle owns. */

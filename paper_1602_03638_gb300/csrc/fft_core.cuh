@@ -233,8 +233,7 @@ __device__ __forceinline__ void dft(cx<T>* v) {
 
 // Powers w^1..w^(R-1) of one twiddle w = exp(-2 pi i k / (NS R)) loaded from the
 // FP64-generated table: one table load per butterfly instead of R-1 scattered
-// loads, the rest formed by a multiplication tree at most 4 products deep
-// (FP32 form; the FP64 form loads every power).
+// loads, the rest formed by a multiplication tree at most 4 products deep.
 template <int R, typename T>
 __device__ __forceinline__ void twiddle_powers(cx<T> w1, cx<T>* w) {
   w[1] = w1;

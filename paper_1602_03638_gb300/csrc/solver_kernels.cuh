@@ -1095,7 +1095,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
   } else {
     const cx<T>* src = reinterpret_cast<const cx<T>*>(MODE == ZM_MAXABS ? a.D : a.W);
     // a stage whose state vanishes outside the 2/3 box: the planes kz >= kc hold zeros
-    // (the y-inverse left them alone) and are filled with zeros instead of read
+    // (the y-inverse left them alone) and are taken as zeros
     int klim = M;
     if constexpr (MODE == ZM_CROSS || MODE == ZM_STORE || MODE == ZM_PRODUCTS) {
       if (rows_vanish(a)) {
@@ -1279,8 +1279,7 @@ struct HwTwL {
 // Half-warp 512-point FFT for the N = 1024 z-pass (FP32). Lane h of a half-warp
 // holds v[m] = x[h + 16 m], m < 32. With k = k1 + 32 k2: a 32-point DFT over m in
 // each lane gives Y[h][k1]; after the twiddle exp(-2 pi i h k1 / 512) one
-// shared-memory exchange gives lane h' the
-// 16-point columns k1 = h' and h' + 16, whose DFTs over h leave
+// shared-memory exchange gives lane h' the 16-point columns k1 = h' and h' + 16, whose DFTs over h leave
 // v[j] = X[h' + 16 j] in the lane: the input layout again.
 // ---------------------------------------------------------------------------
 struct HwTw32 {
