@@ -80,10 +80,10 @@ struct Geometry {
   static constexpr bool XWIDE = (size_t)((6 * XLS + 1) / 2 * 2 + 9 * N) * CB <= 64 * 1024;
   static constexpr int XST = ((XWIDE ? 6 : 3) * XLS + 1) / 2 * 2;  // 16-byte aligned start of the state rows
   static constexpr bool XPRE = CB == 8 && (size_t)(XST + 9 * N) * CB <= 100 * 1024;
-  // Rows of 2 KB and more arrive by bulk copies instead (one thread issues them; no asynchronous copy per value:
+  // Rows of 1 KB and more arrive by bulk copies instead (one thread issues them; no asynchronous copy per value:
   // those took a quarter of the shared-memory pipe's cycles): x-stage 512^3 816 -> 689 us (its bytes: 670 at the
-  // copy bandwidth), 1024^3 8.02 -> 7.19 ms, 1024 x 512 x 256 1022 -> 913 us, 256^3 103 -> 94 us; 128^3, whose
-  // rows are 1 KB, the same within the noise.
+  // copy bandwidth), 1024^3 8.02 -> 7.19 ms, 1024 x 512 x 256 1022 -> 913 us, 256^3 103 -> 94 us, 128^3
+  // with every row 37.0 -> 36.0 us; shorter rows keep the copies per value (not measured).
   static constexpr bool XBULK = XPRE && N >= 128;
   static constexpr size_t XSMEM = (size_t)6 * XLS * CB;
   static constexpr size_t XSMEM_ST = XPRE ? (size_t)(XST + 9 * N) * CB : XSMEM;  // XM_STAGE, XM_RHS
