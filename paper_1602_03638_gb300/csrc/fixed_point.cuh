@@ -45,6 +45,15 @@ __device__ __forceinline__ ll madw(int a, int b, ll c) {
 // upper word of a when its low word is read as a signed number
 __device__ __forceinline__ int fx_hi(ll a) { return (int)(a >> 32) + (int)((unsigned)a >> 31); }
 
+// upper word of |a| (of ~a where a is negative)
+__device__ __forceinline__ unsigned fx_upper(ll a) {
+  const int hi = (int)(a >> 32);
+  return (unsigned)(hi ^ (hi >> 31));
+}
+// a 2^n (floor), |n| <= 63
+__device__ __forceinline__ ll fx_shift(ll a, int n) { return (a << max(n, 0)) >> max(-n, 0); }
+__device__ __forceinline__ fx fx_shift(fx a, int n) { return mk(fx_shift(a.x, n), fx_shift(a.y, n)); }
+
 // (t >> 32) + c: a product by 1 takes the odd register of the pair t as it is
 __device__ __forceinline__ ll fx_add_up(ll t, ll c) { return madw((int)(t >> 32), 1, c); }
 // 4 p with the top two bits of t's low word below
@@ -324,10 +333,11 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
 // The passes of warp_fft_lines on lines of fixed-point values, in place. FROM: what pass 0 reads,
 // fixed point (FX_IN), fixed point of line g to be shifted left by sh[g] bits (FX_SHIFT; right where
 // negative) or doubles to be taken to scale sh[g] (FX_DOUBLE).
+// MAG: the upper words of the results' magnitudes are or'ed into mag[g] (cleared before): the top bit of the largest.
 enum FxFrom { FX_IN = 0, FX_SHIFT = 1, FX_DOUBLE = 2 };
-template <int L, int TWN, int G, int LD, int P, int V, int FROM>
+template <int L, int TWN, int G, int LD, int P, int V, int FROM, bool MAG = false>
 __device__ __forceinline__ void warp_fft_fx_lines(cx<double>* s0, const cx<double>* __restrict__ tw, int lane,
-                                                  const int* sh) {
+                                                  const int* sh, unsigned* mag = nullptr) {
   using PL = FxPlan<L, V>;
   constexpr int R = PL::radix(P), NS = PL::ns(P), NB = L / R, TOT = G * NB, BPL = (TOT + 31) / 32;
   constexpr bool LAST = (P + 1 == PL::npass);
@@ -346,9 +356,9 @@ __device__ __forceinline__ void warp_fft_fx_lines(cx<double>* s0, const cx<doubl
         else v[b][r] = *reinterpret_cast<const fx*>(q);
       }
       if constexpr (P == 0 && FROM == FX_SHIFT) {
-        const int l = max(sh[g], 0), rr = max(-sh[g], 0);
+        const int n = sh[g];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[b][r] = mk((v[b][r].x << l) >> rr, (v[b][r].y << l) >> rr);
+        for (int r = 0; r < R; ++r) v[b][r] = fx_shift(v[b][r], n);
       }
       if constexpr (NS > 1) {
         const int kc = (j % NS) * TWC;
@@ -369,9 +379,26 @@ __device__ __forceinline__ void warp_fft_fx_lines(cx<double>* s0, const cx<doubl
 #pragma unroll
       for (int r = 0; r < R; ++r) *reinterpret_cast<fx*>(ln + padt<double>(base + r * NS) * LD) = v[b][r];
     }
+    if constexpr (LAST && MAG) {
+      unsigned m = 0;
+      if (TOT % 32 == 0 || vj < TOT) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) m |= fx_upper(v[b][r].x) | fx_upper(v[b][r].y);
+      }
+      if constexpr (NB % 32 == 0) {  // the warp's lanes are on one line
+        m = __reduce_or_sync(0xffffffffu, m);
+        if (lane == 0) mag[vj / NB] |= m;
+      } else if constexpr (32 % NB == 0) {  // NB adjacent lanes are
+#pragma unroll
+        for (int o = NB / 2; o > 0; o >>= 1) m |= __shfl_xor_sync(0xffffffffu, m, o);
+        if (vj % NB == 0 && vj < TOT) mag[vj / NB] |= m;
+      } else {
+        if (vj < TOT) atomicOr(mag + vj / NB, m);
+      }
+    }
   }
   __syncwarp();
-  if constexpr (!LAST) warp_fft_fx_lines<L, TWN, G, LD, P + 1, V, FROM>(s0, tw, lane, sh);
+  if constexpr (!LAST) warp_fft_fx_lines<L, TWN, G, LD, P + 1, V, FROM, MAG>(s0, tw, lane, sh, mag);
 }
 
 }  // namespace dns

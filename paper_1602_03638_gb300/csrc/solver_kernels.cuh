@@ -841,13 +841,17 @@ __device__ __forceinline__ void zpass_block_max(double m, unsigned long long* bi
 
 // ---------------------------------------------------------------------------
 // z-pass of the FP64 form, on fixed point (fixed_point.cuh) from the tile's doubles to the
-// results. Every line has its own scale, except that the three components of u (of omega) of a
-// column share the largest of theirs, so that the products of one component can be added.
+// results. Every line has its own scale.
 //   c2r   z'/4 from the pair (X_k, X_{M-k}) (L1 of z' is at most four times that of X): physical
 //         values x = v 2^(K - 1083), |v| <= 2^62
-//   u x w products of the v / 2 cut at 2^-62: p = P 2^(Ku + Kw - 2102), |P| <= 2^61; then shifted by
-//         the L1 of the line of products, so that its DFT has 62 bits again
-//   r2c   V = X_k / 2 (quartered post-processing of the pair): X_k = V 2^(Ku + Kw + 1 - sh - 2102)
+//   u x w a line's values are shifted so that the largest has 61 bits (the L1 of a broad spectrum is many
+//         times the values): x = a 2^(E - 1083). The products a b, cut at 2^-62, have the scale E_u + E_w; of
+//         the two in a component of u x w the smaller scale's u is shifted down to the larger one e, so
+//         that they can be subtracted: p = P 2^(e - 2104), |P| <= 2^61. With one scale for the three components
+//         (and for omega's) a weak third component lost its bits: 1e-6 beside 1 kept 1e-11, 1e-20 nothing, and
+//         with the L1 scale a white field of 512 points 2.6e-15 (FP64 products 1.0e-15).
+//         Then the line of products is shifted by its L1, so that its DFT has 62 bits again
+//   r2c   V = X_k / 2 (quartered post-processing of the pair): X_k = V 2^(e + 1 - sh - 2104)
 // ---------------------------------------------------------------------------
 template <int N, int MODE, int TXO, int NY, int NZ, int V>
 __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, const int by) {
@@ -864,7 +868,10 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   __shared__ int sK[NL];        // scale of a line
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
-  __shared__ unsigned sQ[NP * TX];
+  __shared__ unsigned sQ[NP * TX];  // L1 of a line of products, then its shift
+  __shared__ unsigned sM[NL];       // top bit of a line's physical values
+  __shared__ int sE[NP * TX];       // scale of a line of products; then what fx_to takes for it
+  __shared__ int sT[NP * 2 * TX];   // shifts of the two u (ZM_CROSS) of a line of products
   cd* s = reinterpret_cast<cd*>(smraw);
   fx* sf = reinterpret_cast<fx*>(smraw);
   const cd* tw = reinterpret_cast<const cd*>(a.tw);
@@ -890,6 +897,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   }
   constexpr bool PROD = MODE == ZM_CROSS || MODE == ZM_PRODUCTS;
   if (PROD && threadIdx.x < NP * TX) sQ[threadIdx.x] = 0;
+  if (PROD && threadIdx.x < NL) sM[threadIdx.x] = 0;
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
@@ -918,17 +926,11 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     }
   }
   __syncthreads();
-  // the scale of the three components of u (g = 0) or omega (g = 1) of column x
-  auto scale3 = [&](int g, int x) {
-    const int* k = sK + 3 * g * TX + x;
-    return max(k[0], max(k[TX], k[2 * TX]));
-  };
-
   if constexpr (MODE != ZM_LOAD) {
     // c2r pre-processing (zpass_body), quartered
     for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<double>) {
       const int l = e % NL, k = e / NL;
-      const int K = PROD ? scale3(l / (3 * TX), l % TX) : sK[l];
+      const int K = sK[l];
       if (k == 0) {
         const ll r0 = (fx_from(s[l].x, K) + 2) >> 2;  // Im X_0 ignored, X_M = 0
         sf[l] = mk(r0, -r0);
@@ -947,13 +949,29 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     __syncthreads();
 #pragma unroll 1
     for (int l = warp * GL; l < NL; l += (ZP_THREADS<double> / 32) * GL)
-      warp_fft_fx_lines<M, TW, GL, LD, 0, V, FX_IN>(s + l, tw, lane, nullptr);
+      warp_fft_fx_lines<M, TW, GL, LD, 0, V, FX_IN, PROD>(s + l, tw, lane, nullptr, sM + l);
     __syncthreads();
     // now conj(s) = x_{2n} + i x_{2n+1} (physical values, unnormalised c2r)
   }
 
   if constexpr (PROD) {
-    auto half = [](fx v) { return mk(v.x >> 1, (-v.y) >> 1); };
+    // the shift that leaves 61 bits of line l, and its scale after it
+    auto up = [&](int l) { return __clz(sM[l]) - 3; };
+    auto scale = [&](int l) { return sK[l] - up(l); };
+    if (threadIdx.x < NP * TX) {
+      const int c = threadIdx.x / TX, x = threadIdx.x % TX;
+      if constexpr (MODE == ZM_CROSS) {
+        const int i = (c + 1) % 3 * TX + x, j = (c + 2) % 3 * TX + x;  // u_i w_j - u_j w_i
+        const int e1 = scale(i) + scale(3 * TX + j), e2 = scale(j) + scale(3 * TX + i), e = max(e1, e2);
+        sE[threadIdx.x] = e;
+        sT[2 * threadIdx.x] = max(up(i) - (e - e1), -63);
+        sT[2 * threadIdx.x + 1] = max(up(j) - (e - e2), -63);
+      } else {
+        const int i = c < 3 ? c : (c == 5 ? 1 : 0), j = c < 3 ? c : (c == 3 ? 1 : 2);
+        sE[threadIdx.x] = scale(i * TX + x) + scale(j * TX + x);
+      }
+    }
+    __syncthreads();
     auto mag = [](fx p) { return ((unsigned)abs((int)(p.x >> 32)) >> 9) + ((unsigned)abs((int)(p.y >> 32)) >> 9) + 2u; };
     // a warp takes 32 / XW adjacent positions of XW columns: whole warps on one column where the line
     // is long enough (no bank conflicts along a line)
@@ -964,15 +982,25 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
       unsigned q[NP] = {};
       if (M % CH == 0 || n < M) {
         fx* p = sf + padt<double>(n) * LD + x;
-        const fx u0 = half(p[0 * TX]), u1 = half(p[1 * TX]), u2 = half(p[2 * TX]);
         fx r[NP];
+        // u and omega are conjugated: in their products the signs of the odd points cancel
         if constexpr (MODE == ZM_CROSS) {
-          const fx w0 = half(p[3 * TX]), w1 = half(p[4 * TX]), w2 = half(p[5 * TX]);
+          const fx u0 = p[0 * TX], u1 = p[1 * TX], u2 = p[2 * TX];
+          const fx w0 = fx_shift(p[3 * TX], up(3 * TX + x)), w1 = fx_shift(p[4 * TX], up(4 * TX + x)),
+                   w2 = fx_shift(p[5 * TX], up(5 * TX + x));
           // u x omega on both packed points (real and imaginary parts)
-          r[0] = mk(fx_cross(u1.x, w2.x, u2.x, w1.x), fx_cross(u1.y, w2.y, u2.y, w1.y));
-          r[1] = mk(fx_cross(u2.x, w0.x, u0.x, w2.x), fx_cross(u2.y, w0.y, u0.y, w2.y));
-          r[2] = mk(fx_cross(u0.x, w1.x, u1.x, w0.x), fx_cross(u0.y, w1.y, u1.y, w0.y));
+          auto cross = [&](int c, fx a, fx wb, fx b, fx wa) {
+            const int* t = sT + 2 * (c * TX + x);
+            a = fx_shift(a, t[0]);
+            b = fx_shift(b, t[1]);
+            return mk(fx_cross(a.x, wb.x, b.x, wa.x), fx_cross(a.y, wb.y, b.y, wa.y));
+          };
+          r[0] = cross(0, u1, w2, u2, w1);
+          r[1] = cross(1, u2, w0, u0, w2);
+          r[2] = cross(2, u0, w1, u1, w0);
         } else {
+          const fx u0 = fx_shift(p[0 * TX], up(x)), u1 = fx_shift(p[1 * TX], up(TX + x)),
+                   u2 = fx_shift(p[2 * TX], up(2 * TX + x));
           r[0] = mk(fx_prod(u0.x, u0.x), fx_prod(u0.y, u0.y));
           r[1] = mk(fx_prod(u1.x, u1.x), fx_prod(u1.y, u1.y));
           r[2] = mk(fx_prod(u2.x, u2.x), fx_prod(u2.y, u2.y));
@@ -999,7 +1027,11 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
       }
     }
     __syncthreads();
-    if (threadIdx.x < NP * TX) sQ[threadIdx.x] = (unsigned)(__clz(sQ[threadIdx.x]) - 11);
+    if (threadIdx.x < NP * TX) {
+      const int sh = __clz(sQ[threadIdx.x]) - 11;
+      sQ[threadIdx.x] = (unsigned)sh;
+      sE[threadIdx.x] = max(sE[threadIdx.x] - sh - 1018, 64);
+    }
     __syncthreads();
   }
 
@@ -1024,7 +1056,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
       int B;
       unsigned nan;
       if constexpr (PROD) {
-        B = max(scale3(0, x) + scale3(NF / 6, x) - (int)sQ[l] - 1016, 64);
+        B = sE[l];
         nan = 0;
 #pragma unroll
         for (int f = 0; f < NF; ++f) nan |= sN[f * TX + x];
