@@ -24,7 +24,8 @@
 // 2^-53 |x|_2 up to the longest line; most where all |x_j| are equal, many bits below where few modes
 // carry the line. Measured against extended precision (c2r and r2c of white, Gaussian and power-law
 // fields, 16^3 .. 512^3): 0.5 - 2.3e-16 relative, where FP64 butterflies gave 1.1 - 5.8e-16.
-// A line with a NaN or an infinity gives NaN everywhere; lines below 2^-895 are taken as zero.
+// A line with a NaN or an infinity gives NaN everywhere. Lines whose largest value is below 2^-831 or above
+// 2^960 are taken times a power of two (fx_lift), so that the whole range of a double is kept, subnormal numbers too.
 //
 // Numbers here are cx<long long>. The low word of a factor is signed (w = hi 2^32 + lo, |lo| < 2^31).
 #pragma once
@@ -157,11 +158,24 @@ struct FxScale {
   int K;         // biased exponent: L1 <= 2^(K - 1023)
   unsigned nan;  // 0x7ff80000 if the line holds a NaN or an infinity, else 0
 };
+// The power of two that brings a line of largest magnitude word `mag` to where fx_from takes every element in
+// full (exponents of 192 and more; it reads an exponent of 0 as zero) and fx_to has room above: 0 for
+// all but extreme lines, whose values are multiplied by fx_pow2 of it, exactly.
+__device__ __forceinline__ bool fx_extreme(unsigned mag) { return mag - (192u << 20) >= (1791u << 20); }
+// low: a lower word is not zero (asked for where mag is)
+__device__ __forceinline__ int fx_lift(unsigned mag, bool low) {
+  return mag < (192u << 20) ? (mag || low ? 600 : 0) : (fx_extreme(mag) && mag < 0x7ff00000u ? -64 : 0);
+}
+__device__ __forceinline__ double fx_pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
+// the largest magnitude word after that (at most)
+__device__ __forceinline__ unsigned fx_lifted(unsigned mag, int lift) {
+  return lift ? max(mag, 1u << 20) + ((unsigned)lift << 20) : mag;
+}
 // from the line's largest magnitude word and the sum of its shares
 __device__ __forceinline__ FxScale fx_scale(unsigned mag, unsigned shares) {
   FxScale s;
   s.K = max((int)(mag >> 20) + 20 - __clz(shares), 128);
-  s.nan = s.K > 2040 ? 0x7ff80000u : 0u;  // not finite, or about to overflow
+  s.nan = mag >= 0x7ff00000u ? 0x7ff80000u : 0u;
   return s;
 }
 
@@ -175,9 +189,9 @@ __device__ __forceinline__ ll fx_from(double d, int K) {
   return ((m ^ sm) + 1) >> 1;  // halves away from zero: (m + 1) / 2 or floor(-m / 2)
 }
 __device__ __forceinline__ fx fx_from(cx<double> v, int K) { return mk(fx_from(v.x, K), fx_from(v.y, K)); }
-// the double v 2^(B - 1085), B >= 64 (B = K: a value of a line of scale K); of a negative v the
+// the double v 2^(B - 1085), 64 <= B <= 2040 (B = K: a value of a line of scale K); of a negative v the
 // magnitude is taken as ~v, a last bit (2^-62 L1) too small
-__device__ __forceinline__ double fx_to(ll v, int B, unsigned nan) {
+__device__ __forceinline__ double fx_bits(ll v, int B, unsigned nan) {
   const int s = (int)(v >> 32) >> 31;
   const unsigned ah = (unsigned)((int)(v >> 32) ^ s), al = (unsigned)((int)v ^ s);
   const unsigned top = ah ? ah : al;
@@ -186,7 +200,18 @@ __device__ __forceinline__ double fx_to(ll v, int B, unsigned nan) {
   const unsigned e = top ? (unsigned)(B - 1 - sh) : 0u;                                         // (a carry raises it)
   return __hiloint2double((int)(((unsigned)(q >> 32) + (e << 20)) | (s & 0x80000000u) | nan), (int)(unsigned)q);
 }
-__device__ __forceinline__ cx<double> fx_to(fx v, int B, unsigned nan) { return mk(fx_to(v.x, B, nan), fx_to(v.y, B, nan)); }
+__device__ __forceinline__ cx<double> fx_bits(fx v, int B, unsigned nan) { return mk(fx_bits(v.x, B, nan), fx_bits(v.y, B, nan)); }
+// any other B: the conversion at FX_MID and then fx_rescale, which underflows gradually and overflows to infinity
+constexpr int FX_MID = 1000;
+__device__ __forceinline__ bool fx_far(int B) { return (unsigned)(B - 64) > 1976u; }
+__device__ __forceinline__ cx<double> fx_rescale(cx<double> d, int B) {  // two steps, neither of which leaves the range
+  const int n = max(min(B - FX_MID, 2040), -2040);
+  return scal(scal(d, fx_pow2(n / 2)), fx_pow2(n - n / 2));
+}
+__device__ __forceinline__ cx<double> fx_to(fx v, int B, unsigned nan) {
+  if (fx_far(B)) return fx_rescale(fx_bits(v, FX_MID, nan), B);
+  return fx_bits(v, B, nan);
+}
 
 // ---- radix schedules -----------------------------------------------------------------------
 // A butterfly holds four registers per value: radix 8 passes, 4 x 4 or 4 for what remains of the power of
@@ -259,6 +284,30 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
       }
     }
     m = __reduce_max_sync(0xffffffffu, m);
+    int lift = 0;
+    if (fx_extreme(m)) {
+      unsigned low = 0;
+      if (m == 0) {
+#pragma unroll 1
+        for (int p = lane; p < L; p += 32) {
+          const cx<double> x = src.load(src.at(p));
+          low |= (unsigned)__double2loint(x.x) | (unsigned)__double2loint(x.y);
+        }
+      }
+      lift = fx_lift(m, __any_sync(0xffffffffu, low != 0));
+      if (KEEP && lift) {
+#pragma unroll
+        for (int b = 0; b < BPL; ++b) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) d[b][r] = scal(d[b][r], fx_pow2(lift));
+        }
+      }
+    }
+    auto again = [&](int j, int r) -> cx<double> {  // (KEEP: unused)
+      const cx<double> x = rd(j, r);
+      return lift ? scal(x, fx_pow2(lift)) : x;
+    };
+    m = fx_lifted(m, lift);
     const int top = fx_top(m);
     float s = 0.f;
 #pragma unroll
@@ -268,7 +317,7 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
       for (int r = 0; r < R; ++r) {
         cx<double> x;
         if constexpr (KEEP) x = d[b][r];
-        else x = (NB % 32 == 0 || j < NB) ? rd(j, r) : mk(0.0, 0.0);
+        else x = (NB % 32 == 0 || j < NB) ? again(j, r) : mk(0.0, 0.0);
         s += fx_rel(x.x, top) + fx_rel(x.y, top);
       }
     }
@@ -280,11 +329,12 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if constexpr (KEEP) v[b][r] = fx_from(d[b][r], sc.K);
-          else v[b][r] = fx_from(rd(j, r), sc.K);
+          else v[b][r] = fx_from(again(j, r), sc.K);
         }
         fx_dft<R>(v[b]);
       }
     }
+    sc.K -= lift;  // of the values as they were
   } else {
 #pragma unroll
     for (int b = 0; b < BPL; ++b) {
@@ -305,6 +355,7 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
     }
   }
   __syncwarp();
+  const bool far = LAST && fx_far(sc.K + E);
 #pragma unroll
   for (int b = 0; b < BPL; ++b) {
     const int j = lane + 32 * b;
@@ -313,7 +364,7 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if constexpr (LAST) {
-          const cx<double> o = fx_to(v[b][r], sc.K + E, sc.nan);
+          const cx<double> o = fx_bits(v[b][r], far ? FX_MID : sc.K + E, sc.nan);
           if constexpr (FAST) dst.store(dst.at(base) + Dst::off(r * NS), base + r * NS, o);
           else dst.store(dst.at(base + r * NS), base + r * NS, o);
         } else {
@@ -326,6 +377,11 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
     }
   }
   __syncwarp();
+  if (far) {  // apart from the stores, so that those stay short (in line with them 2 us more a small x-stage)
+#pragma unroll 1
+    for (int p = lane; p < L; p += 32) *dst.at(p) = fx_rescale(*dst.at(p), sc.K + E);
+    __syncwarp();
+  }
   if constexpr (!LAST) warp_fft_fx_pass<L, TWN, P + 1, V, E>(src, work, dst, tw, lane, sc);
 }
 

@@ -865,7 +865,8 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   constexpr int NF = MODE == ZM_CROSS ? 6 : (MODE == ZM_MAXABS ? 1 : 3), NL = NF * TX;
   constexpr int GL = cmin(FxLinesPerWarp<M, V>::value, TX);  // lines per warp
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int sK[NL];        // scale of a line
+  __shared__ int sK[NL];        // scale of a line as the tile holds it
+  __shared__ int sL[NL];        // power of two that it was multiplied by (fx_lift)
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
   __shared__ unsigned sQ[NP * TX];  // L1 of a line of products, then its shift
@@ -905,11 +906,27 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   constexpr int SUB = M >= 64 ? 8 : (M >= 16 ? 4 : 2);
   for (int l0 = warp * (32 / SUB); l0 < NL; l0 += (ZP_THREADS<double> / 32) * (32 / SUB)) {
     const int l = l0 + lane / SUB, q = lane % SUB;
-    const cd* ln = s + (l < NL ? l : NL - 1);
+    cd* ln = s + (l < NL ? l : NL - 1);
     unsigned m = 0;
     for (int k = q; k < klim; k += SUB) m = max(m, fx_mag(ln[padt<double>(k) * LD]));
 #pragma unroll
     for (int o = SUB / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int lift = 0;
+    if (__any_sync(0xffffffffu, fx_extreme(m))) {
+      unsigned low = 0;
+      if (m == 0) {
+        for (int k = q; k < klim; k += SUB) {
+          const cd v = ln[padt<double>(k) * LD];
+          low |= (unsigned)__double2loint(v.x) | (unsigned)__double2loint(v.y);
+        }
+      }
+#pragma unroll
+      for (int o = SUB / 2; o > 0; o >>= 1) low |= __shfl_xor_sync(0xffffffffu, low, o);
+      lift = fx_lift(m, low != 0);
+      if (lift && l < NL)
+        for (int k = q; k < klim; k += SUB) ln[padt<double>(k) * LD] = scal(ln[padt<double>(k) * LD], fx_pow2(lift));
+      m = fx_lifted(m, lift);
+    }
     const int top = fx_top(m);
     float t = 0.f;
     for (int k = q; k < klim; k += SUB) {
@@ -922,6 +939,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     if (q == 0 && l < NL) {
       const FxScale sc = fx_scale(m, sh);
       sK[l] = sc.K;
+      sL[l] = lift;
       sN[l] = sc.nan;
     }
   }
@@ -957,7 +975,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   if constexpr (PROD) {
     // the shift that leaves 61 bits of line l, and its scale after it
     auto up = [&](int l) { return __clz(sM[l]) - 3; };
-    auto scale = [&](int l) { return sK[l] - up(l); };
+    auto scale = [&](int l) { return sK[l] - sL[l] - up(l); };
     if (threadIdx.x < NP * TX) {
       const int c = threadIdx.x / TX, x = threadIdx.x % TX;
       if constexpr (MODE == ZM_CROSS) {
@@ -1030,7 +1048,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     if (threadIdx.x < NP * TX) {
       const int sh = __clz(sQ[threadIdx.x]) - 11;
       sQ[threadIdx.x] = (unsigned)sh;
-      sE[threadIdx.x] = max(sE[threadIdx.x] - sh - 1018, 64);
+      sE[threadIdx.x] -= sh + 1018;
     }
     __syncthreads();
   }
@@ -1060,9 +1078,8 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
         nan = 0;
 #pragma unroll
         for (int f = 0; f < NF; ++f) nan |= sN[f * TX + x];
-        if (B > 2040) nan = 0x7ff80000u;
       } else {
-        B = sK[l] + 1;
+        B = sK[l] - sL[l] + 1;
         nan = sN[l];
       }
       dst[(l / TX) * FS + ((size_t)k * NY + y) * N + x0 + x] = fx_to(X, B, nan);
@@ -1072,13 +1089,13 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     for (int e = threadIdx.x; e < 3 * TX * M; e += ZP_THREADS<double>) {
       const int n = e % M, x = (e / M) % TX, c = e / (M * TX), l = c * TX + x;
       out[((size_t)(c * N + x0 + x) * NY + y) * M + n] =
-          fx_to(conjg(sf[padt<double>(n) * LD + l]), sK[l] + 2, sN[l]);
+          fx_to(conjg(sf[padt<double>(n) * LD + l]), sK[l] - sL[l] + 2, sN[l]);
     }
   } else if constexpr (MODE == ZM_MAXABS) {
     double m = 0.0;
     for (int e = threadIdx.x; e < TX * M; e += ZP_THREADS<double>) {
       const int l = e % TX;
-      const cd v = fx_to(sf[padt<double>(e / TX) * LD + l], sK[l] + 2, sN[l]);
+      const cd v = fx_to(sf[padt<double>(e / TX) * LD + l], sK[l] - sL[l] + 2, sN[l]);
       m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
     }
     zpass_block_max<ZP_THREADS<double>>(m, a.maxbits);
