@@ -1481,12 +1481,15 @@ __device__ __forceinline__ void zt_fft(cx<float> (&v)[ZTma<M>::VALS], unsigned l
   }
 }
 
-// in: W as (x, y, kz, field), kz bounded by the planes that hold values; out: by the planes kept
+// in: W as (x, y, kz, field), kz bounded by the planes that hold values; out: by the planes kept. A block whose copies
+// do not arrive within the limit starts no others, waits for those under way once more and fills the products of
+// the tiles that are left with NaN, which the checks of the state report.
 template <int N, int NY, int NZ>
 __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
-    k_ztma(int kmax3, const void* __restrict__ twp, const __grid_constant__ CUtensorMap in,
+    k_ztma(int kmax3, const void* __restrict__ twp, cx<float>* __restrict__ W, const __grid_constant__ CUtensorMap in,
            const __grid_constant__ CUtensorMap out) {
   constexpr int M = NZ / 2;
+  constexpr size_t FS = Geometry<float, N, NY, NZ>::FS;
   using Z = ZTma<M>;
   constexpr int TX = Z::TX, CX = Z::CX, NW = Z::NW, FB = Z::FB, HL = Z::HL, V = Z::VALS, STEP = HL * Z::ROWB;
   constexpr int XT = N / TX, NT = XT * NY;  // tiles: x-tiles times y
@@ -1583,16 +1586,15 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
     fetch(t, 3, bar0);
     fetch(t, 0, bar1);
   }
-  bool ok = true;  // a copy that does not arrive leaves NaN, which the checks of the state report
   unsigned phase = 0;
 #pragma unroll 1
   for (; t < NT; t += gridDim.x, phase ^= 1) {
     const int tn = t + gridDim.x;
-    ok = ok && mbar_wait(bar0, phase);  // omega fields of tile t
+    bool ok = mbar_wait(bar0, phase);  // omega fields of tile t
     c2r_lines(3);
-    ok = ok && mbar_wait(bar1, phase);  // u fields of tile t
+    ok = mbar_wait(bar1, phase) && ok;  // u fields of tile t
     c2r_lines(0);
-    __syncthreads();
+    if (!__syncthreads_and(ok)) break;
     // u x omega at every point, into the u lines: all fields are permuted alike
     for (int i = threadIdx.x; i < FB / 16; i += 32 * NW) {
       const unsigned p = s + i * 16;
@@ -1610,7 +1612,6 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
     if (threadIdx.x == 0 && tn < NT) fetch(tn, 3, bar0);  // the omega lines are free
     // r2c of the 3 TX product lines; X_k (k < kc) back into the line
     {
-      const float half = ok ? 0.5f : __int_as_float(0x7fffffff);
       cx<float> v[V];
 #pragma unroll 1
       for (int l = Z::GL * w; l < 3 * TX; l += Z::GL * NW) {
@@ -1627,7 +1628,7 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
           zo.y = __shfl_sync(0xffffffffu, v[V - 1 - m].y, partner);
           if (h == 0) zo = v[(V - m) & (V - 1)];
           const cx<float> A = v[m] + conjg(zo), B = v[m] - conjg(zo);
-          if (h + HL * m < kc) sts(pa + m * STEP, scal(A + mul_mi(cmul(ht.wk(m), B)), half));
+          if (h + HL * m < kc) sts(pa + m * STEP, scal(A + mul_mi(cmul(ht.wk(m), B)), 0.5f));
         }
       }
     }
@@ -1644,6 +1645,19 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the u lines have been read out
       if (tn < NT) fetch(tn, 0, bar1);
+    }
+  }
+  if (t < NT) {  // gave up at tile t: both of its copies were started, no later one
+    mbar_wait(bar0, phase);
+    mbar_wait(bar1, phase);
+    const float nan = __int_as_float(0x7fffffff);
+#pragma unroll 1
+    for (; t < NT; t += gridDim.x) {
+#pragma unroll 1
+      for (int e = threadIdx.x; e < 3 * kc * TX; e += 32 * NW) {
+        const int x = e % TX, k = (e / TX) % kc, f = e / (TX * kc);
+        W[f * FS + ((size_t)k * NY + t / XT) * N + (t % XT) * TX + x] = mk(nan, nan);
+      }
     }
   }
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -1953,7 +1967,7 @@ struct SolverImpl {
       cudaError_t e = ztma_map<N, NY, NZ>(&in, a.W, a.prune >= PRUNE_ROWS ? kc : M, 6);
       if (e == cudaSuccess) e = ztma_map<N, NY, NZ>(&out, a.W, kc, 3);
       if (e != cudaSuccess) return e;
-      k_ztma<N, NY, NZ><<<num_sms(), 32 * ZTma<M>::NW, ZTma<M>::SMEM, st>>>(k3z(a), a.tw, in, out);
+      k_ztma<N, NY, NZ><<<num_sms(), 32 * ZTma<M>::NW, ZTma<M>::SMEM, st>>>(k3z(a), a.tw, reinterpret_cast<cx<float>*>(a.W), in, out);
     } else if constexpr (!ISO) {
       z_go<0>(a, st);
     } else {
