@@ -322,8 +322,14 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
         line_fft<T, N, TW, V>(SRow<T>{s + (warp * LS + 1) / 2 * 2}, line, line, tw, lane);
       }
       ok = mbar_wait(bs, 0) && ok;
-      if (!ok) nu = (T)__int_as_float(0x7fffffff);  // a copy that does not arrive: NaN, which the checks of the state report
-      __syncthreads();
+      // copies that do not arrive within the limit: waited for once more, since they must not land after the block has
+      // gone, and the whole row becomes NaN, which the checks of the state report
+      if (!__syncthreads_and(ok)) {
+        nu = (T)__int_as_float(0x7fffffff);
+        if (row_kept) mbar_wait(bw, 0);
+        mbar_wait(bs, 0);
+        __syncthreads();
+      }
     } else if constexpr (G::XPRE) {
       if (row_kept) {
         for (int e = threadIdx.x; e < 3 * N; e += NT) {
