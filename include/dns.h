@@ -429,9 +429,15 @@ int dns_mlp_set_normalisation(dns_mlp* net, const float* X, const float* T, int 
 /* loss and the gradient of every parameter (zeros for the normalisation entries), synchronous */
 int dns_mlp_loss_grad(dns_mlp* net, const float* X, const float* T, int P, float* grad_host, float* loss_host,
                       void* stream);
-/* one Adam step on the full batch; loss_host (may be NULL) receives the loss before the update */
+/* One Adam step on the full batch; loss_host (may be NULL) receives the loss before the update. A pass whose
+ * tensor-core waits gave up (DNS_ERR_TIMEOUT, from the next call that synchronises: this one with
+ * loss_host, dns_mlp_loss_grad or dns_mlp_get_params) leaves weights, moments and the step count as they
+ * were, as do the steps after it until that has been reported. */
 int dns_mlp_train_step(dns_mlp* net, const float* X, const float* T, int P, double lr, float* loss_host,
                        void* stream);
+
+/* Test hook: marks the network as a training pass whose waits gave up does. Nothing else is touched. */
+int dns_mlp_debug_give_up(dns_mlp* net);
 
 /* Attaches the network as a subgrid-stress closure of the handle's run (no
  * counterpart in the paper: the learned closure of the coarse-grid runs). From

@@ -89,6 +89,7 @@ SIGNATURES = {
     "dns_mlp_destroy": (_I, [_P]),
     "dns_mlp_set_params": (_I, [_P, ctypes.POINTER(ctypes.c_float), _I]),
     "dns_mlp_get_params": (_I, [_P, ctypes.POINTER(ctypes.c_float), _I]),
+    "dns_mlp_debug_give_up": (_I, [_P]),
     "dns_mlp_forward": (_I, [_P, _P, _P, _I, _P]),
     "dns_mlp_set_normalisation": (_I, [_P, _P, _P, _I, _P]),
     "dns_set_closure": (_I, [_P, _P, _D]),

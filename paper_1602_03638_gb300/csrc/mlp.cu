@@ -105,6 +105,9 @@ constexpr int TC_M = 128, TC_THREADS = 128, TC_TMEM_COLS = 128;
 constexpr int TC_X = 0, TC_H1 = TC_X + 128 * 16 * 2, TC_H2 = TC_H1 + 128 * 64 * 2, TC_W = TC_H2 + 128 * 64 * 2,
               TC_BAR = TC_W + IMG_FWD, TC_SMEM = TC_BAR + 16;
 constexpr unsigned long long TC_WAIT_NS = 1000000000ull;  // 1 s bound on every mbarrier wait
+// the network's error words: a wait gave up (any kernel); one of a training pass did, whose sums are not
+// valid; the Adam steps that were not taken since
+enum { ERR_ANY = 0, ERR_TRAIN = 1, ERR_SKIPPED = 2, ERR_WORDS = 3 };
 
 // shared-memory matrix descriptor: start address, leading (K) and stride (row-group)
 // byte offsets, the fixed version bits 46-47 = 1, no swizzle
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
     ok = __syncthreads_and(ok);  // shared operands and TMEM columns are free for the next tile
     tc_fence_after();
   }
-  if (!ok && t == 0) atomicExch(err, 1);
+  if (!ok && t == 0) atomicExch(err + ERR_ANY, 1);
   tc_fence_before();
   __syncthreads();
   if (warp == 0)
@@ -565,7 +568,10 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __rest
 #pragma unroll
     for (int c = 0; c < NOUT; ++c) out[(O_W3 - TRAIN_BEGIN) + (row - 64) * NOUT + c] = v[c];
   }
-  if (!ok && t == 0) atomicExch(err, 1);
+  if (!ok && t == 0) {
+    atomicExch(err + ERR_ANY, 1);
+    atomicExch(err + ERR_TRAIN, 1);
+  }
   tc_fence_before();
   __syncthreads();
   if (t < 2 * NH + NOUT + 1) {
@@ -579,14 +585,15 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __rest
 
 // The blocks' rows of partial sums added in order: gradients and loss into gsum (and, for the host, the
 // error flag behind them); ADAM: one Adam step on the trainable range (moments m, v; bias
-// corrections c1, c2) and the changed weights into the image.
+// corrections c1, c2) and the changed weights into the image. No step is taken on the sums of a training
+// pass that gave up, nor after it until that has been reported.
 // 32 columns a block, 8 threads each on every eighth row.
 constexpr int RED_COLS = 32, RED_ROWS = 8;
 template <bool ADAM>
 __global__ void __launch_bounds__(RED_COLS * RED_ROWS) k_reduce(const float* __restrict__ part, int rows,
                                                                 float* __restrict__ gsum, float* __restrict__ prm,
                                                                 float* __restrict__ m, float* __restrict__ v,
-                                                                unsigned char* __restrict__ img, const int* __restrict__ err,
+                                                                unsigned char* __restrict__ img, int* __restrict__ err,
                                                                 float lr, float b1, float b2, float eps, float c1, float c2) {
   __shared__ float red[RED_ROWS][RED_COLS];
   const int x = threadIdx.x % RED_COLS, y = threadIdx.x / RED_COLS, j = blockIdx.x * RED_COLS + x;
@@ -603,11 +610,13 @@ __global__ void __launch_bounds__(RED_COLS * RED_ROWS) k_reduce(const float* __r
   for (int r = 0; r < RED_ROWS; ++r) g += red[r][x];
   if (j == NTRAIN) {
     gsum[NPARAM] = g;
-    gsum[NPARAM + 1] = (float)*err;
+    gsum[NPARAM + 1] = (float)err[ERR_ANY];
+    if (ADAM && err[ERR_TRAIN]) ++err[ERR_SKIPPED];
     return;
   }
   const int i = TRAIN_BEGIN + j;
   if constexpr (ADAM) {
+    if (err[ERR_TRAIN]) return;
     const float mi = b1 * m[i] + (1.f - b1) * g;
     const float vi = b2 * v[i] + (1.f - b2) * g * g;
     m[i] = mi;
@@ -630,7 +639,7 @@ struct dns_mlp {
   float* m = nullptr;
   float* v = nullptr;
   unsigned char* img = nullptr;  // the BF16 weights as the kernels' operands (device)
-  int* err = nullptr;  // device flag: a tensor-core wait gave up
+  int* err = nullptr;  // ERR_WORDS (device): tensor-core waits that gave up
   int t = 0;           // Adam steps taken
 };
 
@@ -722,12 +731,13 @@ __global__ void __launch_bounds__(NORM_THREADS) k_norm(float* __restrict__ prm, 
   }
 }
 
-// Reports (and clears) a tensor-core wait that gave up; synchronises.
+// Reports (and clears) a tensor-core wait that gave up, the Adam steps that it prevented uncounted; synchronises.
 int mlp_check_err(dns_mlp* n, const char* where) {
-  int err = 0;
-  MLP_CUDA(cudaMemcpy(&err, n->err, sizeof(int), cudaMemcpyDeviceToHost), where);
-  if (!err) return DNS_OK;
-  MLP_CUDA(cudaMemset(n->err, 0, sizeof(int)), where);
+  int err[ERR_WORDS] = {};
+  MLP_CUDA(cudaMemcpy(err, n->err, sizeof(err), cudaMemcpyDeviceToHost), where);
+  if (!err[ERR_ANY]) return DNS_OK;
+  n->t -= err[ERR_SKIPPED];
+  MLP_CUDA(cudaMemset(n->err, 0, sizeof(err)), where);
   return mlp_fail(DNS_ERR_TIMEOUT, "dns_mlp: a kernel's tensor-core wait gave up after 1 s; its output is not valid");
 }
 
@@ -763,8 +773,8 @@ int dns_mlp_create(dns_mlp** out) {
   if (e == cudaSuccess) e = cudaMalloc(&n->v, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->img, IMG_BYTES);
   if (e == cudaSuccess) e = cudaMemset(n->img, 0, IMG_BYTES);
-  if (e == cudaSuccess) e = cudaMalloc(&n->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(n->err, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&n->err, ERR_WORDS * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(n->err, 0, ERR_WORDS * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->prm, 0, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(n->gsum, 0, (NPARAM + 2) * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(n->m, 0, NPARAM * sizeof(float));
@@ -800,6 +810,7 @@ int dns_mlp_set_params(dns_mlp* n, const float* host, int count) {
   MLP_CUDA(cudaMemset(n->m, 0, NPARAM * sizeof(float)), "dns_mlp_set_params");
   MLP_CUDA(cudaMemset(n->v, 0, NPARAM * sizeof(float)), "dns_mlp_set_params");
   n->t = 0;
+  MLP_CUDA(cudaMemset(n->err + ERR_TRAIN, 0, (ERR_WORDS - ERR_TRAIN) * sizeof(int)), "dns_mlp_set_params");
   k_pack<<<16, 256>>>(n->prm, n->img);
   MLP_CUDA(cudaGetLastError(), "dns_mlp_set_params pack");
   MLP_CUDA(cudaDeviceSynchronize(), "dns_mlp_set_params");
@@ -811,6 +822,13 @@ int dns_mlp_get_params(dns_mlp* n, float* host, int count) {
   MLP_CUDA(cudaDeviceSynchronize(), "dns_mlp_get_params");
   MLP_CUDA(cudaMemcpy(host, n->prm, NPARAM * sizeof(float), cudaMemcpyDeviceToHost), "dns_mlp_get_params copy");
   return mlp_check_err(n, "dns_mlp_get_params");
+}
+
+int dns_mlp_debug_give_up(dns_mlp* n) {
+  if (!n) return mlp_fail(DNS_ERR_ARG, "dns_mlp_debug_give_up: net is NULL");
+  const int err[2] = {1, 1};  // ERR_ANY, ERR_TRAIN
+  MLP_CUDA(cudaMemcpy(n->err, err, sizeof(err), cudaMemcpyHostToDevice), "dns_mlp_debug_give_up");
+  return DNS_OK;
 }
 
 int dns_mlp_forward(dns_mlp* n, const float* X, float* Y, int P, void* stream) {
