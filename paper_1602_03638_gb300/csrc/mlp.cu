@@ -101,9 +101,9 @@ __device__ __forceinline__ unsigned bf2(float lo, float hi) {
 // ---------------------------------------------------------------------------
 constexpr int TC_M = 128, TC_THREADS = 128, TC_TMEM_COLS = 128;
 // shared memory: A operands X (4 KB), H1, H2 (16 KB each); the image of the forward weights; then the
-// mbarrier
+// mbarriers: of the products, and of what is left of them when a wait gave up
 constexpr int TC_X = 0, TC_H1 = TC_X + 128 * 16 * 2, TC_H2 = TC_H1 + 128 * 64 * 2, TC_W = TC_H2 + 128 * 64 * 2,
-              TC_BAR = TC_W + IMG_FWD, TC_SMEM = TC_BAR + 16;
+              TC_BAR = TC_W + IMG_FWD, TC_DRAIN = TC_BAR + 8, TC_SMEM = TC_BAR + 16;
 constexpr unsigned long long TC_WAIT_NS = 1000000000ull;  // 1 s bound on every mbarrier wait
 // the network's error words: a wait gave up (any kernel); one of a training pass did, whose sums are not
 // valid; the Adam steps that were not taken since
@@ -148,6 +148,12 @@ __device__ __forceinline__ bool tc_wait(unsigned bar, unsigned parity) {
     if (it == 0) t0 = t;
     else if (t - t0 > TC_WAIT_NS) return false;
   }
+}
+// A wait gave up (the whole block calls this): waits, with the same limit, for every product that thread 0 has issued,
+// so that none is under way when the TMEM columns and the shared memory are given back.
+__device__ __forceinline__ void tc_drain(unsigned drain) {
+  if (threadIdx.x == 0) tc_commit(drain);
+  tc_wait(drain, 0);
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -198,13 +204,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
   __shared__ float s_b[2 * NH + 16];  // b1, b2, b3
   const int t = threadIdx.x, warp = t >> 5;
   const unsigned sbase = (unsigned)__cvta_generic_to_shared(tsm);
-  const unsigned bar = sbase + TC_BAR;
+  const unsigned bar = sbase + TC_BAR, drain = sbase + TC_DRAIN;
   for (int i = t; i < IMG_FWD / 16; i += TC_THREADS)
     reinterpret_cast<uint4*>(tsm + TC_W)[i] = reinterpret_cast<const uint4*>(img)[i];
   for (int i = t; i < 2 * NH + 16; i += TC_THREADS)
     s_b[i] = i < NH ? prm[O_B1 + i] : (i < 2 * NH ? prm[O_B2 + i - NH] : (i - 2 * NH < NOUT ? prm[O_B3 + i - 2 * NH] : 0.f));
   if (t == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(drain) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -295,7 +302,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
     ok = __syncthreads_and(ok);  // shared operands and TMEM columns are free for the next tile
     tc_fence_after();
   }
-  if (!ok && t == 0) atomicExch(err + ERR_ANY, 1);
+  if (!ok) {  // the same for the whole block
+    if (t == 0) atomicExch(err + ERR_ANY, 1);
+    tc_drain(drain);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 0)
@@ -321,7 +331,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_mlp_tc(const float* __restrict__
 constexpr int TR_THREADS = 256, TR_TMEM_COLS = 256, TR_T = 0, TR_GW = 64, TR_G1 = 144;
 constexpr int TR_EG = 18;  // groups of 8 columns of the array dZ1 (64) | dZ2 (64) | dY (16)
 constexpr int TR_X = 0, TR_H = TR_X + 128 * 16 * 2, TR_E = TR_H + 128 * 128 * 2, TR_W = TR_E + 128 * TR_EG * 16,
-              TR_BAR = TR_W + IMG_BYTES, TR_SMEM = TR_BAR + 16;
+              TR_BAR = TR_W + IMG_BYTES, TR_DRAIN = TR_BAR + 8, TR_SMEM = TR_BAR + 16;
 constexpr int PART = 5264;  // floats of a row of partial sums: NTRAIN gradients, the loss, padding
 
 // sums over the warp's 32 lanes of v[i], i < 32: lane l returns the sum of v[l]
@@ -349,7 +359,7 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __rest
   __shared__ float s_sum[4][2 * NH + 16];      // per quarter: gb1, gb2, gb3 and the loss
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, q = warp & 3, hf = warp >> 2, row = 32 * q + lane;
   const unsigned sbase = (unsigned)__cvta_generic_to_shared(tsm);
-  const unsigned bar = sbase + TR_BAR;
+  const unsigned bar = sbase + TR_BAR, drain = sbase + TR_DRAIN;
   for (int i = t; i < IMG_BYTES / 16; i += TR_THREADS)
     reinterpret_cast<uint4*>(tsm + TR_W)[i] = reinterpret_cast<const uint4*>(img)[i];
   if (t < 2 * NH + 16)
@@ -362,6 +372,7 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __rest
   }
   if (t == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(drain) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -531,6 +542,8 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_mlp_train(const float* __rest
     ok = __syncthreads_and(ok);  // the block leaves the loop together
   }
   if (done > 0) wait();
+  ok = __syncthreads_and(ok);
+  if (!ok) tc_drain(drain);
   // the block's sums: weights from TMEM, biases and loss through shared memory
   s_sum[q][32 * hf + lane] = gb1;
   s_sum[q][NH + 32 * hf + lane] = gb2;
