@@ -68,16 +68,17 @@ __global__ void k_pack(const float* __restrict__ p, unsigned char* __restrict__ 
 
 // Logistic functions of two values, 1 / (1 + exp(-z)), with one reciprocal for both: 1 / a = b / (a b).
 // The multi-function unit (two exponentials and one reciprocal, 16 lanes per SM and clock) is what
-// bounds the activations. -z is capped at 60 ln 2 so that the product stays finite; below it the
-// logistic is under 1e-18. Relative error about 1e-6, far below the BF16 rounding that follows.
+// bounds the activations. -z is capped at 60 ln 2 = 41.6 so that the product stays finite; there the
+// logistic is under 1e-18 and taken as zero (a value left over would be multiplied by z, which has no bound, in
+// the activation and in its slope). Relative error about 1e-6, far below the BF16 rounding that follows.
 __device__ __forceinline__ void logistic2(float z0, float z1, float& s0, float& s1) {
   float e0, e1, r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fminf(z0 * -1.4426950408889634f, 60.f)));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fminf(z1 * -1.4426950408889634f, 60.f)));
   const float a = 1.f + e0, b = 1.f + e1;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a * b));
-  s0 = r * b;
-  s1 = r * a;
+  s0 = z0 > -41.58f ? r * b : 0.f;
+  s1 = z1 > -41.58f ? r * a : 0.f;
 }
 __device__ __forceinline__ unsigned bf2(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
