@@ -63,7 +63,7 @@ def _sources_digest() -> str:
     return h.hexdigest()
 
 
-KERNEL_SOURCES = ("fft_core.cuh", "solver_kernels.cuh", "dns_internal.h", "solver_inst.cu", "instances.h")
+KERNEL_SOURCES = ("fft_core.cuh", "fixed_point.cuh", "solver_kernels.cuh", "dns_internal.h", "solver_inst.cu", "instances.h")
 
 
 def kernel_digest() -> str:
