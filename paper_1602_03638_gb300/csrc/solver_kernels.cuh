@@ -1838,7 +1838,7 @@ struct SolverImpl {
   // z-pass tile widths offered besides the default (the generic z-pass of the small grids)
   static constexpr bool ztile_ok(int t) {
     return ISO && N <= BATCH_MAX_N && t >= 4 && t <= 32 && pow2_part(N) % t == 0 &&
-           (size_t)padded_len(M) * odd_ld(6 * t) * sizeof(cx<T>) <= 112 * 1024;
+           G::zbytes(t) <= 112 * 1024;  // two blocks an SM
   }
   template <int TXO>
   static void ztile_attr(cudaError_t& e) {
