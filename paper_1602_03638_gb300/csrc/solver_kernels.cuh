@@ -108,11 +108,10 @@ struct Geometry {
   static constexpr size_t ZSMEM = zbytes(ZTX);
 };
 
-// Tile of the y-pass by direction. The inverse pass (6 full fields) takes 128-byte
-// rows in FP32 up to N = 512 with 8 warps looping over its 16 columns (3 blocks per
-// SM); the forward pass (3 fields, pruned) takes 64-byte rows, one warp per column, 4
-// blocks per SM (both measured at 512^3). FP64 keeps 128-byte rows up to N = 512,
-// 64-byte rows above.
+// Tile of the y-pass by direction: 128-byte rows (64-byte rows for the FP32 forward pass and above 512 points).
+// SHORT: FP32 lines of up to 128 points (yshort_tile), 4 warps that take several columns each. FP64: one column per
+// warp. FP32 lines of 256 points and more run through k_yreg; k_ypass is left to products_low there
+// (k_yreg was not tried for it).
 // TXO > 0 replaces the tile width (a tuned schedule of the small grids).
 // NY: the line length (points along y) where it differs from N (the x extent).
 template <typename T, int N, int INV, int TXO = 0, int NY = N>
@@ -1932,7 +1931,7 @@ struct SolverImpl {
     DNS_ATTR((k_ypass<T, N, 1, 0, 0, NY, NZ, 0, 1>), (YCfg<T, N, 1, 0, NY>::SMEM));
     DNS_ATTR((k_ypass<T, N, 0, 1, 0, NY, NZ>), (YCfg<T, N, 0, 0, NY>::SMEM));
     if constexpr (!YREG) DNS_ATTR((k_ypass<T, N, 0, 0, 0, NY, NZ>), (YCfg<T, N, 0, 0, NY>::SMEM));
-    DNS_ATTR((k_zpass<T, N, ZM_CROSS, 0, NY, NZ>), G::ZSMEM);
+    if constexpr (!ZTMA) DNS_ATTR((k_zpass<T, N, ZM_CROSS, 0, NY, NZ>), G::ZSMEM);
     if constexpr (PLANS > 1) {
       DNS_ATTR((k_xpass<T, N, XM_INV_CURL, N, N, 1>), G::XSMEM);
       DNS_ATTR((k_xpass<T, N, XM_STAGE, N, N, 1>), G::XSMEM_ST);
@@ -2102,7 +2101,7 @@ struct SolverImpl {
 
   // one batched stage; the members share one radix plan (the ensemble groups them by it)
   static cudaError_t rk_stage_batch(const PassArgs* A, int count, int kmax3, cudaStream_t st) {
-    if constexpr (BATCHED && N != 512 && N != 1024) {
+    if constexpr (BATCHED) {
       if (count < 1 || count > BATCH_MAX_COUNT) return cudaErrorInvalidValue;
       for (int i = 1; i < count; ++i)
         if (A[i].plan != A[0].plan) return cudaErrorInvalidValue;
