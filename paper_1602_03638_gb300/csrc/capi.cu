@@ -276,60 +276,6 @@ namespace dns {
 void set_error_message(const char* msg) { g_err = msg; }
 }  // namespace dns
 
-namespace dns {
-namespace {
-constexpr size_t PIN_UNIT = 64;  // a cache line
-struct PinnedBlock {
-  std::mutex m;
-  char* base = nullptr;
-  std::map<size_t, size_t> used;  // offset -> bytes of its pieces
-};
-PinnedBlock& pinned_block() {
-  static PinnedBlock* b = new PinnedBlock;  // outlives the objects that are freed while the process ends
-  return *b;
-}
-}  // namespace
-
-cudaError_t pinned_get(void** p, size_t bytes) {
-  *p = nullptr;
-  bytes = (bytes + PIN_UNIT - 1) / PIN_UNIT * PIN_UNIT;
-  PinnedBlock& b = pinned_block();
-  std::lock_guard<std::mutex> lock(b.m);
-  size_t at = 0;  // the first gap
-  for (const auto& piece : b.used) {
-    if (piece.first - at >= bytes) break;
-    at = piece.first + piece.second;
-  }
-  if (at + bytes > PINNED_BYTES) return cudaMallocHost(p, bytes);
-  if (!b.base) {
-    const cudaError_t e = cudaMallocHost((void**)&b.base, PINNED_BYTES);
-    if (e != cudaSuccess) {
-      b.base = nullptr;
-      return e;
-    }
-  }
-  b.used[at] = bytes;
-  *p = b.base + at;
-  return cudaSuccess;
-}
-
-void pinned_put(void* p) {
-  if (!p) return;
-  PinnedBlock& b = pinned_block();
-  std::lock_guard<std::mutex> lock(b.m);
-  const uintptr_t at = (uintptr_t)p - (uintptr_t)b.base;
-  if (!b.base || (uintptr_t)p < (uintptr_t)b.base || at >= PINNED_BYTES) {
-    cudaFreeHost(p);
-    return;
-  }
-  b.used.erase((size_t)at);
-  if (b.used.empty()) {
-    cudaFreeHost(b.base);
-    b.base = nullptr;
-  }
-}
-}  // namespace dns
-
 struct dns_handle {
   int N = 0;  // points along x (and along y and z on a cubic grid)
   int Ny = 0, Nz = 0;  // points along y and z
@@ -412,7 +358,7 @@ void release(dns_handle* h) {
     if (ev) cudaEventDestroy(ev);
   for (cudaStream_t cs : h->cl_side)
     if (cs) cudaStreamDestroy(cs);
-  pinned_put(h->host_flag);
+  if (h->host_flag) cudaFreeHost(h->host_flag);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->own_stream) cudaStreamDestroy(h->own_stream);
 }
@@ -689,7 +635,7 @@ int dns_create3(int Nx, int Ny, int Nz, double nu, double dt, int dtype, dns_han
     }
     if (ce == cudaSuccess) ce = cudaMemset(h->U, 0, 3 * h->fs * cb);
     if (ce == cudaSuccess) ce = cudaMemset(row_flag(h), 0, sizeof(int));
-    if (ce == cudaSuccess) ce = pinned_get((void**)&h->host_flag, sizeof(int));
+    if (ce == cudaSuccess) ce = cudaMallocHost(&h->host_flag, sizeof(int));
     if (ce != cudaSuccess) rc = cuda_fail(ce, "dns_create initialisation");
   }
   if (rc != DNS_OK) {

@@ -128,11 +128,4 @@ cudaError_t closure_force(const void* S6, int N, void* F3, int dtype, cudaStream
 cudaError_t filter_internal(const void* fine, int Nf, void* coarse, int Nc, int fields, int dtype, cudaStream_t st);
 cudaError_t fill_f32(float* p, size_t n, float v, cudaStream_t st);
 
-// Pinned host memory for small read-backs (row flags, the network's loss and gradient). Pinning takes 0.35 ms a call, as
-// much as the rest of a small dns_create, so the objects alive share one block of PINNED_BYTES, pinned for the first and given
-// back with the last; what does not fit is pinned by itself. Any thread.
-constexpr size_t PINNED_BYTES = 128 * 1024;
-cudaError_t pinned_get(void** p, size_t bytes);
-void pinned_put(void* p);
-
 }  // namespace dns

@@ -781,7 +781,7 @@ int dns_mlp_create(dns_mlp** out) {
   dns_mlp* n = new dns_mlp();
   cudaError_t e = cudaMalloc(&n->prm, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->gsum, (NPARAM + 2) * sizeof(float));
-  if (e == cudaSuccess) e = dns::pinned_get((void**)&n->host, (NPARAM + 2) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMallocHost(&n->host, (NPARAM + 2) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->part, (size_t)TR_PER_SM * mlp_sms() * PART * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->m, NPARAM * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&n->v, NPARAM * sizeof(float));
@@ -812,7 +812,7 @@ int dns_mlp_destroy(dns_mlp* n) {
   cudaFree(n->v);
   cudaFree(n->img);
   cudaFree(n->part);
-  dns::pinned_put(n->host);
+  if (n->host) cudaFreeHost(n->host);
   cudaFree(n->err);
   delete n;
   return DNS_OK;
