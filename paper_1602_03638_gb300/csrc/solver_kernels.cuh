@@ -1486,15 +1486,33 @@ __device__ __forceinline__ void zt_fft(cx<float> (&v)[ZTma<M>::VALS], unsigned l
   }
 }
 
-// in: W as (x, y, kz, field), kz bounded by the planes that hold values; out: by the planes kept. A block whose copies
-// do not arrive within the limit starts no others, waits for those under way once more and fills the products of
-// the tiles that are left with NaN, which the checks of the state report.
+// A block whose copies did not arrive within the limit: waits once more for the two under way and fills the products
+// of its tiles from t on with NaN, which the checks of the state report. Out of line: in the kernel it cost
+// the 1024-point transforms their registers (13.25 -> 13.79 ms, so 13.15).
+template <int N, int NY, int NZ>
+__device__ __noinline__ void ztma_give_up(cx<float>* W, int t, int kc, unsigned bar0, unsigned bar1, unsigned phase) {
+  using Z = ZTma<NZ / 2>;
+  constexpr size_t FS = Geometry<float, N, NY, NZ>::FS;
+  constexpr int TX = Z::TX, XT = N / TX, NT = XT * NY;
+  mbar_wait(bar0, phase);
+  mbar_wait(bar1, phase);
+  const float nan = __int_as_float(0x7fffffff);
+#pragma unroll 1
+  for (; t < NT; t += gridDim.x) {
+#pragma unroll 1
+    for (int e = threadIdx.x; e < 3 * kc * TX; e += 32 * Z::NW) {
+      const int x = e % TX, k = (e / TX) % kc, f = e / (TX * kc);
+      W[f * FS + ((size_t)k * NY + t / XT) * N + (t % XT) * TX + x] = mk(nan, nan);
+    }
+  }
+}
+
+// in: W as (x, y, kz, field), kz bounded by the planes that hold values; out: by the planes kept
 template <int N, int NY, int NZ>
 __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
     k_ztma(int kmax3, const void* __restrict__ twp, cx<float>* __restrict__ W, const __grid_constant__ CUtensorMap in,
            const __grid_constant__ CUtensorMap out) {
   constexpr int M = NZ / 2;
-  constexpr size_t FS = Geometry<float, N, NY, NZ>::FS;
   using Z = ZTma<M>;
   constexpr int TX = Z::TX, CX = Z::CX, NW = Z::NW, FB = Z::FB, HL = Z::HL, V = Z::VALS, STEP = HL * Z::ROWB;
   constexpr int XT = N / TX, NT = XT * NY;  // tiles: x-tiles times y
@@ -1652,19 +1670,8 @@ __global__ void __launch_bounds__(32 * ZTma<NZ / 2>::NW, 1)
       if (tn < NT) fetch(tn, 0, bar1);
     }
   }
-  if (t < NT) {  // gave up at tile t: both of its copies were started, no later one
-    mbar_wait(bar0, phase);
-    mbar_wait(bar1, phase);
-    const float nan = __int_as_float(0x7fffffff);
-#pragma unroll 1
-    for (; t < NT; t += gridDim.x) {
-#pragma unroll 1
-      for (int e = threadIdx.x; e < 3 * kc * TX; e += 32 * NW) {
-        const int x = e % TX, k = (e / TX) % kc, f = e / (TX * kc);
-        W[f * FS + ((size_t)k * NY + t / XT) * N + (t % XT) * TX + x] = mk(nan, nan);
-      }
-    }
-  }
+  // gave up at tile t: both of its copies were started, no later one
+  if (t < NT) ztma_give_up<N, NY, NZ>(W, t, kc, bar0, bar1, phase);
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
