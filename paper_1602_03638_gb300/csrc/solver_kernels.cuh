@@ -321,14 +321,19 @@ __device__ __forceinline__ void xpass_body(const PassArgs a, const int bx, const
         line_fft<T, N, TW, V>(SRow<T>{s + (warp * LS + 1) / 2 * 2}, line, line, tw, lane);
       }
       ok = mbar_wait(bs, 0) && ok;
-      // copies that do not arrive within the limit: waited for once more, since they must not land after the block has
-      // gone, and the whole row becomes NaN, which the checks of the state report
-      if (!__syncthreads_and(ok)) {
+      // Copies that a warp does not see arrive within the limit: it waits once more, since they must not land after
+      // the block has gone, and turns its columns and its line of N_hat to NaN, which the checks of the state
+      // report. Before the barrier and warp by warp: agreed on by the block at the barrier, the launch took 700 us at
+      // 512^3, so 696 (690 where nothing is waited for again).
+      if (!__all_sync(0xffffffffu, ok)) {
         nu = (T)__int_as_float(0x7fffffff);
         if (row_kept) mbar_wait(bw, 0);
         mbar_wait(bs, 0);
-        __syncthreads();
+        __syncwarp();
+        if (row_kept && warp < 3)
+          for (int p = lane; p < N; p += 32) s[warp * LS + padt<T>(p)] = mk(nu, nu);
       }
+      __syncthreads();
     } else if constexpr (G::XPRE) {
       if (row_kept) {
         for (int e = threadIdx.x; e < 3 * N; e += NT) {
