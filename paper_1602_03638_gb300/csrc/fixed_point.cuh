@@ -55,6 +55,9 @@ __device__ __forceinline__ unsigned fx_upper(ll a) {
 __device__ __forceinline__ ll fx_shift(ll a, int n) { return (a << max(n, 0)) >> max(-n, 0); }
 __device__ __forceinline__ fx fx_shift(fx a, int n) { return mk(fx_shift(a.x, n), fx_shift(a.y, n)); }
 
+// the left shift that takes a line of L1 norm l1 2^41 (l1 rounded up) to 62 bits
+__device__ __forceinline__ int fx_shift_of(unsigned l1) { return __clz(l1) - 11; }
+
 // (t >> 32) + c: a product by 1 takes the odd register of the pair t as it is
 __device__ __forceinline__ ll fx_add_up(ll t, ll c) { return madw((int)(t >> 32), 1, c); }
 // 4 p with the top two bits of t's low word below
@@ -387,8 +390,8 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
 
 // ---- several short lines per warp --------------------------------------------------------
 // The passes of warp_fft_lines on lines of fixed-point values, in place. FROM: what pass 0 reads,
-// fixed point (FX_IN), fixed point of line g to be shifted left by sh[g] bits (FX_SHIFT; right where
-// negative) or doubles to be taken to scale sh[g] (FX_DOUBLE).
+// fixed point (FX_IN), fixed point of line g to be shifted by fx_shift_of(sh[g]) (FX_SHIFT) or doubles to be
+// taken to scale sh[g] (FX_DOUBLE).
 // MAG: the upper words of the results' magnitudes are or'ed into mag[g] (cleared before): the top bit of the largest.
 enum FxFrom { FX_IN = 0, FX_SHIFT = 1, FX_DOUBLE = 2 };
 template <int L, int TWN, int G, int LD, int P, int V, int FROM, bool MAG = false>
@@ -412,7 +415,7 @@ __device__ __forceinline__ void warp_fft_fx_lines(cx<double>* s0, const cx<doubl
         else v[b][r] = *reinterpret_cast<const fx*>(q);
       }
       if constexpr (P == 0 && FROM == FX_SHIFT) {
-        const int n = sh[g];
+        const int n = fx_shift_of((unsigned)sh[g]);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[b][r] = fx_shift(v[b][r], n);
       }

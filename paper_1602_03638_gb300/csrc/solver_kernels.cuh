@@ -879,7 +879,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   __shared__ int sL[NL];        // power of two that it was multiplied by (fx_lift)
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
-  __shared__ unsigned sQ[NP * TX];  // L1 of a line of products, then its shift
+  __shared__ unsigned sQ[NP * TX];  // L1 of a line of products
   __shared__ unsigned sM[NL];       // top bit of a line's physical values
   __shared__ int sE[NP * TX];       // scale of a line of products; then what fx_to takes for it
   __shared__ int sT[NP * 2 * TX];   // shifts of the two u (ZM_CROSS) of a line of products
@@ -1055,12 +1055,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
       }
     }
     __syncthreads();
-    if (threadIdx.x < NP * TX) {
-      const int sh = __clz(sQ[threadIdx.x]) - 11;
-      sQ[threadIdx.x] = (unsigned)sh;
-      sE[threadIdx.x] -= sh + 1018;
-    }
-    __syncthreads();
+    if (threadIdx.x < NP * TX) sE[threadIdx.x] -= fx_shift_of(sQ[threadIdx.x]) + 1018;  // read after the transforms
   }
 
   if constexpr (PROD || MODE == ZM_LOAD) {
