@@ -24,8 +24,9 @@
 // 2^-53 |x|_2 up to the longest line; most where all |x_j| are equal, many bits below where few modes
 // carry the line. Measured against extended precision (c2r and r2c of white, Gaussian and power-law
 // fields, 16^3 .. 512^3): 0.5 - 2.3e-16 relative, where FP64 butterflies gave 1.1 - 5.8e-16.
-// A line with a NaN or an infinity gives NaN everywhere. Lines whose largest value is below 2^-831 or above
-// 2^960 are taken times a power of two (fx_lift), so that the whole range of a double is kept, subnormal numbers too.
+// A line with a NaN or an infinity gives NaN everywhere. Lines whose largest value is below 2^-959 are
+// taken times a power of two (FX_LIFT) and results past the fast conversion are rescaled (fx_far), so that the whole
+// range of a double is kept, subnormal numbers too.
 //
 // Numbers here are cx<long long>. The low word of a factor is signed (w = hi 2^32 + lo, |lo| < 2^31).
 #pragma once
@@ -161,23 +162,17 @@ struct FxScale {
   int K;         // biased exponent: L1 <= 2^(K - 1023)
   unsigned nan;  // 0x7ff80000 if the line holds a NaN or an infinity, else 0
 };
-// The power of two that brings a line of largest magnitude word `mag` to where fx_from takes every element in
-// full (exponents of 192 and more; it reads an exponent of 0 as zero) and fx_to has room above: 0 for
-// all but extreme lines, whose values are multiplied by fx_pow2 of it, exactly.
-__device__ __forceinline__ bool fx_extreme(unsigned mag) { return mag - (192u << 20) >= (1791u << 20); }
-// low: a lower word is not zero (asked for where mag is)
-__device__ __forceinline__ int fx_lift(unsigned mag, bool low) {
-  return mag < (192u << 20) ? (mag || low ? 600 : 0) : (fx_extreme(mag) && mag < 0x7ff00000u ? -64 : 0);
-}
+// fx_from reads an exponent of 0 as zero and shifts elements of a line of scale K out below 2^(K - 1086): a line whose
+// largest magnitude word is below 2^-959 is therefore multiplied by 2^FX_LIFT first, exactly, where it lies.
+constexpr int FX_LIFT = 600;
+__device__ __forceinline__ bool fx_tiny(unsigned mag) { return mag < (64u << 20); }  // or zero
 __device__ __forceinline__ double fx_pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
 // the largest magnitude word after that (at most)
-__device__ __forceinline__ unsigned fx_lifted(unsigned mag, int lift) {
-  return lift ? max(mag, 1u << 20) + ((unsigned)lift << 20) : mag;
-}
+__device__ __forceinline__ unsigned fx_lifted(unsigned mag) { return max(mag, 1u << 20) + ((unsigned)FX_LIFT << 20); }
 // from the line's largest magnitude word and the sum of its shares
 __device__ __forceinline__ FxScale fx_scale(unsigned mag, unsigned shares) {
   FxScale s;
-  s.K = max((int)(mag >> 20) + 20 - __clz(shares), 128);
+  s.K = mag ? (int)(mag >> 20) + 20 - __clz(shares) : 128;
   s.nan = mag >= 0x7ff00000u ? 0x7ff80000u : 0u;
   return s;
 }
@@ -288,29 +283,35 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
     }
     m = __reduce_max_sync(0xffffffffu, m);
     int lift = 0;
-    if (fx_extreme(m)) {
-      unsigned low = 0;
-      if (m == 0) {
+    if (fx_tiny(m)) {
+      unsigned any = m;
+      if (m == 0) {  // zero, or below 2^-1042
 #pragma unroll 1
         for (int p = lane; p < L; p += 32) {
           const cx<double> x = src.load(src.at(p));
-          low |= (unsigned)__double2loint(x.x) | (unsigned)__double2loint(x.y);
+          any |= (unsigned)__double2loint(x.x) | (unsigned)__double2loint(x.y);
         }
       }
-      lift = fx_lift(m, __any_sync(0xffffffffu, low != 0));
-      if (KEEP && lift) {
+      if (__any_sync(0xffffffffu, any != 0)) {
+        lift = FX_LIFT;
+        m = fx_lifted(m);
+#pragma unroll 1
+        for (int p = lane; p < L; p += 32) {
+          cx<double>* q = const_cast<cx<double>*>(src.at(p));  // this warp's line, which nobody reads after it
+          *q = scal(*q, fx_pow2(FX_LIFT));
+        }
+        __syncwarp();
+        if constexpr (KEEP) {
 #pragma unroll
-        for (int b = 0; b < BPL; ++b) {
+          for (int b = 0; b < BPL; ++b) {
+            const int j = lane + 32 * b;
 #pragma unroll
-          for (int r = 0; r < R; ++r) d[b][r] = scal(d[b][r], fx_pow2(lift));
+            for (int r = 0; r < R; ++r)
+              if (NB % 32 == 0 || j < NB) d[b][r] = rd(j, r);
+          }
         }
       }
     }
-    auto again = [&](int j, int r) -> cx<double> {  // (KEEP: unused)
-      const cx<double> x = rd(j, r);
-      return lift ? scal(x, fx_pow2(lift)) : x;
-    };
-    m = fx_lifted(m, lift);
     const int top = fx_top(m);
     float s = 0.f;
 #pragma unroll
@@ -320,7 +321,7 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
       for (int r = 0; r < R; ++r) {
         cx<double> x;
         if constexpr (KEEP) x = d[b][r];
-        else x = (NB % 32 == 0 || j < NB) ? again(j, r) : mk(0.0, 0.0);
+        else x = (NB % 32 == 0 || j < NB) ? rd(j, r) : mk(0.0, 0.0);
         s += fx_rel(x.x, top) + fx_rel(x.y, top);
       }
     }
@@ -332,7 +333,7 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if constexpr (KEEP) v[b][r] = fx_from(d[b][r], sc.K);
-          else v[b][r] = fx_from(again(j, r), sc.K);
+          else v[b][r] = fx_from(rd(j, r), sc.K);
         }
         fx_dft<R>(v[b]);
       }

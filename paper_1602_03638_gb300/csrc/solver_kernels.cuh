@@ -876,7 +876,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   constexpr int GL = cmin(FxLinesPerWarp<M, V>::value, TX);  // lines per warp
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int sK[NL];        // scale of a line as the tile holds it
-  __shared__ int sL[NL];        // power of two that it was multiplied by (fx_lift)
+  __shared__ int sL[NL];        // power of two that it was multiplied by (0 or FX_LIFT)
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
   __shared__ unsigned sQ[NP * TX];  // L1 of a line of products
@@ -922,20 +922,22 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
 #pragma unroll
     for (int o = SUB / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     int lift = 0;
-    if (__any_sync(0xffffffffu, fx_extreme(m))) {
-      unsigned low = 0;
+    if (__any_sync(0xffffffffu, fx_tiny(m))) {
+      unsigned any = m;
       if (m == 0) {
         for (int k = q; k < klim; k += SUB) {
           const cd v = ln[padt<double>(k) * LD];
-          low |= (unsigned)__double2loint(v.x) | (unsigned)__double2loint(v.y);
+          any |= (unsigned)__double2loint(v.x) | (unsigned)__double2loint(v.y);
         }
       }
 #pragma unroll
-      for (int o = SUB / 2; o > 0; o >>= 1) low |= __shfl_xor_sync(0xffffffffu, low, o);
-      lift = fx_lift(m, low != 0);
-      if (lift && l < NL)
-        for (int k = q; k < klim; k += SUB) ln[padt<double>(k) * LD] = scal(ln[padt<double>(k) * LD], fx_pow2(lift));
-      m = fx_lifted(m, lift);
+      for (int o = SUB / 2; o > 0; o >>= 1) any |= __shfl_xor_sync(0xffffffffu, any, o);
+      if (fx_tiny(m) && any) {
+        lift = FX_LIFT;
+        m = fx_lifted(m);
+        if (l < NL)
+          for (int k = q; k < klim; k += SUB) ln[padt<double>(k) * LD] = scal(ln[padt<double>(k) * LD], fx_pow2(FX_LIFT));
+      }
     }
     const int top = fx_top(m);
     float t = 0.f;

@@ -20,8 +20,16 @@ def _p2(x, e):
 
 @pytest.mark.parametrize("N", [8, 12, 16, 48, 64, 128, 512])
 def test_transforms_over_the_whole_range(N):
-    shape = (N,) * 3
-    g = torch.Generator(device="cuda").manual_seed(N)
+    _transforms((N,) * 3)
+
+
+def test_long_rows_over_the_whole_range():
+    _transforms((1024, 512, 256))  # lines of 1024 points are read twice
+
+
+def _transforms(shape):
+    nx, ny, _ = shape
+    g = torch.Generator(device="cuda").manual_seed(nx)
     with Solver(shape, 0.01, 0.01, "f64") as s:
         u = torch.rand(s.phys_shape, generator=g, dtype=torch.float64, device="cuda") + 0.5
         spec = torch.empty(s.spec_shape, dtype=torch.complex128, device="cuda")
@@ -35,7 +43,7 @@ def test_transforms_over_the_whole_range(N):
         out, phys = torch.empty_like(spec), torch.empty_like(u)
         # to the largest results, and to where the least ones (of the passes between too, smaller by up to N each)
         # are normal yet
-        for e in (-1021 - small + 2 * N.bit_length() + 8, -900, 940, 1021 - top):
+        for e in (-1021 - small + nx.bit_length() + ny.bit_length() + 8, -900, 940, 1021 - top):
             s.transform_r2c(_p2(u, e), out)
             assert torch.equal(_p2(torch.view_as_real(out), -e), torch.view_as_real(spec)), e
             s.transform_c2r(out, phys)
@@ -49,7 +57,7 @@ def test_transforms_over_the_whole_range(N):
             torch.cuda.synchronize()
             d = _p2(torch.view_as_real(out), 1000) - torch.view_as_real(spec)
             # three passes; a pass adds up N roundings at most
-            assert d.abs().max() <= _p2(torch.tensor(TINY, dtype=torch.float64, device="cuda"), 1000) * (1 + N + N * N)
+            assert d.abs().max() <= _p2(torch.tensor(TINY, dtype=torch.float64, device="cuda"), 1000) * (1 + nx + nx * ny)
             assert torch.view_as_real(out).abs().max() > 0
         s.transform_r2c(_p2(u, 1023 - top + 3), out)
         assert not torch.isfinite(torch.view_as_real(out)).all()
