@@ -269,21 +269,24 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
   };
   if constexpr (FIRST) {
     cx<double> d[KEEP ? BPL : 1][KEEP ? R : 1];
-    unsigned m = 0;
-#pragma unroll
-    for (int b = 0; b < BPL; ++b) {
-      const int j = lane + 32 * b;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        cx<double> x = mk(0.0, 0.0);
-        if (NB % 32 == 0 || j < NB) x = rd(j, r);
-        if constexpr (KEEP) d[b][r] = x;
-        m = max(m, fx_mag(x));
-      }
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
+    unsigned m;
     int lift = 0;
-    if (fx_tiny(m)) {
+#pragma unroll 1
+    for (;;) {
+      m = 0;
+#pragma unroll
+      for (int b = 0; b < BPL; ++b) {
+        const int j = lane + 32 * b;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          cx<double> x = mk(0.0, 0.0);
+          if (NB % 32 == 0 || j < NB) x = rd(j, r);
+          if constexpr (KEEP) d[b][r] = x;
+          m = max(m, fx_mag(x));
+        }
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (!fx_tiny(m) || lift) break;
       unsigned any = m;
       if (m == 0) {  // zero, or below 2^-1042
 #pragma unroll 1
@@ -292,25 +295,14 @@ __device__ __forceinline__ void warp_fft_fx_pass(const Src& src, const Work& wor
           any |= (unsigned)__double2loint(x.x) | (unsigned)__double2loint(x.y);
         }
       }
-      if (__any_sync(0xffffffffu, any != 0)) {
-        lift = FX_LIFT;
-        m = fx_lifted(m);
+      if (!__any_sync(0xffffffffu, any != 0)) break;
+      lift = FX_LIFT;
 #pragma unroll 1
-        for (int p = lane; p < L; p += 32) {
-          cx<double>* q = const_cast<cx<double>*>(src.at(p));  // this warp's line, which nobody reads after it
-          *q = scal(*q, fx_pow2(FX_LIFT));
-        }
-        __syncwarp();
-        if constexpr (KEEP) {
-#pragma unroll
-          for (int b = 0; b < BPL; ++b) {
-            const int j = lane + 32 * b;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-              if (NB % 32 == 0 || j < NB) d[b][r] = rd(j, r);
-          }
-        }
+      for (int p = lane; p < L; p += 32) {
+        cx<double>* q = const_cast<cx<double>*>(src.at(p));  // this warp's line, which nobody reads after it
+        *q = scal(*q, fx_pow2(FX_LIFT));
       }
+      __syncwarp();
     }
     const int top = fx_top(m);
     float s = 0.f;
