@@ -280,6 +280,15 @@ def time_steps(torch, s, st, steps):
     return e0.elapsed_time(e1)
 
 
+def form_roofline(N, rb, ms, pruned, peak):
+    """HBM fraction of an FP64 step by the bytes of the two-pass model of what it transforms: 132 cv, or those of a
+    state inside the 2/3 box (its passes are limited by integer issue before that)."""
+    cv = truncated_step_cv(N) if pruned else STEP_CV
+    achieved = cv * cv_bytes(N, rb) / (ms * 1e-3) / 1e9
+    return {"bound": "hbm", "limit": "integer issue", "model_cv": cv, "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "frac": achieved / peak}
+
+
 def run_form(torch, Solver, inputs, N, dtype, warm, steps):
     cdt = torch.complex64 if dtype == "f32" else torch.complex128
     with Solver(N, NU, DT, dtype) as s:
@@ -308,8 +317,7 @@ def run_form(torch, Solver, inputs, N, dtype, warm, steps):
         kc = (N + 2) // 3
         zk, yk = kc / (N // 2), (2 * kc - 1) / N
         flops = flops_full * ((1.0 + zk + zk * yk) / 3.0 if pruned else 1.0)
-        out["roofline"] = {"bound": "integer issue", "achieved": STEP_CV * cv_bytes(N, rb) / (ms * 1e-3) / 1e9,
-                           "peak": measured_peaks()[0], "unit": "GB/s", "frac": model_ms / ms,
+        out["roofline"] = {**form_roofline(N, rb, ms, pruned, measured_peaks()[0]),
                            "flops_per_step": flops, "flops_per_step_full_transforms": flops_full, "rows_pruned": pruned,
                            "fp64_equivalent_tflops": flops / (ms * 1e-3) / 1e12, "fp64_fma_peak_tflops": fp64_peak_tflops(),
                            "peak_kind": "measured copy bandwidth; the FP64 FMA peak by a dependent-FMA probe, CUDA events"}
