@@ -50,7 +50,8 @@ constexpr int ilcm(int a, int b) { return a / igcd(a, b) * b; }
 // of 16 values meets every bank), chosen by counting the bank conflicts of the passes of warp_fft_lines over
 // all (PAD, RES) and the tile widths 4 to 32. Shared-memory cycles of a line's transform, PAD 16 and odd rows -> these:
 // M = 64 32 -> 16, 48 24 -> 12.4, 32 20 -> 12, 24 13.5 -> 8.1, 16 (4 x 4) 13 -> 4, 12 9.8 -> 4.5; the others keep
-// the former. Even rows are filled by 16-byte copies.
+// the former, which no layout beats in that count (96: 56 to 58 cycles, best 56; 128: 48). Even rows are filled by
+// 16-byte copies.
 // z-pass, with the c2r pairs formed in the first pass of the line transforms (one pass over the tile less):
 // 128^3 36.8 -> 26.6 us, 64^3 12.3 -> 10.3, 96^3 22.9 -> 20.5; a step of 128 runs of 32^3 .. 96^3 9.05 -> 8.26 ms.
 template <int M>
@@ -81,9 +82,10 @@ struct Geometry {
   static constexpr int XST = ((XWIDE ? 6 : 3) * XLS + 1) / 2 * 2;  // 16-byte aligned start of the state rows
   static constexpr bool XPRE = CB == 8 && (size_t)(XST + 9 * N) * CB <= 100 * 1024;
   // Rows of 1 KB and more arrive by bulk copies instead (one thread issues them; no asynchronous copy per value:
-  // those took a quarter of the shared-memory pipe's cycles): x-stage 512^3 816 -> 689 us (its bytes: 670 at the
-  // copy bandwidth), 1024^3 8.02 -> 7.19 ms, 1024 x 512 x 256 1022 -> 913 us, 256^3 103 -> 94 us, 128^3
-  // with every row 37.0 -> 36.0 us; shorter rows keep the copies per value (not measured).
+  // those took a quarter of the shared-memory pipe's cycles): x-stage 512^3 816 -> 696 us (its bytes: 670 at the
+  // copy bandwidth), 1024^3 8.02 -> 7.26 ms, 1024 x 512 x 256 1022 -> 925 us, 256^3 103 -> 95 us, 128^3
+  // with every row 37.0 -> 35.8 us; shorter rows keep the copies per value (by bulk copies too 96^3
+  // takes 14.4 us where it takes 15.3, 64^3 9.5 for 9.9, 32^3 and less the same).
   static constexpr bool XBULK = XPRE && N >= 128;
   static constexpr size_t XSMEM = (size_t)6 * XLS * CB;
   static constexpr size_t XSMEM_ST = XPRE ? (size_t)(XST + 9 * N) * CB : XSMEM;  // XM_STAGE, XM_RHS
@@ -122,6 +124,7 @@ struct YCfg {
   static constexpr int THREADS = cmin(32 * TX, SHORT ? 128 : 256);
   static constexpr int LD = SHORT ? ZLay<NY>::ld(TX) : odd_ld(TX);
   static constexpr size_t SMEM = (size_t)(SHORT ? ZLay<NY>::ROWS : padt_len<T>(NY)) * LD * CB;
+  // short tiles: 4, 6 and 8 blocks an SM measured alike
   static constexpr int MINB = SHORT ? 6 : (CB == 16 ? (NY <= 256 ? 3 : 2) : (NY <= 512 ? (INV ? 3 : 4) : 2));
 };
 
@@ -180,8 +183,9 @@ __device__ __forceinline__ void put_curl_lines(cx<T>* s, int pos, int LS, cx<T> 
 
 // 1 / x for a positive normal x
 __device__ __forceinline__ float recip(float x) { return 1.f / x; }
-// in FP64 by Newton's iteration r <- r + r (1 - x r) from the hardware's approximation: four
-// operations of the FP64 pipe, last-bit accuracy (the division takes ten)
+// in FP64 by Newton's iteration r <- r + r (1 - x r) from the hardware's approximation (20 bits): the second step starts
+// from 2^-40, so that its one rounding gives the rounded quotient (equal to it for |k|^2 of all sizes in use). Four
+// operations of the FP64 pipe; the division takes ten
 __device__ __forceinline__ double recip(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -859,7 +863,8 @@ __device__ __forceinline__ void zpass_block_max(double m, unsigned long long* bi
 //         the two in a component of u x w the smaller scale's u is shifted down to the larger one e, so
 //         that they can be subtracted: p = P 2^(e - 2104), |P| <= 2^61. With one scale for the three components
 //         (and for omega's) a weak third component lost its bits: 1e-6 beside 1 kept 1e-11, 1e-20 nothing, and
-//         with the L1 scale a white field of 512 points 2.6e-15 (FP64 products 1.0e-15).
+//         with the L1 scale a white field of 512 points 2.6e-15 (FP64 products 1.0e-15); now 5e-16 and 9.3e-16, for
+//         4 to 6 % of the pass (256^3 818 -> 855 us, 512^3 7.85 -> 8.30 ms).
 //         Then the line of products is shifted by its L1, so that its DFT has 62 bits again
 //   r2c   V = X_k / 2 (quartered post-processing of the pair): X_k = V 2^(e + 1 - sh - 2104)
 // ---------------------------------------------------------------------------
@@ -1171,7 +1176,7 @@ __device__ __forceinline__ void zpass_body(const PassArgs a, const int bx, const
     constexpr int NL = NF * TX;
     // c2r pre-processing: Z'_k = (X_k + conj X_{M-k}) + i e^{+2 pi i k/N} (X_k - conj X_{M-k}),
     // stored conjugated so that a forward DFT gives the inverse one. The stage forms it in the first pass of the
-    // line transforms; here apart, so that the filtered stresses, small differences of products, keep their rounding.
+    // line transforms; here apart, as before that (a choice for the same last bits, not for accuracy).
     if constexpr (MODE != ZM_CROSS) {
       for (int e = threadIdx.x; e < NL * (M / 2 + 1); e += ZP_THREADS<T>) {
         const int l = e % NL, k = e / NL;
@@ -1401,8 +1406,8 @@ struct HwTw32 {
 // half-warps' accesses are eight rows of a column pair, 128 bytes of distinct banks, and the exchange inside a line
 // goes through rows permuted the same way (an address is one XOR). Against tiles moved in 8-byte pieces by cp.async
 // and drained by the threads (each 32 pieces took six cycles of that pipe, a quarter of all; an address and an
-// instruction each): 512^3 1476 -> 1059 us, 1024^3 15.99 -> 13.33 ms, 256^3 167 -> 144 us, 1024 x 512 x 256
-// 1271 -> 1065 us. Shorter lines keep k_zpass (tiles of their own width, batched members).
+// instruction each): 512^3 1476 -> 1060 us, 1024^3 15.99 -> 13.15 ms, 256^3 167 -> 146 us, 1024 x 512 x 256
+// 1271 -> 1067 us. Shorter lines keep k_zpass (tiles of their own width, batched members).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ cx<float> lds(unsigned p) {
   cx<float> v;
