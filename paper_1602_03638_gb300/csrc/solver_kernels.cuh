@@ -881,7 +881,7 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
   constexpr int GL = cmin(FxLinesPerWarp<M, V>::value, TX);  // lines per warp
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int sK[NL];        // scale of a line as the tile holds it
-  __shared__ int sL[NL];        // power of two that it was multiplied by (0 or FX_LIFT)
+  __shared__ int sL[NL];        // power of two that it was multiplied by (0 or FX_LIFT; any for a line of zeros)
   __shared__ unsigned sN[NL];   // its NaN word
   constexpr int NP = MODE == ZM_PRODUCTS ? 6 : 3;  // lines of products of a column
   __shared__ unsigned sQ[NP * TX];  // L1 of a line of products
@@ -956,7 +956,8 @@ __device__ __forceinline__ void zpass64_body(const PassArgs& a, const int bx, co
     if (q == 0 && l < NL) {
       const FxScale sc = fx_scale(m, sh);
       sK[l] = sc.K;
-      sL[l] = lift;
+      // a zero line's scale lies below all others: its product must not push the bits of the other one out
+      sL[l] = PROD && m == 0 ? 5000 : lift;
       sN[l] = sc.nan;
     }
   }

@@ -95,3 +95,22 @@ def test_filtered_products_of_a_weak_component(n, nc, weak):
         torch.cuda.synchronize()
     for c in range(6):
         assert (p[c] - ref[c]).abs().max() <= 8 * 2.0 ** -52 * ref[c].abs().max(), c
+
+
+@pytest.mark.parametrize("n", [8, 12, 16, 48, 64, 128])
+def test_a_product_with_a_zero_line_takes_no_bits(n):
+    """u = (0, e cos x, A sin x + e sin y): the third component of u x omega is u_x omega_y - u_y omega_x = 0 A - e^2
+    cos x cos y, which stays whatever A is (at kz = 0 the projection leaves that component alone)."""
+    A, e = 1e150, 1e-100
+    uh = torch.zeros((3, n, n, n // 2 + 1), dtype=torch.complex128, device="cuda")
+    uh[1, 1, 0, 0] = uh[1, -1, 0, 0] = 0.5 * n ** 3 * e
+    uh[2, 1, 0, 0], uh[2, -1, 0, 0] = -0.5j * n ** 3 * A, 0.5j * n ** 3 * A
+    uh[2, 0, 1, 0], uh[2, 0, -1, 0] = -0.5j * n ** 3 * e, 0.5j * n ** 3 * e
+    with Solver(n, 1e-300, 1e-3, "f64") as s:
+        s.set_state_spectral(uh)
+        out = torch.empty_like(uh)
+        s.rhs(out)
+        torch.cuda.synchronize()
+    want = -0.25 * n ** 3 * e * e
+    for x, y in ((1, 1), (1, -1), (-1, 1), (-1, -1)):
+        assert abs(out[2, x, y, 0].item() - want) <= TOL * abs(want), (x, y)
