@@ -5,7 +5,7 @@
 // lanes per SM and clock), so a butterfly in 64-bit integers takes a thirtieth of the time of the
 // same butterfly in FP64. Bound by integer issue now (256^3: both integer pipes about 55 % busy), no
 // longer by the FP64 pipe. RK4 step with the zero rows skipped, FP64 butterflies -> these:
-// 1024^3 2820 -> 872 ms, 512^3 302 -> 67.7 ms, 256^3 36.6 -> 7.7 ms, 128^3 4.84 -> 1.08 ms, 32^3 252 -> 94 us.
+// 1024^3 2820 -> 877 ms, 512^3 302 -> 68.6 ms, 256^3 36.6 -> 7.73 ms, 128^3 4.84 -> 1.08 ms, 32^3 252 -> 90 us.
 // A line transform of the FP64 form therefore runs on integers with one power
 // of two as the scale of the whole line:
 //
